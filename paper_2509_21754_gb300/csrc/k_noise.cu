@@ -188,9 +188,11 @@ template <bool VEC>
 __global__ void __launch_bounds__(kNoiseThreads) k_rs_hist(const float* __restrict__ vals,
                                                            int64_t stride, int nblk, int pass,
                                                            int mad, const unsigned* rsel,
-                                                           const double* cs, unsigned* hist) {
+                                                           const double* cs, unsigned* hist,
+                                                           int skip_done) {
   __shared__ unsigned sh[kBins];
   const int g = blockIdx.y;
+  if (skip_done && cs[2 * g + 1] >= 0.0) return;   // the split form has finished this map
   for (int b = threadIdx.x; b < kBins; b += blockDim.x) sh[b] = 0;
   __syncthreads();
   const unsigned prefix = rsel[4 * g + 0];
@@ -234,11 +236,13 @@ constexpr int kSelectThreads = 256;
 __global__ void __launch_bounds__(kSelectThreads) k_rs_select(int groups, int64_t n, int pass,
                                                               int mad, unsigned* hist,
                                                               unsigned* rsel, double* cs,
-                                                              unsigned long long* invalid) {
+                                                              unsigned long long* invalid,
+                                                              int skip_done) {
   __shared__ unsigned long long scan[kSelectThreads];
   __shared__ int found_bin;
   __shared__ unsigned found_below;
   const int g = blockIdx.x;
+  if (skip_done && cs[2 * g + 1] >= 0.0) return;
   const int tid = threadIdx.x;
   unsigned* h = hist + (size_t)g * kBins;
   unsigned* st = rsel + 4 * g;
@@ -1179,7 +1183,7 @@ constexpr int kSplitRuns = 512;
 constexpr int kSplitPool = kSplitRuns * 32;     // sample keys (64 KB of shared memory)
 constexpr int kSplitChunk = 4096;               // values per CTA of a pass
 constexpr int kSplitSlot = 1024;                // copies a chunk keeps (a quarter of its values)
-constexpr int kSplitMaxChunks = (int)(kFastMaxPerGroup / kSplitChunk);
+constexpr int kSplitMaxChunks = (int)(kFastMaxPerGroup / kSplitChunk);   // without the gather kernel
 constexpr int kSplitPassThreads = 128;
 constexpr int kSplitThreads = 1024;             // bracket and select kernels
 constexpr int kSplitBins = 2048;
@@ -1189,27 +1193,34 @@ static_assert(kSplitMaxChunks <= kSplitThreads, "one chunk count per select thre
 struct SplitState {
   uint32_t lo, hi;     // copy range of the current pass (inclusive keys)
   uint32_t nfin;       // finite values (set by the median's select)
-  uint32_t stage;      // 0: median pass, 1: MAD pass, 2: finished, 3: left to the cluster form
+  uint32_t stage;      // 0: median pass, 1: MAD pass, 2: finished, 3: left to the fallback
   float med;
   uint32_t nsample;    // finite sample values
-  uint32_t pad[2];
+  uint32_t ngather;    // keys the gather kernel has appended to the map's list
+  uint32_t pad;
 };
 static_assert(sizeof(SplitState) == 32, "SplitState layout");
 
 static int split_chunks(int64_t stride) { return (int)((stride + kSplitChunk - 1) / kSplitChunk); }
+static bool split_large(int64_t stride) { return stride > kFastMaxPerGroup; }
 
 static size_t split_head(int groups) {
   return ((size_t)groups * (sizeof(SplitState) + kSplitBins * sizeof(unsigned)) + 255) / 256 * 256;
 }
 
-size_t noise_split_bytes(int groups, int64_t stride) {
-  if (stride > kFastMaxPerGroup || groups > 65535) return 0;
+size_t noise_split_need(int groups, int64_t stride) {
+  if (stride > (int64_t)INT32_MAX - kSplitChunk || groups > 65535) return 0;
   const size_t nc = (size_t)groups * (size_t)split_chunks(stride);
-  return split_head(groups) + nc * sizeof(uint4) + nc * kSplitSlot * sizeof(uint32_t);
+  return split_head(groups) + nc * sizeof(uint4) + nc * kSplitSlot * sizeof(uint32_t) +
+         (split_large(stride) ? (size_t)groups * kSplitGather * sizeof(uint32_t) : 0);
+}
+
+size_t noise_split_bytes(int groups, int64_t stride) {
+  return split_large(stride) ? 0 : noise_split_need(groups, stride);
 }
 
 void noise_split_carve(void* base, int groups, int64_t stride, NoiseScratch* s) {
-  s->split = noise_split_bytes(groups, stride) ? base : nullptr;
+  s->split = noise_split_need(groups, stride) ? base : nullptr;
   s->split_cap = s->split ? (int64_t)split_chunks(stride) * kSplitSlot : 0;
 }
 
@@ -1218,6 +1229,7 @@ struct SplitPtrs {
   unsigned* hist;      // [groups][kSplitBins]
   uint4* cnt;          // [groups][nchunk]: keys below lo, finite values, copies (unclipped)
   uint32_t* copies;    // [groups][nchunk][kSplitSlot]
+  uint32_t* list;      // [groups][kSplitGather]: the rank's bin, gathered (large maps only)
   int nchunk;
 };
 
@@ -1231,6 +1243,7 @@ static SplitPtrs split_ptrs(void* base, int groups, int64_t stride) {
   r.cnt = reinterpret_cast<uint4*>(p);
   p += (size_t)groups * r.nchunk * sizeof(uint4);
   r.copies = reinterpret_cast<uint32_t*>(p);
+  r.list = split_large(stride) ? r.copies + (size_t)groups * r.nchunk * kSplitSlot : nullptr;
   return r;
 }
 
@@ -1291,11 +1304,19 @@ __device__ bool split_find(const unsigned* h, unsigned long long rank, unsigned*
   return ok;
 }
 
-// The sample: up to kSplitRuns runs of 32 consecutive values, evenly spread
-// over the map (the same runs in every call), as keys of v (mad = false) or
-// of |v - med| in FP32.  A value that is not finite leaves key 0, below every
-// finite key.  Returns the number of finite sample values; kminmax gets their
-// smallest and largest key.  Every thread must call it.
+// The sample (the same in every call), as keys of v (mad = false) or of
+// |v - med| in FP32: up to kSplitRuns runs of 32 consecutive values, evenly
+// spread over the map, or, above kSplitScatter values, kSplitPool single
+// values, one at a hashed place of each of as many equal stretches.  Runs are
+// one coalesced read each, but in sliding mode neighbouring values share most
+// of their window, so that a run says little more than one value, and an even
+// spread of runs can fall on the same columns of every row: on maps of 16.8 M
+// pixels the bracket then missed the rank in about one map of twenty, and that
+// map's fallback cost more than all the others' estimates.
+// A value that is not finite leaves key 0, below every finite key.  Returns
+// the number of finite sample values; kminmax gets their smallest and largest
+// key.  Every thread must call it.
+constexpr int64_t kSplitScatter = 1 << 20;
 __device__ unsigned split_sample(const float* v, int64_t stride, bool mad, float med,
                                  uint32_t* pool, unsigned* slots, uint32_t* kminmax,
                                  unsigned* nfin_sh) {
@@ -1303,49 +1324,68 @@ __device__ unsigned split_sample(const float* v, int64_t stride, bool mad, float
   constexpr int nwarps = kSplitThreads / 32;
   constexpr int per_warp = kSplitRuns / nwarps;   // runs a warp reads (16)
   static_assert(per_warp <= 32, "one run start per lane");
-  // the split form takes maps of at most 2 Mi values, so 32-bit arithmetic
-  // holds c * runs; lane l of warp w computes the start of run w + 32 l once
-  // (no division per run)
+  static_assert(kSplitPool % (8 * kSplitThreads) == 0 && kSplitScatter >= kSplitPool, "scattered sample");
+  const bool scatter = stride > kSplitScatter;
   const uint32_t runs = (uint32_t)((stride + 31) / 32);
   const uint32_t use = runs < (uint32_t)kSplitRuns ? runs : (uint32_t)kSplitRuns;
-  const uint32_t cl = (uint32_t)warp + (uint32_t)nwarps * (uint32_t)lane;
-  const uint32_t start = cl < use ? cl * runs / use * 32u : 0u;
   if (tid == 0) {
     kminmax[0] = 0xffffffffu;
     kminmax[1] = 0u;
     *nfin_sh = 0;
-    *slots = use * 32u;
+    *slots = use * 32u;   // kSplitPool when scattered
   }
-  for (int k = 0; k < per_warp; ++k) {   // every run into L2 first
-    const uint32_t c = (uint32_t)warp + (uint32_t)nwarps * (uint32_t)k;
-    const int64_t i = (int64_t)__shfl_sync(0xffffffffu, start, k) + lane;
-    if (c < use && i < stride) asm volatile("prefetch.global.L2 [%0];" ::"l"((const void*)(v + i)));
-  }
-  __syncthreads();
   uint32_t lmin = 0xffffffffu, lmax = 0u;
   unsigned nf = 0;
   constexpr int B = 8;
-  for (int k0 = 0; k0 < per_warp; k0 += B) {
-    const int64_t c0 = warp + (int64_t)nwarps * k0;
-    float x[B];
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-      const int64_t c = c0 + (int64_t)b * nwarps;
-      const int64_t i = (int64_t)__shfl_sync(0xffffffffu, start, k0 + b) + lane;
-      x[b] = (c < use && i < stride) ? v[i] : NAN;
+  auto take = [&](float x, uint32_t slot) {
+    uint32_t key = 0;
+    if (finite_bits(x)) {
+      key = mad ? f32_key(fabsf(x - med)) : f32_key(x);
+      lmin = min(lmin, key);
+      lmax = max(lmax, key);
+      ++nf;
     }
+    pool[slot] = key;
+  };
+  if (scatter) {
+    const uint32_t width = (uint32_t)(stride / kSplitPool);   // of a stretch, >= 64
+    for (uint32_t i0 = tid; i0 < (uint32_t)kSplitPool; i0 += B * kSplitThreads) {
+      float x[B];
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
-      const int64_t c = c0 + (int64_t)b * nwarps;
-      if (c >= use) break;
-      uint32_t key = 0;
-      if (finite_bits(x[b])) {
-        key = mad ? f32_key(fabsf(x[b] - med)) : f32_key(x[b]);
-        lmin = min(lmin, key);
-        lmax = max(lmax, key);
-        ++nf;
+      for (int b = 0; b < B; ++b) {
+        const uint32_t i = i0 + b * kSplitThreads;
+        x[b] = v[(size_t)i * width + __umulhi(i * 2654435761u, width)];
       }
-      pool[c * 32 + lane] = key;
+#pragma unroll
+      for (int b = 0; b < B; ++b) take(x[b], i0 + b * kSplitThreads);
+    }
+    __syncthreads();   // kminmax and nfin_sh are initialised
+  } else {
+    // lane l of warp w computes the start of run w + 32 l once (no division
+    // per run; 32-bit arithmetic holds c * runs)
+    const uint32_t cl = (uint32_t)warp + (uint32_t)nwarps * (uint32_t)lane;
+    const uint32_t start = cl < use ? cl * runs / use * 32u : 0u;
+    for (int k = 0; k < per_warp; ++k) {   // every run into L2 first
+      const uint32_t c = (uint32_t)warp + (uint32_t)nwarps * (uint32_t)k;
+      const int64_t i = (int64_t)__shfl_sync(0xffffffffu, start, k) + lane;
+      if (c < use && i < stride) asm volatile("prefetch.global.L2 [%0];" ::"l"((const void*)(v + i)));
+    }
+    __syncthreads();
+    for (int k0 = 0; k0 < per_warp; k0 += B) {
+      const int64_t c0 = warp + (int64_t)nwarps * k0;
+      float x[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        const int64_t c = c0 + (int64_t)b * nwarps;
+        const int64_t i = (int64_t)__shfl_sync(0xffffffffu, start, k0 + b) + lane;
+        x[b] = (c < use && i < stride) ? v[i] : NAN;
+      }
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        const int64_t c = c0 + (int64_t)b * nwarps;
+        if (c >= use) break;
+        take(x[b], (uint32_t)(c * 32 + lane));
+      }
     }
   }
 #pragma unroll
@@ -1441,7 +1481,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_bracket(const float* __
     s.stage = 0;
     s.med = 0.f;
     s.nsample = ns;
-    s.pad[0] = s.pad[1] = 0u;
+    s.ngather = s.pad = 0u;
     st[g] = s;
   }
 }
@@ -1458,8 +1498,8 @@ template <bool VEC, bool MAD>
 __global__ void __launch_bounds__(kSplitPassThreads, 12) k_split_pass(const float* __restrict__ vals,
                                                                      int64_t stride,
                                                                      const SplitState* __restrict__ st,
-                                                                     unsigned* hist_g, uint4* cnt,
-                                                                     uint32_t* copies, int nchunk) {
+                                                                     uint4* cnt, uint32_t* copies,
+                                                                     int nchunk) {
   pdl_begin();
   constexpr int NW = kSplitPassThreads / 32;
   constexpr int U = kSplitChunk / kSplitPassThreads;   // values per thread (32)
@@ -1505,7 +1545,6 @@ __global__ void __launch_bounds__(kSplitPassThreads, 12) k_split_pass(const floa
   asm volatile("cp.async.commit_group;" ::: "memory");
   const SplitState s = st[g];   // read while the copies land
   const uint32_t lo = s.lo, hi = s.hi;
-  const unsigned sh = split_shift(lo, hi);
   const float med = s.med;
   // order-preserving key from the bits (the same map as f32_key), kNoKey for
   // a value that is not finite; |v - med| is never negative, so its key is
@@ -1581,58 +1620,38 @@ __global__ void __launch_bounds__(kSplitPassThreads, 12) k_split_pass(const floa
   }
   if (tot > (unsigned)kSplitSlot) return;   // the select hands this map on
   uint32_t* out = copies + ((size_t)g * nchunk + c) * kSplitSlot;
-  unsigned* hg = hist_g + (size_t)g * kSplitBins;
   unsigned pos = wbase + (unsigned)(incl - nc);
-  for (uint32_t m = cmask; m; m &= m - 1) {
-    const uint32_t key = key_of(buf[off(__ffs(m) - 1)]);
-    out[pos++] = key;
-    atomicAdd(&hg[(key - lo) >> sh], 1u);
-  }
+  for (uint32_t m = cmask; m; m &= m - 1) out[pos++] = key_of(buf[off(__ffs(m) - 1)]);
 }
 
-// 3./5. Exact selection among the copies; after the median, the MAD's bracket.
+// The chunks' counts of one pass, summed, and the bin of the copies' histogram
+// over [s.lo, s.hi] (in `hist`, filled by the caller without a barrier after)
+// that holds the rank (lo..hi with `rank` inside it).  Every thread of the
+// CTA must call it; the answer is in every thread.
+enum { kLocEmpty = 0, kLocMiss = 1, kLocFound = 2 };
+struct SplitLoc {
+  uint32_t lo, hi;
+  unsigned long long rank;
+  unsigned nfin;
+};
 template <bool MAD>
-__global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __restrict__ vals,
-                                                                int64_t stride, int64_t n,
-                                                                SplitState* st, unsigned* hist_g,
-                                                                const uint4* __restrict__ cnt,
-                                                                const uint32_t* __restrict__ copies,
-                                                                int nchunk, double* cs,
-                                                                unsigned long long* invalid) {
-  pdl_begin();
-  extern __shared__ uint32_t spool[];   // kSplitPool (the sample, median stage), the gathered bin
-  __shared__ unsigned hist[kSplitBins];
-  __shared__ unsigned long long wsum[kSplitThreads / 32], found[2];
-  __shared__ uint32_t kmm[2];
-  __shared__ unsigned slots, nfin_sh, ngather;
-  __shared__ unsigned ccount[kSplitMaxChunks];   // copies of each chunk (unclipped)
-  __shared__ unsigned long long tsum[3];         // keys below lo, finite values, copies
-  __shared__ unsigned tover;                     // a chunk overflowed its slot
-  const int g = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const SplitState s = st[g];
-  if (s.stage != (MAD ? 1u : 0u)) return;
-  unsigned* hg = hist_g + (size_t)g * kSplitBins;
-  auto hand_on = [&]() {   // the cluster kernel computes this map
-    if (tid == 0) {
-      cs[2 * g + 1] = -1.0;
-      st[g].stage = 3;
-    }
-  };
-  // the chunks' counts (and the pass histogram, read beside them)
+__device__ int split_locate(const SplitState& s, const unsigned* hist, const uint4* cnt, int nchunk,
+                            unsigned long long* wsum, unsigned long long* found,
+                            unsigned long long* tsum, unsigned* tover, SplitLoc* loc) {
+  const int tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) {
     tsum[0] = tsum[1] = tsum[2] = 0ull;
-    tover = 0u;
-    ngather = 0u;
+    *tover = 0u;
   }
-  for (int b = tid; b < kSplitBins; b += kSplitThreads) hist[b] = hg[b];
-  uint4 q = make_uint4(0u, 0u, 0u, 0u);
-  if (tid < nchunk) {
-    q = cnt[(size_t)g * nchunk + tid];
-    ccount[tid] = q.z;
+  unsigned long long cb = 0, cf = 0, cc = 0;
+  unsigned over = 0;
+  for (int c = tid; c < nchunk; c += kSplitThreads) {
+    const uint4 q = cnt[c];
+    cb += q.x;
+    cf += q.y;
+    cc += q.z;
+    over |= q.z > (unsigned)kSplitSlot;
   }
-  unsigned long long cb = q.x, cf = q.y, cc = q.z;
-  unsigned over = q.z > (unsigned)kSplitSlot;
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
     cb += __shfl_xor_sync(0xffffffffu, cb, o);
@@ -1641,47 +1660,43 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __r
     over |= __shfl_xor_sync(0xffffffffu, over, o);
   }
   __syncthreads();   // tsum and tover are initialised
-  if (lane == 0 && warp * 32 < nchunk) {
+  if (lane == 0 && (tid & ~31) < nchunk) {
     atomicAdd(&tsum[0], cb);
     atomicAdd(&tsum[1], cf);
     atomicAdd(&tsum[2], cc);
-    if (over) atomicOr(&tover, 1u);
+    if (over) atomicOr(tover, 1u);
   }
   __syncthreads();
   const unsigned long long nbelow = tsum[0], ncopy = tsum[2];
   const unsigned nfin = MAD ? s.nfin : (unsigned)tsum[1];
-  if (!MAD && nfin == 0) {
-    if (tid == 0) {
-      cs[2 * g] = NAN;
-      cs[2 * g + 1] = 0.0;
-      if (invalid && n > 0) atomicAdd(invalid, (unsigned long long)n);
-      st[g].stage = 2;
-    }
-    return;
-  }
+  loc->nfin = nfin;
+  if (!MAD && nfin == 0) return kLocEmpty;
   const unsigned long long R = (nfin - 1) / 2;
-  if (s.nsample == 0 || tover || R < nbelow || R >= nbelow + ncopy) {
-    hand_on();
-    return;
-  }
-  // the bin of the pass histogram holding the rank, then its copies
-  unsigned long long rank = R - nbelow;
+  if (s.nsample == 0 || *tover || R < nbelow || R >= nbelow + ncopy) return kLocMiss;
   const unsigned sh = split_shift(s.lo, s.hi);
   unsigned bin;
   unsigned long long below;
-  if (!split_find(hist, rank, &bin, &below, wsum, found)) {
-    hand_on();
-    return;
-  }
-  rank -= below;
-  uint32_t lo = s.lo + (bin << sh);
-  const unsigned long long top = (unsigned long long)lo + (1ull << sh) - 1;
-  uint32_t hi = top < s.hi ? (uint32_t)top : s.hi;
-  // one warp per chunk slot, eight loads in flight per lane
+  if (!split_find(hist, R - nbelow, &bin, &below, wsum, found)) return kLocMiss;
+  loc->rank = R - nbelow - below;
+  loc->lo = s.lo + (bin << sh);
+  const unsigned long long top = (unsigned long long)loc->lo + (1ull << sh) - 1;
+  loc->hi = top < s.hi ? (uint32_t)top : s.hi;
+  return kLocFound;
+}
+
+// The copies of chunks c0, c0 + step, .. below nchunk (a warp per chunk slot,
+// eight loads in flight per lane) through put(); each lies in the pass's
+// [lo, hi].  A chunk with more copies than its slot holds wrote none (what the
+// slot holds is not this pass's), and its map is handed on by the select.
+template <typename Put>
+__device__ __forceinline__ void split_copies(const uint4* cnt, const uint32_t* copies, int nchunk,
+                                             int c0, int step, Put put) {
+  const int lane = threadIdx.x & 31;
   constexpr int GB = 8;
-  for (int c = warp; c < nchunk; c += kSplitThreads / 32) {
-    const unsigned nc = ccount[c];
-    const uint32_t* cp = copies + ((size_t)g * nchunk + c) * kSplitSlot;
+  for (int c = c0; c < nchunk; c += step) {
+    const unsigned nc = cnt[c].z;
+    if (nc > (unsigned)kSplitSlot) continue;
+    const uint32_t* cp = copies + (size_t)c * kSplitSlot;
     for (unsigned j0 = lane; j0 < nc; j0 += GB * 32) {
       uint32_t k[GB];
 #pragma unroll
@@ -1690,14 +1705,146 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __r
         k[b] = j < nc ? cp[j] : 1u;
       }
 #pragma unroll
-      for (int b = 0; b < GB; ++b) {
-        const unsigned j = j0 + b * 32;
-        if (j < nc && k[b] >= lo && k[b] <= hi) {
-          const unsigned i = atomicAdd(&ngather, 1u);
-          if (i < kSplitGather) spool[i] = k[b];
-        }
-      }
+      for (int b = 0; b < GB; ++b)
+        if (j0 + b * 32 < nc) put(k[b]);
     }
+  }
+}
+
+// Large maps (above kFastMaxPerGroup values): one CTA would walk thousands of
+// slots at one warp's latency each, so gridDim.x CTAs share a map's chunks,
+// first for the histogram of its copies (k_split_hist: shared memory, then one
+// global add per occupied bin), then to gather the rank's bin into the map's
+// list (k_split_gather, each CTA locating the bin for itself).  Counting the
+// copies in the pass itself, one global add each, was bound by those adds:
+// all of a map's CTAs hit its 2048 counters at once (30 maps of 16.8 M values:
+// 1.66 and 1.29 ms a pass, 0.40 and 0.33 without, and 25 us for this kernel).
+template <bool MAD>
+__global__ void __launch_bounds__(kSplitThreads) k_split_hist(const SplitState* __restrict__ st,
+                                                              unsigned* hist_g,
+                                                              const uint4* __restrict__ cnt,
+                                                              const uint32_t* __restrict__ copies,
+                                                              int nchunk) {
+  pdl_begin();
+  __shared__ unsigned hist[kSplitBins];
+  const int g = blockIdx.y, tid = threadIdx.x;
+  const SplitState s = st[g];
+  if (s.stage != (MAD ? 1u : 0u)) return;
+  for (int b = tid; b < kSplitBins; b += kSplitThreads) hist[b] = 0;
+  __syncthreads();
+  const unsigned sh = split_shift(s.lo, s.hi);
+  const uint32_t lo = s.lo;
+  split_copies(cnt + (size_t)g * nchunk, copies + (size_t)g * nchunk * kSplitSlot, nchunk,
+               (int)blockIdx.x * (kSplitThreads / 32) + (tid >> 5),
+               (int)gridDim.x * (kSplitThreads / 32),
+               [&](uint32_t k) { atomicAdd(&hist[(k - lo) >> sh], 1u); });
+  __syncthreads();
+  unsigned* hg = hist_g + (size_t)g * kSplitBins;
+  for (int b = tid; b < kSplitBins; b += kSplitThreads)
+    if (hist[b]) atomicAdd(&hg[b], hist[b]);
+}
+
+template <bool MAD>
+__global__ void __launch_bounds__(kSplitThreads) k_split_gather(SplitState* st,
+                                                                const unsigned* __restrict__ hist_g,
+                                                                const uint4* __restrict__ cnt,
+                                                                const uint32_t* __restrict__ copies,
+                                                                int nchunk, uint32_t* list) {
+  pdl_begin();
+  __shared__ unsigned hist[kSplitBins];
+  __shared__ unsigned long long wsum[kSplitThreads / 32], found[2], tsum[3];
+  __shared__ unsigned tover;
+  const int g = blockIdx.y;
+  const SplitState s = st[g];
+  if (s.stage != (MAD ? 1u : 0u)) return;
+  for (int b = threadIdx.x; b < kSplitBins; b += kSplitThreads)
+    hist[b] = hist_g[(size_t)g * kSplitBins + b];
+  SplitLoc loc;
+  if (split_locate<MAD>(s, hist, cnt + (size_t)g * nchunk, nchunk, wsum, found, tsum, &tover,
+                        &loc) != kLocFound)
+    return;   // the select comes to the same answer
+  uint32_t* out = list + (size_t)g * kSplitGather;
+  split_copies(cnt + (size_t)g * nchunk, copies + (size_t)g * nchunk * kSplitSlot, nchunk,
+               (int)blockIdx.x * (kSplitThreads / 32) + (int)(threadIdx.x >> 5),
+               (int)gridDim.x * (kSplitThreads / 32), [&](uint32_t k) {
+                 if (k < loc.lo || k > loc.hi) return;
+                 const unsigned i = atomicAdd(&st[g].ngather, 1u);
+                 if (i < (unsigned)kSplitGather) out[i] = k;
+               });
+}
+
+// 3./5. Exact selection among the copies; after the median, the MAD's bracket.
+// With `list` the rank's bin has been gathered by k_split_gather.
+template <bool MAD>
+__global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __restrict__ vals,
+                                                                int64_t stride, int64_t n,
+                                                                SplitState* st, unsigned* hist_g,
+                                                                const uint4* __restrict__ cnt,
+                                                                const uint32_t* __restrict__ copies,
+                                                                int nchunk,
+                                                                const uint32_t* __restrict__ list,
+                                                                double* cs,
+                                                                unsigned long long* invalid) {
+  pdl_begin();
+  extern __shared__ uint32_t spool[];   // kSplitPool (the sample, median stage), the gathered bin
+  __shared__ unsigned hist[kSplitBins];
+  __shared__ unsigned long long wsum[kSplitThreads / 32], found[2];
+  __shared__ uint32_t kmm[2];
+  __shared__ unsigned slots, nfin_sh, ngather;
+  __shared__ unsigned long long tsum[3];         // keys below lo, finite values, copies
+  __shared__ unsigned tover;                     // a chunk overflowed its slot
+  const int g = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const SplitState s = st[g];
+  if (s.stage != (MAD ? 1u : 0u)) return;
+  unsigned* hg = hist_g + (size_t)g * kSplitBins;
+  auto hand_on = [&]() {   // the fallback computes this map
+    if (tid == 0) {
+      cs[2 * g + 1] = -1.0;
+      st[g].stage = 3;
+    }
+  };
+  if (tid == 0) ngather = list ? s.ngather : 0u;
+  const uint4* cnt_m = cnt + (size_t)g * nchunk;
+  const uint32_t* copies_m = copies + (size_t)g * nchunk * kSplitSlot;
+  if (list) {
+    for (int b = tid; b < kSplitBins; b += kSplitThreads) hist[b] = hg[b];
+  } else {
+    for (int b = tid; b < kSplitBins; b += kSplitThreads) hist[b] = 0;
+    __syncthreads();
+    const unsigned sh = split_shift(s.lo, s.hi);
+    split_copies(cnt_m, copies_m, nchunk, warp, kSplitThreads / 32,
+                 [&](uint32_t k) { atomicAdd(&hist[(k - s.lo) >> sh], 1u); });
+  }
+  SplitLoc loc;
+  const int where = split_locate<MAD>(s, hist, cnt_m, nchunk, wsum, found, tsum, &tover, &loc);
+  const unsigned nfin = loc.nfin;
+  if (where == kLocEmpty) {
+    if (tid == 0) {
+      cs[2 * g] = NAN;
+      cs[2 * g + 1] = 0.0;
+      if (invalid && n > 0) atomicAdd(invalid, (unsigned long long)n);
+      st[g].stage = 2;
+    }
+    return;
+  }
+  if (where == kLocMiss) {
+    hand_on();
+    return;
+  }
+  unsigned long long rank = loc.rank;
+  uint32_t lo = loc.lo, hi = loc.hi;
+  unsigned bin;
+  unsigned long long below;
+  if (list) {
+    const unsigned m = s.ngather < (unsigned)kSplitGather ? s.ngather : (unsigned)kSplitGather;
+    for (unsigned i = tid; i < m; i += kSplitThreads) spool[i] = list[(size_t)g * kSplitGather + i];
+  } else {
+    split_copies(cnt_m, copies_m, nchunk, warp, kSplitThreads / 32, [&](uint32_t k) {
+      if (k < lo || k > hi) return;
+      const unsigned i = atomicAdd(&ngather, 1u);
+      if (i < (unsigned)kSplitGather) spool[i] = k;
+    });
   }
   __syncthreads();
   const unsigned ng = ngather;
@@ -1749,7 +1896,8 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __r
     hand_on();
     return;
   }
-  for (int b = tid; b < kSplitBins; b += kSplitThreads) hg[b] = 0;
+  if (list)
+    for (int b = tid; b < kSplitBins; b += kSplitThreads) hg[b] = 0;
   if (tid == 0) {
     SplitState n2 = s;
     n2.lo = mlo + 1;       // keys <= m_lo are counted below
@@ -1757,6 +1905,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __r
     n2.nfin = nfin;
     n2.stage = 1;
     n2.med = val;
+    n2.ngather = 0;
     st[g] = n2;
   }
 }
@@ -1781,22 +1930,38 @@ static cudaError_t launch_split_t(const float* vals, int groups, int64_t stride,
     configured = true;
   }
   const dim3 pgrid((unsigned)sp.nchunk, (unsigned)groups);
+  // CTAs that share a large map's copies: two waves of the chip over all maps,
+  // at least one chunk per warp
+  const int ng = std::max(1, std::min(sp.nchunk / (kSplitThreads / 32), 152 * 4 / groups));
+  const dim3 ggrid((unsigned)ng, (unsigned)groups);
   cudaError_t e = launch_pdl(k_split_bracket, dim3(groups), dim3(kSplitThreads), dyn, st, vals,
                              stride, sp.st, sp.hist);
   if (e == cudaSuccess)
     e = launch_pdl(k_split_pass<VEC, false>, pgrid, dim3(kSplitPassThreads), 0, st, vals, stride,
-                   sp.st, sp.hist, sp.cnt, sp.copies, sp.nchunk);
+                   sp.st, sp.cnt, sp.copies, sp.nchunk);
+  if (e == cudaSuccess && sp.list)
+    e = launch_pdl(k_split_hist<false>, ggrid, dim3(kSplitThreads), 0, st, sp.st, sp.hist, sp.cnt,
+                   sp.copies, sp.nchunk);
+  if (e == cudaSuccess && sp.list)
+    e = launch_pdl(k_split_gather<false>, ggrid, dim3(kSplitThreads), 0, st, sp.st, sp.hist, sp.cnt,
+                   sp.copies, sp.nchunk, sp.list);
   if (e == cudaSuccess)
     e = launch_pdl(k_split_select<false>, dim3(groups), dim3(kSplitThreads), dyn, st, vals, stride,
-                   n, sp.st, sp.hist, sp.cnt, sp.copies, sp.nchunk, cs, ns.invalid);
+                   n, sp.st, sp.hist, sp.cnt, sp.copies, sp.nchunk, sp.list, cs, ns.invalid);
   if (e == cudaSuccess)
     e = launch_pdl(k_split_pass<VEC, true>, pgrid, dim3(kSplitPassThreads), 0, st, vals, stride,
-                   sp.st, sp.hist, sp.cnt, sp.copies, sp.nchunk);
+                   sp.st, sp.cnt, sp.copies, sp.nchunk);
+  if (e == cudaSuccess && sp.list)
+    e = launch_pdl(k_split_hist<true>, ggrid, dim3(kSplitThreads), 0, st, sp.st, sp.hist, sp.cnt,
+                   sp.copies, sp.nchunk);
+  if (e == cudaSuccess && sp.list)
+    e = launch_pdl(k_split_gather<true>, ggrid, dim3(kSplitThreads), 0, st, sp.st, sp.hist, sp.cnt,
+                   sp.copies, sp.nchunk, sp.list);
   if (e == cudaSuccess)
     e = launch_pdl(k_split_select<true>, dim3(groups), dim3(kSplitThreads), dyn, st, vals, stride,
-                   n, sp.st, sp.hist, sp.cnt, sp.copies, sp.nchunk, cs, ns.invalid);
+                   n, sp.st, sp.hist, sp.cnt, sp.copies, sp.nchunk, sp.list, cs, ns.invalid);
   if (e != cudaSuccess) return e;
-  count_launches(5);
+  count_launches(sp.list ? 9 : 5);
   return cudaGetLastError();
 }
 
@@ -1826,14 +1991,22 @@ cudaError_t launch_noise(const float* vals, int groups, int64_t stride, int64_t 
     return cudaGetLastError();
   }
   if (mode != FITRIG_NOISE_MEDMAD) return cudaErrorInvalidValue;
-  // groups of up to 2 Mi values with split scratch: the split form, then the
-  // cluster form for any group it leaves
-  if (s.split && s.allow_cluster && stride <= kFastMaxPerGroup && groups <= 65535 &&
-      stride <= (int64_t)INT32_MAX) {
+  // The split form reads a map twice whatever its size, the grid-wide passes
+  // six times with shared atomics per value: 30 maps of 16.8 M values take
+  // 0.93 ms against 6.05 ms, 6 maps of 24.2 M with eta's 0.54 against 2.27 ms
+  // (serialised launches).
+  // with split scratch: the split form, then, for any group it leaves, the form
+  // that takes maps of that size without scratch: the cluster form, or above
+  // kClusterMaxPerGroup the grid-wide passes, whose launches return at once
+  // for the groups that are done
+  int skip_done = 0;
+  if (s.split && s.allow_cluster && groups <= 65535) {
     const cudaError_t e = vec ? launch_split_t<true>(vals, groups, stride, n, s, cs, st)
                               : launch_split_t<false>(vals, groups, stride, n, s, cs, st);
     if (e != cudaSuccess) return e;
-    return launch_medmad_cluster(vals, groups, stride, n, vec, cs, s.invalid, 1, st);
+    if (stride <= kClusterMaxPerGroup)
+      return launch_medmad_cluster(vals, groups, stride, n, vec, cs, s.invalid, 1, st);
+    skip_done = 1;
   }
   // groups of moderate size: one cluster per group, all passes in one launch
   if (stride <= kClusterMaxPerGroup && s.allow_cluster) {
@@ -1853,12 +2026,12 @@ cudaError_t launch_noise(const float* vals, int groups, int64_t stride, int64_t 
     for (int pass = 0; pass < 3; ++pass) {
       if (vec)
         k_rs_hist<true><<<grid, kNoiseThreads, 0, st>>>(vals, stride, nblk, pass, mad, s.rsel,
-                                                        cs, s.hist);
+                                                        cs, s.hist, skip_done);
       else
         k_rs_hist<false><<<grid, kNoiseThreads, 0, st>>>(vals, stride, nblk, pass, mad, s.rsel,
-                                                         cs, s.hist);
+                                                         cs, s.hist, skip_done);
       k_rs_select<<<groups, kSelectThreads, 0, st>>>(groups, n, pass, mad, s.hist, s.rsel, cs,
-                                                     s.invalid);
+                                                     s.invalid, skip_done);
     }
   }
   count_launches(12);

@@ -1011,6 +1011,27 @@ static cudaError_t enqueue_post(fitrig_plan_t p, cudaStream_t st, bool timed) {
   // 1024 tiles the image candidates come straight from the peak bitmap,
   // already in (snapshot, y, x) order
   const bool rows_emit = image && p->d_arg && ca.w <= 8 && p->Tx <= 1024;
+  // Maps too large for the plan's own split scratch borrow the candidates'
+  // second buffer, which nothing uses before the image candidates are formed
+  // (after the branches join): the automatic capacity of 4 Mi + tiles / 12
+  // entries of 32 bytes always holds the copies of both branches (about one
+  // byte per value each); an explicit MAX_SELECTED may not, and such a plan
+  // keeps the multi-pass forms.
+  NoiseScratch ns_img = p->ns_img, ns_freq = p->ns_freq;
+  if (p->noise == FITRIG_NOISE_MEDMAD) {
+    char* lent = reinterpret_cast<char*>(p->d_cand_tmp);
+    size_t left = sizeof(fitrig_candidate) * (size_t)p->cand_cap;
+    auto lend = [&](int groups, NoiseScratch* ns) {
+      const size_t need = ns->split ? 0 : noise_split_need(groups, p->vstride);
+      if (need == 0 || need > left) return;
+      noise_split_carve(lent, groups, p->vstride, ns);
+      const size_t step = std::min(left, (need + 255) / 256 * 256);
+      lent += step;
+      left -= step;
+    };
+    if (image) lend(U, &ns_img);
+    if (freq) lend(1, &ns_freq);
+  }
   cudaStream_t is = st;
   if (image && freq) {
     CKE(cudaEventRecord(p->fork_ev, st));
@@ -1019,7 +1040,7 @@ static cudaError_t enqueue_post(fitrig_plan_t p, cudaStream_t st, bool timed) {
   }
   if (image) {
     if (timed) rec(p, FITRIG_KERNEL_NOISE, 0, is);
-    CKE(launch_noise(p->d_vp, U, p->vstride, p->T, p->noise, p->ns_img, p->d_cs, is));
+    CKE(launch_noise(p->d_vp, U, p->vstride, p->T, p->noise, ns_img, p->d_cs, is));
     CKE(launch_thresholds(p->d_cs, U, p->tau, p->d_thr, p->d_inv, is));
     if (timed) rec(p, FITRIG_KERNEL_NOISE, 1, is);
     if (timed) rec(p, FITRIG_KERNEL_SELECT, 0, is);
@@ -1047,7 +1068,7 @@ static cudaError_t enqueue_post(fitrig_plan_t p, cudaStream_t st, bool timed) {
                           p->d_bin, st));
     mark(FITRIG_KERNEL_SPECTRUM, 1);
     double* cs = p->d_cs + 2 * U;
-    CKE(launch_noise(p->d_eta, 1, p->vstride, p->T, p->noise, p->ns_freq, cs, st));
+    CKE(launch_noise(p->d_eta, 1, p->vstride, p->T, p->noise, ns_freq, cs, st));
     CKE(launch_thresholds(cs, 1, p->tau, p->d_thr + U, p->d_inv + U, st));
     CKE(launch_block_select(p->d_eta, 1, p->vstride, p->Tx, p->Ty, p->d_thr + U, p->blk_f,
                             p->d_fpeaks, p->T, status, p->sel.want, st));
