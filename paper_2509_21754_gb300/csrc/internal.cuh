@@ -194,7 +194,12 @@ struct StackArgs {
   StackGeom g;
   const float* key = nullptr;   // difference-coded stack: FP32 snapshot 0 ([ny][kpitch]),
   int64_t kpitch = 0;           // the stack slots 1.. then hold half differences
+  int seg_units = 0;            // units per time segment (blockIdx.z), set by the launcher
 };
+
+// Units per time segment of a march over `boxes` CTAs' boxes and `units` units
+// with `per_sm` CTAs resident per SM (see k_stack.cu).
+int march_seg_units(int64_t boxes, int per_sm, int units);
 
 // One field of a batched (persistent, multi-field) stack march.  The TMA
 // descriptor must stay 64-byte aligned in device memory.
@@ -256,6 +261,7 @@ struct SlideArgs {
   unsigned* status;
   uint64_t timeout_ns;
   SlideGeom g;
+  int seg_units = 0;   // as StackArgs::seg_units
 };
 bool slide_geometry(int w, int elem_bytes, SlideGeom* g);
 cudaError_t launch_slide(const CUtensorMap* tmap, const SlideArgs& a, int storage, int rmode,

@@ -52,7 +52,11 @@ __global__ void __launch_bounds__(kSlideMaxThreads) k_slide(const __grid_constan
   const uint32_t bar0 = smem_u32(bars);
   const uint32_t stage0 = smem_u32(smem);
   const uint32_t box_bytes = (uint32_t)(g.boxW * g.EH * (int)sizeof(T));
-  const int L = a.nsnap;
+  const int s0 = blockIdx.z * a.seg_units;                // first unit of the segment
+  const int L = min(a.seg_units, a.nsnap - 2 - s0) + 2;   // its snapshots
+  const int z0 = a.zrot + s0;
+  float* const vp = a.vp + (size_t)s0 * (size_t)a.vstride;
+  unsigned* const smax = a.smax ? a.smax + s0 : nullptr;
   const bool active = tid < g.EW * g.nseg;
 
   if (tid == 0) {
@@ -64,7 +68,7 @@ __global__ void __launch_bounds__(kSlideMaxThreads) k_slide(const __grid_constan
   if (tid == 0) {
     for (int j = 0; j < NS && j < L; ++j) {
       mbar_expect_tx(bar0 + 8 * j, box_bytes);
-      tma_load_3d(stage0 + j * (uint32_t)g.stage_bytes, &tmap, xload, y0 - g.h, (a.zrot + j) % L,
+      tma_load_3d(stage0 + j * (uint32_t)g.stage_bytes, &tmap, xload, y0 - g.h, (z0 + j) % a.nsnap,
                   bar0 + 8 * j);
     }
   }
@@ -108,12 +112,12 @@ __global__ void __launch_bounds__(kSlideMaxThreads) k_slide(const __grid_constan
       return;
     }
     mx = fmaxf(mx, sm);
-    if (a.smax) warp_max_to(sm, a.smax + j);
+    if (smax) warp_max_to(sm, smax + j);
     if (tid == 0 && j + NS < L) {
       fence_proxy_async_smem();
       mbar_expect_tx(bar0 + 8 * stg, box_bytes);
       tma_load_3d(stage0 + stg * (uint32_t)g.stage_bytes, &tmap, xload, y0 - g.h,
-                  (a.zrot + j + NS) % L, bar0 + 8 * stg);
+                  (z0 + j + NS) % a.nsnap, bar0 + 8 * stg);
     }
     if (j < 2) continue;
     // horizontal pass: window rows over the extended block
@@ -149,7 +153,7 @@ __global__ void __launch_bounds__(kSlideMaxThreads) k_slide(const __grid_constan
       const float n = (float)(ny_ * nx_);
       float v = (S1 / n) * S2 * (S3 / n);
       if (!isfinite(S1) || !isfinite(v)) v = NAN;
-      a.vp[(size_t)(j - 2) * (size_t)a.vstride + (size_t)y * a.nx + x] = v;
+      vp[(size_t)(j - 2) * (size_t)a.vstride + (size_t)y * a.nx + x] = v;
     }
   }
 #pragma unroll
@@ -230,7 +234,11 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_shf(const __grid_co
   const int xe = x0 - H;                        // first extended column
   const int xload = xe >= 0 ? (xe & ~7) : -(((-xe) + 7) & ~7);
   const int col = (xe - xload) + warp * OWW + lane;
-  const int L = a.nsnap;
+  const int s0 = blockIdx.z * a.seg_units;                // first unit of the segment
+  const int L = min(a.seg_units, a.nsnap - 2 - s0) + 2;   // its snapshots
+  const int z0 = a.zrot + s0;
+  float* const vp = a.vp + (size_t)s0 * (size_t)a.vstride;
+  unsigned* const smax = a.smax ? a.smax + s0 : nullptr;
   if (tid == 0) {
     prefetch_tmap(&tmap);
     for (int i = 0; i < NS; ++i) mbar_init(bar0 + 8 * i, 1);
@@ -240,7 +248,7 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_shf(const __grid_co
   if (tid == 0) {
     for (int j = 0; j < NS && j < L; ++j) {
       mbar_expect_tx(bar0 + 8 * j, box_bytes);
-      tma_load_3d(stage0 + j * (uint32_t)g.stage_bytes, &tmap, xload, y0 - H, (a.zrot + j) % L,
+      tma_load_3d(stage0 + j * (uint32_t)g.stage_bytes, &tmap, xload, y0 - H, (z0 + j) % a.nsnap,
                   bar0 + 8 * j);
     }
   }
@@ -293,7 +301,7 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_shf(const __grid_co
               const float inv = (nyw == W && nxw == W) ? kInvFull : 1.f / (np * np);
               float v = S1 * S2 * S3 * inv;
               if (!isfinite(S1) || !isfinite(v)) v = NAN;
-              a.vp[(size_t)(j - 2) * (size_t)a.vstride + (size_t)y * a.nx + ox] = v;
+              vp[(size_t)(j - 2) * (size_t)a.vstride + (size_t)y * a.nx + ox] = v;
             }
           }
         }
@@ -312,12 +320,12 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_shf(const __grid_co
       return;
     }
     mx = fmaxf(mx, sm);
-    if (a.smax) warp_max_to(sm, a.smax + j);
+    if (smax) warp_max_to(sm, smax + j);
     if (tid == 0 && j + NS < L) {
       fence_proxy_async_smem();
       mbar_expect_tx(bar0 + 8 * stg, box_bytes);
       tma_load_3d(stage0 + stg * (uint32_t)g.stage_bytes, &tmap, xload, y0 - H,
-                  (a.zrot + j + NS) % L, bar0 + 8 * stg);
+                  (z0 + j + NS) % a.nsnap, bar0 + 8 * stg);
     }
   }
 #pragma unroll
@@ -384,6 +392,20 @@ bool slide_geometry(int w, int elem_bytes, SlideGeom* g) {
   return true;
 }
 
+template <typename K>
+static cudaError_t launch_segments(K kern, const CUtensorMap* tmap, SlideArgs a, cudaStream_t st) {
+  int per_sm = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, a.g.threads,
+                                                                      a.g.smem_bytes);
+  if (e != cudaSuccess) return e;
+  const int units = a.nsnap - 2;
+  a.seg_units = march_seg_units((int64_t)a.g.gridX * a.g.gridY, per_sm, units);
+  const dim3 grid(a.g.gridX, a.g.gridY, (units + a.seg_units - 1) / a.seg_units);
+  kern<<<grid, a.g.threads, a.g.smem_bytes, st>>>(*tmap, a);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
 template <typename T, int W, bool SIGNED>
 static cudaError_t launch_shf_t(const CUtensorMap* tmap, const SlideArgs& a, cudaStream_t st) {
   auto kern = k_slide_shf<T, W, SIGNED>;
@@ -394,10 +416,7 @@ static cudaError_t launch_shf_t(const CUtensorMap* tmap, const SlideArgs& a, cud
     if (e != cudaSuccess) return e;
     configured = a.g.smem_bytes;
   }
-  dim3 grid(a.g.gridX, a.g.gridY);
-  kern<<<grid, a.g.threads, a.g.smem_bytes, st>>>(*tmap, a);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_segments(kern, tmap, a, st);
 }
 
 template <typename T, bool SIGNED>
@@ -419,10 +438,7 @@ static cudaError_t launch_slide_t(const CUtensorMap* tmap, const SlideArgs& a, c
     if (e != cudaSuccess) return e;
     configured = a.g.smem_bytes;
   }
-  dim3 grid(a.g.gridX, a.g.gridY);
-  kern<<<grid, a.g.threads, a.g.smem_bytes, st>>>(*tmap, a);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_segments(kern, tmap, a, st);
 }
 
 cudaError_t launch_slide(const CUtensorMap* tmap, const SlideArgs& a, int storage, int rmode,

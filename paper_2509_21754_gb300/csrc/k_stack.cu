@@ -32,31 +32,13 @@
 #include <cfloat>
 #include <cmath>
 
-#include "internal.cuh"
+#include "march.cuh"
 
 namespace fitrig {
 
 constexpr int kStackMaxThreads = 512;
 constexpr int kSmallMaxThreads = 256;   // thread-per-tile path: 32 x TBY tiles per CTA
 constexpr int kSmallMaxW = 6;
-
-// Approximate reciprocal (rcp.approx.ftz: relative error below 2^-23).
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Maximum of v over the calling threads into *key.  Full warps reduce with
-// shuffles first; the threads of a trailing partial warp (a block size that is
-// not a multiple of 32) go straight to the atomic.
-__device__ __forceinline__ void max_to(float v, unsigned* key, bool full_warp) {
-  if (full_warp) {
-    warp_max_to(v, key);
-    return;
-  }
-  if (v > -INFINITY) atomicMax(key, f32_key(v));
-}
 
 template <typename T, int R, bool SIGNED>
 __global__ void __launch_bounds__(kStackMaxThreads) k_stack_tile(const __grid_constant__ CUtensorMap tmap,
@@ -81,7 +63,11 @@ __global__ void __launch_bounds__(kStackMaxThreads) k_stack_tile(const __grid_co
   const uint32_t bar0 = smem_u32(bars);
   const uint32_t stage0 = smem_u32(smem);
   const uint32_t box_bytes = (uint32_t)(g.boxW * g.BH * (int)sizeof(T));
-  const int L = a.nsnap;
+  const int s0 = blockIdx.z * a.seg_units;                    // first unit of the segment
+  const int L = min(a.seg_units, a.nsnap - 2 - s0) + 2;       // its snapshots
+  const int z0 = a.zrot + s0;
+  float* const vp = a.vp + (size_t)s0 * (size_t)a.vstride;
+  unsigned* const smax = a.smax ? a.smax + s0 : nullptr;
 
   if (tid == 0) {
     prefetch_tmap(&tmap);
@@ -92,7 +78,7 @@ __global__ void __launch_bounds__(kStackMaxThreads) k_stack_tile(const __grid_co
   if (tid == 0) {
     for (int j = 0; j < NS && j < L; ++j) {
       mbar_expect_tx(bar0 + 8 * j, box_bytes);
-      tma_load_3d(stage0 + j * (uint32_t)g.stage_bytes, &tmap, xload, y0, (a.zrot + j) % L, bar0 + 8 * j);
+      tma_load_3d(stage0 + j * (uint32_t)g.stage_bytes, &tmap, xload, y0, (z0 + j) % a.nsnap, bar0 + 8 * j);
     }
   }
 
@@ -169,11 +155,11 @@ __global__ void __launch_bounds__(kStackMaxThreads) k_stack_tile(const __grid_co
     }
     mx = fmaxf(mx, sm);
     const bool full_warp = (tid >> 5) < (g.threads >> 5);
-    if (a.smax) max_to(sm, a.smax + j, full_warp);
+    if (smax) max_to(sm, smax + j, full_warp);
     if (tid == 0 && j + NS < L) {
       fence_proxy_async_smem();
       mbar_expect_tx(bar0 + 8 * stg, box_bytes);
-      tma_load_3d(stage0 + stg * (uint32_t)g.stage_bytes, &tmap, xload, y0, (a.zrot + j + NS) % L,
+      tma_load_3d(stage0 + stg * (uint32_t)g.stage_bytes, &tmap, xload, y0, (z0 + j + NS) % a.nsnap,
                   bar0 + 8 * stg);
     }
     if (++stg == NS) {
@@ -181,38 +167,56 @@ __global__ void __launch_bounds__(kStackMaxThreads) k_stack_tile(const __grid_co
       phase ^= 1u;
     }
     if (j >= 2) {
-      // One full warp per tile combines the tile's nseg * w column partials:
-      // lanes stride over them, then a fixed shuffle tree (deterministic).
-      // Warps take tiles round-robin; a trailing partial warp takes none.
-      const int warp = tid >> 5, lane = tid & 31, nwf = g.threads >> 5;
       const int NT = g.TBX * g.TBY, per = g.nseg * g.w;
       const float4* pp = part + (j & 1) * g.threads;
-      for (int tt = warp; tt < NT && warp < nwf; tt += nwf) {
-        const int tb = tt / g.TBX;
-        const int tbx = tt - tb * g.TBX;
-        float S1 = 0.f, S2 = 0.f, S3 = 0.f;
-        for (int i = lane; i < per; i += 32) {
-          const int sg = i / g.w, cc = i - sg * g.w;
-          const float4 q = pp[(tb * g.nseg + sg) * g.BW + tbx * g.w + cc];
-          S1 += q.x;
-          S2 = fmaxf(S2, q.y);
-          S3 += q.z;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          S1 += __shfl_xor_sync(0xffffffffu, S1, o);
-          S2 = fmaxf(S2, __shfl_xor_sync(0xffffffffu, S2, o));
-          S3 += __shfl_xor_sync(0xffffffffu, S3, o);
-        }
+      auto finish = [&](int tb, int tbx, float S1, float S2, float S3) {
         const int tx = blockIdx.x * g.TBX + tbx;
         const int ty = blockIdx.y * g.TBY + tb;
-        if (lane == 0 && tx < a.Tx && ty < a.Ty) {
-          const int hw = min(g.w, a.ny - ty * g.w);
-          const int ww = min(g.w, a.nx - tx * g.w);
-          const float n = (float)(hw * ww);
-          float v = (S1 / n) * S2 * (S3 / n);
-          if (!isfinite(S1) || !isfinite(v)) v = NAN;
-          a.vp[(size_t)(j - 2) * (size_t)a.vstride + (size_t)ty * a.Tx + tx] = v;
+        if (tx >= a.Tx || ty >= a.Ty) return;
+        const int hw = min(g.w, a.ny - ty * g.w);
+        const int ww = min(g.w, a.nx - tx * g.w);
+        const float n = (float)(hw * ww);
+        float v = (S1 / n) * S2 * (S3 / n);
+        if (!isfinite(S1) || !isfinite(v)) v = NAN;
+        vp[(size_t)(j - 2) * (size_t)a.vstride + (size_t)ty * a.Tx + tx] = v;
+      };
+      if (per <= 2) {
+        // windows of 1 and 2: the one or two partials of a tile by one thread
+        // (a warp per tile took 51.7 ms for 64 x 2048^2 at w = 1)
+        for (int tt = tid; tt < NT; tt += g.threads) {
+          const int tb = tt / g.TBX, tbx = tt - (tt / g.TBX) * g.TBX;
+          float4 q = pp[tb * g.BW + tbx * per];
+          if (per == 2) {
+            const float4 h = pp[tb * g.BW + tbx * per + 1];
+            q.x += h.x;
+            q.y = fmaxf(q.y, h.y);
+            q.z += h.z;
+          }
+          finish(tb, tbx, q.x, q.y, q.z);
+        }
+      } else {
+        // One full warp per tile combines the tile's nseg * w column partials:
+        // lanes stride over them, then a fixed shuffle tree (deterministic).
+        // Warps take tiles round-robin; a trailing partial warp takes none.
+        const int warp = tid >> 5, lane = tid & 31, nwf = g.threads >> 5;
+        for (int tt = warp; tt < NT && warp < nwf; tt += nwf) {
+          const int tb = tt / g.TBX;
+          const int tbx = tt - tb * g.TBX;
+          float S1 = 0.f, S2 = 0.f, S3 = 0.f;
+          for (int i = lane; i < per; i += 32) {
+            const int sg = i / g.w, cc = i - sg * g.w;
+            const float4 q = pp[(tb * g.nseg + sg) * g.BW + tbx * g.w + cc];
+            S1 += q.x;
+            S2 = fmaxf(S2, q.y);
+            S3 += q.z;
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            S1 += __shfl_xor_sync(0xffffffffu, S1, o);
+            S2 = fmaxf(S2, __shfl_xor_sync(0xffffffffu, S2, o));
+            S3 += __shfl_xor_sync(0xffffffffu, S3, o);
+          }
+          if (lane == 0) finish(tb, tbx, S1, S2, S3);
         }
       }
     }
@@ -242,7 +246,9 @@ struct Ring {
 
 // One field as the march sees it.
 struct FieldView {
-  int nx, ny, L, Tx, Ty;
+  int nx, ny, Tx, Ty;
+  int L;      // snapshots to march over
+  int ring;   // stack slots: snapshot j is slot (zrot + j) % ring
   int zrot;
   const float* key = nullptr;   // FP32 key frame of a difference-coded stack
   int64_t kpitch = 0;
@@ -303,7 +309,7 @@ __device__ __forceinline__ bool ring_wait(const Ring& rg, uint64_t deadline) {
 // j + NS and advance the ring.
 __device__ __forceinline__ bool ring_release(Ring& rg, bool ok, const CUtensorMap* tmap,
                                              unsigned* status, int j, int L, int x0, int y0,
-                                             int zrot) {
+                                             int zrot, int ring) {
   if (__syncthreads_or(!ok)) {
     if (threadIdx.x == 0) {
       atomicOr(status, kErrTimeout);
@@ -323,7 +329,7 @@ __device__ __forceinline__ bool ring_release(Ring& rg, bool ok, const CUtensorMa
   if (threadIdx.x == 0 && j + rg.NS < L) {
     fence_proxy_async_smem();
     mbar_expect_tx(rg.bar0 + 8 * rg.stg, rg.box_bytes);
-    tma_load_3d(rg.stage0 + rg.stg * rg.stage_bytes, tmap, x0, y0, (zrot + j + rg.NS) % L,
+    tma_load_3d(rg.stage0 + rg.stg * rg.stage_bytes, tmap, x0, y0, (zrot + j + rg.NS) % ring,
                 rg.bar0 + 8 * rg.stg);
   }
   if (++rg.stg == rg.NS) {
@@ -362,17 +368,12 @@ __device__ __forceinline__ void load_row(const T* src, float* dst) {
 // arrays, so that the caller alternates them and no value is copied), and
 // returns the tile sums.  Row partials first, then the rows in order: short
 // dependency chains for the sums, the maximum with its first position in
-// row-major order (strict >), and this snapshot's maximum sm.
-//
-// ABS reading: for x != 0, r = sat(Delta * |1/x|) needs no guard.  A row whose
-// reference pixels multiply to a non-zero product has no zero among them and
-// takes that form; any other row (a zero pixel, the zero fill outside the
-// image, or a product that underflows) takes the guarded form of Eq. 5.  Both
-// give the same r for a non-zero x.
+// row-major order (strict >, only with ARG), and this snapshot's maximum sm.
 // With DELTA the stage holds the differences q^(s+2) and the row is decoded
-// first: x^(s+2) = fl32(x^(s+1) + q^(s+2)), the coder's own sum.
-template <typename T, int W, bool SIGNED, bool DELTA = false>
-__device__ __forceinline__ void tile_unit(const T* st, const float (&xp)[W * W],
+// first: x^(s+2) = fl32(x^(s+1) + q^(s+2)), the coder's own sum.  With FAST no
+// x^(s+1) of the tile is zero.
+template <typename T, int W, int LD, bool SIGNED, bool DELTA, bool ARG, bool FAST>
+__device__ __forceinline__ void tile_rows(const T* st, const float (&xp)[W * W],
                                           const float (&dp)[W * W], float (&xn)[W * W],
                                           float (&dn)[W * W], float& sm, float& s1, float& s2,
                                           float& s3, int& am) {
@@ -385,7 +386,7 @@ __device__ __forceinline__ void tile_unit(const T* st, const float (&xp)[W * W],
     float r1 = 0.f, r3 = 0.f, rm = 0.f;
     int ri = 0;
     float dd[W];
-    load_row<T, W>(st + r * (32 * W), &xn[r * W]);
+    load_row<T, W>(st + r * LD, &xn[r * W]);
     if (DELTA) {
 #pragma unroll
       for (int q = 0; q < W; ++q) xn[r * W + q] = __fadd_rn(xp[r * W + q], xn[r * W + q]);
@@ -397,28 +398,55 @@ __device__ __forceinline__ void tile_unit(const T* st, const float (&xp)[W * W],
       dn[i] = fabsf(xn[i] - xp[i]);       // D^(s+1)
       dd[q] = fabsf(dn[i] - dp[i]);       // Delta
       r1 += dd[q];
-      if (dd[q] > rm) {
+      if (ARG && dd[q] > rm) {
         rm = dd[q];
         ri = q;
       }
-    }
-    float pz = xp[r * W];
-#pragma unroll
-    for (int q = 1; q < W; ++q) pz *= xp[r * W + q];
-    if (SIGNED || pz == 0.f) {
-#pragma unroll
-      for (int q = 0; q < W; ++q) r3 += r_term<SIGNED>(dd[q], xp[r * W + q]);
-    } else {
-#pragma unroll
-      for (int q = 0; q < W; ++q) r3 += __saturatef(dd[q] * fabsf(rcp_approx(xp[r * W + q])));
+      if (FAST) r3 += __saturatef(dd[q] * fabsf(rcp_approx(xp[i])));
+      else r3 += r_term<SIGNED>(dd[q], xp[i]);
     }
     s1 += r1;
     s3 += r3;
-    if (rm > s2) {
-      s2 = rm;
-      am = r * W + ri;
+    if (ARG) {
+      if (rm > s2) {
+        s2 = rm;
+        am = r * W + ri;
+      }
+    } else {
+      s2 = row_max<W>(s2, dd);
     }
   }
+}
+
+// ABS reading: for x != 0, r = sat(Delta * |1/x|) needs no guard.  A row whose
+// reference pixels multiply to a non-zero product has no zero among them; a
+// tile of such rows takes that form, any other (a zero pixel, the zero fill
+// outside the image, a product that underflows) the guarded form of Eq. 5.
+// Both give the same r for a non-zero x.  The test is made once per tile, so
+// that all rows are straight-line code and one row's loads and reciprocals
+// overlap the next row's sums, and the registers of one row at a time are live:
+// w = 5 fell from 180 to 127, four CTAs per SM instead of two (a test and two
+// branches per row before: 64 x 2048^2 FP32, w = 4: 222 -> 178 us, w = 6: 292 ->
+// 238; 64 x 4096^2, w = 5: BF16 684 -> 664, difference-coded 724 -> 698).
+template <typename T, int W, int LD, bool SIGNED, bool DELTA, bool ARG>
+__device__ __forceinline__ void tile_unit(const T* st, const float (&xp)[W * W],
+                                          const float (&dp)[W * W], float (&xn)[W * W],
+                                          float (&dn)[W * W], float& sm, float& s1, float& s2,
+                                          float& s3, int& am) {
+  bool fast = !SIGNED;
+  if (!SIGNED) {
+#pragma unroll
+    for (int r = 0; r < W; ++r) {
+      float pz = xp[r * W];
+#pragma unroll
+      for (int q = 1; q < W; ++q) pz *= xp[r * W + q];
+      fast = fast && pz != 0.f;
+    }
+  }
+  if (fast)
+    tile_rows<T, W, LD, SIGNED, DELTA, ARG, true>(st, xp, dp, xn, dn, sm, s1, s2, s3, am);
+  else
+    tile_rows<T, W, LD, SIGNED, DELTA, ARG, false>(st, xp, dp, xn, dn, sm, s1, s2, s3, am);
 }
 
 // Snapshots 0 and 1 of a tile: x^(j) into xn, and D^(0) once j == 1.  With
@@ -488,7 +516,8 @@ __device__ __forceinline__ bool march_small(const CUtensorMap* tmap, const Field
     int s = rg.stg;
     for (int j = j0; j < j0 + rg.NS && j < L; ++j) {
       mbar_expect_tx(rg.bar0 + 8 * s, rg.box_bytes);
-      tma_load_3d(rg.stage0 + s * rg.stage_bytes, tmap, x0, y0, (f.zrot + j) % L, rg.bar0 + 8 * s);
+      tma_load_3d(rg.stage0 + s * rg.stage_bytes, tmap, x0, y0, (f.zrot + j) % f.ring,
+                  rg.bar0 + 8 * s);
       if (++s == rg.NS) s = 0;
     }
   }
@@ -515,7 +544,7 @@ __device__ __forceinline__ bool march_small(const CUtensorMap* tmap, const Field
       if (j == 0) tile_load<T, W>(stage(), xb, xa, da, true, sm);
       else tile_load<T, W, DELTA>(stage(), xa, xb, db, false, sm);
     }
-    if (!ring_release(rg, ok, tmap, f.status, j, L, x0, y0, f.zrot)) return false;
+    if (!ring_release(rg, ok, tmap, f.status, j, L, x0, y0, f.zrot, f.ring)) return false;
     mx = fmaxf(mx, sm);
     if (f.smax) warp_max_to(sm, f.smax + j);
   }
@@ -526,8 +555,8 @@ __device__ __forceinline__ bool march_small(const CUtensorMap* tmap, const Field
     float sm = -INFINITY;
     float s1 = 0.f, s2 = 0.f, s3 = 0.f;
     int am = 0;
-    if (ok) tile_unit<T, W, SIGNED, DELTA>(stage(), xp, dp, xn, dn, sm, s1, s2, s3, am);
-    if (!ring_release(rg, ok, tmap, f.status, j, L, x0, y0, f.zrot)) return false;
+    if (ok) tile_unit<T, W, 32 * W, SIGNED, DELTA, true>(stage(), xp, dp, xn, dn, sm, s1, s2, s3, am);
+    if (!ring_release(rg, ok, tmap, f.status, j, L, x0, y0, f.zrot, f.ring)) return false;
     mx = fmaxf(mx, sm);
     if (f.smax) warp_max_to(sm, f.smax + j);
     if (live) {
@@ -559,16 +588,19 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_stack_small(const __grid_c
   Ring rg;
   ring_init(rg, smem, a.g, (int)sizeof(T));
   FieldView f;
+  const int s0 = blockIdx.z * a.seg_units;   // first unit of the segment
+  const size_t v0 = (size_t)s0 * (size_t)a.vstride;
   f.nx = a.nx;
   f.ny = a.ny;
-  f.L = a.nsnap;
+  f.L = min(a.seg_units, a.nsnap - 2 - s0) + 2;
+  f.ring = a.nsnap;
   f.Tx = a.Tx;
   f.Ty = a.Ty;
-  f.zrot = a.zrot;
+  f.zrot = a.zrot + s0;
   f.vstride = a.vstride;
-  f.vp = a.vp;
-  f.arg = a.arg;
-  f.smax = a.smax;
+  f.vp = a.vp + v0;
+  f.arg = a.arg ? a.arg + v0 : nullptr;
+  f.smax = a.smax ? a.smax + s0 : nullptr;
   f.status = a.status;
   f.key = a.key;
   f.kpitch = a.kpitch;
@@ -606,7 +638,10 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
   const int w = g.w, gl = w / 4;             // lanes (and warps) per tile side
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nw = g.threads >> 5;
-  const int L = a.nsnap;
+  const int s0 = blockIdx.z * a.seg_units;                // first unit of the segment
+  const int L = min(a.seg_units, a.nsnap - 2 - s0) + 2;   // its snapshots
+  const int z0 = a.zrot + s0;
+  unsigned* const smax = a.smax ? a.smax + s0 : nullptr;
   const int x0 = blockIdx.x * kSubCols, y0 = blockIdx.y * g.BH;
   float4* part = reinterpret_cast<float4*>(smem + sub_part_offset(g));   // [2][nw][TBX]
   const int off = (warp * 4) * kSubCols + lane * 4;
@@ -615,7 +650,8 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
     int s = rg.stg;
     for (int j = j0; j < j0 + rg.NS && j < L; ++j) {
       mbar_expect_tx(rg.bar0 + 8 * s, rg.box_bytes);
-      tma_load_3d(rg.stage0 + s * rg.stage_bytes, tmap, x0, y0, (a.zrot + j) % L, rg.bar0 + 8 * s);
+      tma_load_3d(rg.stage0 + s * rg.stage_bytes, tmap, x0, y0, (z0 + j) % a.nsnap,
+                  rg.bar0 + 8 * s);
       if (++s == rg.NS) s = 0;
     }
   }
@@ -632,13 +668,13 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
     const int hw = min(w, a.ny - rty * w), ww = min(w, a.nx - rtx * w);
     inv_n = 1.f / (float)(hw * ww);
   }
-  float* out = a.vp + (rlive ? (size_t)rty * a.Tx + rtx : 0);
+  float* out = a.vp + (size_t)s0 * (size_t)a.vstride + (rlive ? (size_t)rty * a.Tx + rtx : 0);
   float xa[N], da[N], xb[N], db[N];
   if (DELTA) {
     float sm = -INFINITY;
     key_load<4, 4>(a.key, a.kpitch, x0 + lane * 4, y0 + warp * 4, a.nx, a.ny, xa, sm);
     mx = fmaxf(mx, sm);
-    if (a.smax) warp_max_to(sm, a.smax);
+    if (smax) warp_max_to(sm, smax);
   }
 #pragma unroll
   for (int j = j0; j < 2; ++j) {
@@ -649,9 +685,9 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
       if (j == 0) tile_load<T, 4>(stage(), xb, xa, da, true, sm);
       else tile_load<T, 4, DELTA>(stage(), xa, xb, db, false, sm);
     }
-    if (!ring_release(rg, ok, tmap, a.status, j, L, x0, y0, a.zrot)) return false;
+    if (!ring_release(rg, ok, tmap, a.status, j, L, x0, y0, z0, a.nsnap)) return false;
     mx = fmaxf(mx, sm);
-    if (a.smax) warp_max_to(sm, a.smax + j);
+    if (smax) warp_max_to(sm, smax + j);
   }
   auto unit = [&](int j, const float (&xp)[N], const float (&dp)[N], float (&xn)[N],
                   float (&dn)[N]) -> bool {
@@ -659,7 +695,7 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
     float sm = -INFINITY;
     float s1 = 0.f, s2 = 0.f, s3 = 0.f;
     int am = 0;
-    if (ok) tile_unit<T, 4, SIGNED, DELTA>(stage(), xp, dp, xn, dn, sm, s1, s2, s3, am);
+    if (ok) tile_unit<T, 4, kSubCols, SIGNED, DELTA, false>(stage(), xp, dp, xn, dn, sm, s1, s2, s3, am);
     for (int o = gl >> 1; o > 0; o >>= 1) {
       s1 += __shfl_xor_sync(0xffffffffu, s1, o);
       s2 = fmaxf(s2, __shfl_xor_sync(0xffffffffu, s2, o));
@@ -667,9 +703,9 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
     }
     float4* pp = part + (size_t)(j & 1) * nw * g.TBX;
     if (lane % gl == 0) pp[warp * g.TBX + lane / gl] = make_float4(s1, s2, s3, 0.f);
-    if (!ring_release(rg, ok, tmap, a.status, j, L, x0, y0, a.zrot)) return false;
+    if (!ring_release(rg, ok, tmap, a.status, j, L, x0, y0, z0, a.nsnap)) return false;
     mx = fmaxf(mx, sm);
-    if (a.smax) warp_max_to(sm, a.smax + j);
+    if (smax) warp_max_to(sm, smax + j);
     if (rlive) {
       float S1 = 0.f, S2 = 0.f, S3 = 0.f;
       for (int k = 0; k < gl; ++k) {
@@ -691,10 +727,11 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
   return true;
 }
 
-// MAXT = 256 (w <= 32, eight warps) leaves room for three CTAs per SM;
-// MAXT = 512 (w = 64, sixteen warps) for one.
+// MAXT = 256 (w <= 32, eight warps): two CTAs per SM and 128 registers, which
+// spill nothing (three CTAs at 80 registers spilled 48 bytes a thread: w = 32,
+// 200 x 2048^2: 746 against 688 us); MAXT = 512 (w = 64, sixteen warps): one.
 template <typename T, bool SIGNED, int MAXT, bool DELTA>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1) k_stack_sub(const __grid_constant__ CUtensorMap tmap,
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) k_stack_sub(const __grid_constant__ CUtensorMap tmap,
                                                                 const StackArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   if (threadIdx.x == 0) prefetch_tmap(&tmap);
@@ -743,7 +780,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_stack_multi(const FieldDes
     FieldView f;
     f.nx = d.nx;
     f.ny = d.ny;
-    f.L = d.L;
+    f.L = f.ring = d.L;
     f.Tx = d.Tx;
     f.Ty = d.Ty;
     f.zrot = d.zrot;
@@ -989,6 +1026,30 @@ bool stack_geometry(int w, int elem_bytes, StackGeom* g) {
   return true;
 }
 
+// A unit needs its own three snapshots only, so a march may be split along time
+// into segments that share two snapshots (read twice).  The boxes alone decide
+// how full the chip is: 1024 boxes of w = 32 on 456 resident CTAs are 2.25
+// waves that take the time of three, a 512 x 512 field has 104 boxes in all.
+// The number of segments is the one with the least (waves) x (snapshots per
+// CTA, its shared two and about one to fill the ring included); many waves
+// leave it at one, where nothing is read twice.  Measured: 1500 x 2048^2 at
+// w = 32 5.99 -> 5.47 ms (four segments), 16 x 512^2 at w = 5 18.5 -> 10.8 us.
+int march_seg_units(int64_t boxes, int per_sm, int units) {
+  const int64_t slots = 152ll * std::max(1, per_sm);
+  int best = units;
+  int64_t cost = INT64_MAX;
+  for (int s = 1; s <= std::min(units, 64); ++s) {
+    const int u = (units + s - 1) / s;
+    const int64_t n = (units + u - 1) / u;   // segments of u units
+    const int64_t c = (boxes * n + slots - 1) / slots * (u + 3);
+    if (c < cost) {
+      cost = c;
+      best = u;
+    }
+  }
+  return best;
+}
+
 template <typename T, int R, bool SIGNED>
 static cudaError_t launch_one(const CUtensorMap* tmap, const StackArgs& a, cudaStream_t st) {
   auto kern = k_stack_tile<T, R, SIGNED>;
@@ -999,10 +1060,7 @@ static cudaError_t launch_one(const CUtensorMap* tmap, const StackArgs& a, cudaS
     if (e != cudaSuccess) return e;
     configured = a.g.smem_bytes;
   }
-  dim3 grid(a.g.gridX, a.g.gridY);
-  kern<<<grid, a.g.threads, a.g.smem_bytes, st>>>(*tmap, a);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_segments(kern, tmap, a, st);
 }
 
 template <typename T, int W, bool SIGNED, bool DELTA>
@@ -1015,10 +1073,7 @@ static cudaError_t launch_small(const CUtensorMap* tmap, const StackArgs& a, cud
     if (e != cudaSuccess) return e;
     configured = a.g.smem_bytes;
   }
-  dim3 grid(a.g.gridX, a.g.gridY);
-  kern<<<grid, a.g.threads, a.g.smem_bytes, st>>>(*tmap, a);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_segments(kern, tmap, a, st);
 }
 
 template <typename T, bool SIGNED, bool DELTA>
@@ -1032,10 +1087,7 @@ static cudaError_t launch_sub(const CUtensorMap* tmap, const StackArgs& a, cudaS
     if (e != cudaSuccess) return e;
     configured[big] = a.g.smem_bytes;
   }
-  dim3 grid(a.g.gridX, a.g.gridY);
-  kern<<<grid, a.g.threads, a.g.smem_bytes, st>>>(*tmap, a);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_segments(kern, tmap, a, st);
 }
 
 // Difference-coded half stacks (a.key set): the thread-per-tile and sub-tile
