@@ -176,6 +176,7 @@ struct StackGeom {
   size_t stage_bytes; // boxW * BH * elem, rounded to 128
   size_t smem_bytes;
   int gridX, gridY;
+  bool col = false;   // the column march (k_col.cuh): windows 7 and 9..15
 };
 
 struct StackArgs {
@@ -221,6 +222,9 @@ cudaError_t launch_stack_multi(const FieldDesc* fields, int nfields, int64_t nit
 int multi_blocks_per_sm(const StackGeom& g, int storage, int rmode);
 
 bool stack_geometry(int w, int elem_bytes, StackGeom* g);
+bool col_geometry(int w, int elem_bytes, StackGeom* g);
+template <typename T, bool SIGNED>
+cudaError_t launch_col(const CUtensorMap* tmap, const StackArgs& a, cudaStream_t st);
 // Thread-per-tile geometry for 3 <= w <= 6 with TBY tile rows per CTA and a
 // ring of `stages` buffers (the autotuner's search space).
 bool small_geometry(int w, int elem_bytes, int tby, int stages, StackGeom* g);

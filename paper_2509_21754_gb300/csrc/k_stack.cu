@@ -969,6 +969,7 @@ bool stack_geometry(int w, int elem_bytes, StackGeom* g) {
   if (w < 1 || w > 128) return false;
   if (w >= 3 && w <= kSmallMaxW && small_geometry(w, elem_bytes, 4, 4, g)) return true;
   if (sub_geometry(w, elem_bytes, g)) return true;
+  if (col_geometry(w, elem_bytes, g)) return true;
   // rows per thread R (a template value) and row segments per tile band
   int R, nseg;
   if (w <= 8) {
@@ -1113,6 +1114,7 @@ static cudaError_t launch_delta(const CUtensorMap* tmap, const StackArgs& a, cud
 template <typename T, bool SIGNED>
 static cudaError_t launch_r(const CUtensorMap* tmap, const StackArgs& a, cudaStream_t st) {
   if (a.key) return launch_delta<T, SIGNED>(tmap, a, st);
+  if (a.g.col) return launch_col<T, SIGNED>(tmap, a, st);
   if (a.g.R < 0) return launch_sub<T, SIGNED, false>(tmap, a, st);
   if (a.g.R == 0) {
     switch (a.g.w) {

@@ -26,6 +26,29 @@ __device__ __forceinline__ void max_to(float v, unsigned* key, bool full_warp) {
   if (v > -INFINITY) atomicMax(key, f32_key(v));
 }
 
+// The sums and maximum of one tile's PER column partials, added in the order
+// of a warp that holds one per lane and adds across the lanes by halves (16, 8,
+// 4, 2, 1): node<PER, O, l> is lane l after the step of distance O.  One thread does it, because a warp per
+// tile with its fifteen shuffles costs more instructions than a small tile's
+// pixels.
+template <int PER, int O, int LANE>
+__device__ __forceinline__ float3 partials_node(const float4* p) {
+  static_assert(PER <= 32, "one partial per lane");
+  if constexpr (O == 32) {
+    const float4 q = p[LANE];
+    return make_float3(q.x, q.y, q.z);
+  } else {
+    float3 r = partials_node<PER, 2 * O, LANE>(p);
+    if constexpr (LANE + O < PER) {   // the absent lanes' zeros change nothing
+      const float3 h = partials_node<PER, 2 * O, LANE + O>(p);
+      r.x += h.x;
+      r.y = fmaxf(r.y, h.y);
+      r.z += h.z;
+    }
+    return r;
+  }
+}
+
 // Launches a march kernel over its boxes and time segments.  A difference-coded
 // stack is decoded from its first snapshot on, so it has one segment.
 template <typename K>
