@@ -357,7 +357,8 @@ struct BlockScratch {
   uint32_t* sbits;            // [groups][Ty][words] selected-tile bitmap (v > thr)
   unsigned long long* pairs;  // [blocks][pairs per block] selected neighbours across block edges
   int64_t pcap;
-  int4* bstat;                // [blocks] boundary components, pairs, selected tiles of each block
+  int4* bstat;                // [blocks] boundary components, pairs, selected tiles of each block,
+                              // 1 while the block is left to k_blk_cc_full
   int* counters;              // [2] peaks
   int64_t cap;                // boundary-component slots (blocks x slots per block)
   int words;                  // bitmap words per tile row
@@ -416,9 +417,9 @@ cudaError_t launch_emit_candidates(const CandArgs& a, const SelectScratch& s, in
 cudaError_t launch_emit_peaks(const CandArgs& a, const SelItem* peaks, const int* npeak,
                               int* base, fitrig_candidate* tmp, cudaStream_t st);
 // The image candidates of a launch_block_select run without a peak list
-// (peaks == nullptr), from its peak bitmap: needs a.arg, a.w <= 8 and
-// Tx <= 1024 (one bitmap word per lane of a row's warp); the
-// same candidates, in the same places, as launch_emit_peaks on the list.
+// (peaks == nullptr), from its peak bitmap: needs a.w <= 8 and a.arg, or a.w
+// == 1; the same candidates, in the same places, as launch_emit_peaks on the
+// list.
 // Adds the peak count to *a.nout.
 cudaError_t launch_emit_rows(const CandArgs& a, const float* vals, int groups, const BlockScratch& b,
                              int64_t cap, int* base, cudaStream_t st);

@@ -549,107 +549,115 @@ __global__ void __launch_bounds__(kMaskThreads) k_blk_mask(const float* __restri
   }
 }
 
-__global__ void __launch_bounds__(kBlkThreads, 6) k_blk_cc(const float* __restrict__ vals,
-                                                        int64_t stride, int Tx, int Ty,
-                                                        BlockScratch b, unsigned* status) {
-  pdl_begin();
-  __shared__ uint32_t wsh[kBlkY + 2][4];      // bitmap words: rows ty0-1 .. ty0+kBlkY, words w0-1 .. w0+2
-  __shared__ unsigned long long mrow[kBlkY];   // the block's rows
-  __shared__ unsigned long long htop, hbot;   // halo rows above / below (block columns)
-  __shared__ unsigned long long hleft, hright;   // halo columns (bit = block row)
-  __shared__ uint32_t hcorner;                // bits: 0 top-left, 1 top-right, 2 bottom-left, 3 bottom-right
-  __shared__ int runbase[kBlkY + 1];          // first run of each row; runbase[kBlkY] = runs
-  __shared__ uint32_t rinfo[kBlkMaxRuns];     // run: row << 16 | start << 8 | end
-  __shared__ __align__(16) short par[kBlkMaxRuns];   // union-find over runs (CAS on aligned words)
-  __shared__ unsigned long long pkey[kBlkMaxRuns];   // peak key of each root; its id once known
-  __shared__ uint32_t bnd[kBlkMaxRuns / 32];         // boundary flag of each root (bit mask)
-  __shared__ uint32_t pw[kBlkY][2];
-  __shared__ int nsel_sh, nbnd_sh, npair_sh;
-  const int g = blockIdx.z;
+// The labelling of one block by NT threads, for blocks of at most MAXR runs.
+// Returns false, with nothing written, when the block has more (then every
+// thread sees it).
+template <int NT, int MAXR>
+struct BlkShared {
+  unsigned long long mrow[kBlkY];   // the block's rows
+  unsigned long long htop, hbot;    // halo rows above / below (block columns)
+  unsigned long long hleft, hright;   // halo columns (bit = block row)
+  unsigned long long pkey[MAXR];    // peak key of each root; its id once known
+  uint32_t rinfo[MAXR];             // run: row << 16 | start << 8 | end
+  uint32_t bnd[MAXR / 32];          // boundary flag of each root (bit mask)
+  uint32_t pw[kBlkY][2];
+  int runbase[kBlkY + 1];           // first run of each row; runbase[kBlkY] = runs
+  int wrun[NT / 32];
+  __align__(4) short par[MAXR];     // union-find over runs (CAS on aligned words)
+  uint32_t hcorner;                 // bits: 0 top-left, 1 top-right, 2 bottom-left, 3 bottom-right
+  int nsel, nbnd, npair;
+};
+
+template <int NT, int MAXR>
+__device__ __forceinline__ bool blk_label(BlkShared<NT, MAXR>& sh, const float* __restrict__ vals,
+                                          int64_t stride, int Tx, int Ty, const BlockScratch& b,
+                                          int64_t bidx, int g, int bx, int by, unsigned* status) {
+  static_assert(NT >= 64 && MAXR <= kBlkMaxRuns, "a thread per row");
+  constexpr int kIter = (MAXR + NT - 1) / NT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // this block's slots: boundary ids bidx * kBlkIds + k, pairs bidx * kBlkPairs + k
-  const int64_t bidx = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  const int tx0 = blockIdx.x * kBlkX, ty0 = blockIdx.y * kBlkY;
+  const int tx0 = bx * kBlkX, ty0 = by * kBlkY;
   const int w0 = tx0 / 32;
-  // 1. the bitmap words of the block's rows and of the halo rows (the words
-  // on either side hold the halo columns' bits); outside the map: 0
-  const uint32_t* sb = b.sbits + (size_t)g * Ty * b.words;
-  for (int q = tid; q < (kBlkY + 2) * 4; q += kBlkThreads) {
-    const int r = q >> 2, k = q & 3;
-    const int ty = ty0 - 1 + r, w = w0 - 1 + k;
-    uint32_t word = 0u;
-    if (ty >= 0 && ty < Ty && w >= 0 && w < b.words) word = sb[(size_t)ty * b.words + w];
-    wsh[r][k] = word;
-  }
   if (tid == 0) {
-    hleft = hright = 0ull;
-    hcorner = 0u;
-    nsel_sh = nbnd_sh = npair_sh = 0;
+    sh.hleft = sh.hright = 0ull;
+    sh.hcorner = 0u;
+    sh.nsel = sh.nbnd = sh.npair = 0;
   }
-  if (tid < kBlkY) pw[tid][0] = pw[tid][1] = 0u;
   __syncthreads();
-  // 2. rows as 64-bit masks, the halo rows, columns and corners
-  if (tid < kBlkY + 2) {
-    const int r = tid - 1;   // block row -1 .. kBlkY
-    const unsigned long long m = ((unsigned long long)wsh[tid][2] << 32) | wsh[tid][1];
-    const bool left = (wsh[tid][0] >> 31) != 0u, right = (wsh[tid][3] & 1u) != 0u;
+  // 1. the block's rows as 64-bit masks, the halo rows, columns and corners,
+  // from the bitmap words of rows ty0-1 .. ty0+kBlkY (the words on either side
+  // hold the halo columns' bits); outside the map: 0.  The last threads take
+  // the halo rows.
+  const uint32_t* sb = b.sbits + (size_t)g * Ty * b.words;
+  int rc = 0, rincl = 0;
+  unsigned long long mine = 0ull;
+  for (int q = tid; q < kBlkY + 2; q += NT) {
+    const int r = q < kBlkY ? q : (q == kBlkY ? -1 : kBlkY);   // block row
+    const int ty = ty0 + r;
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int wx = w0 - 1 + k;
+      w[k] = (ty >= 0 && ty < Ty && wx >= 0 && wx < b.words) ? sb[(size_t)ty * b.words + wx] : 0u;
+    }
+    const unsigned long long m = ((unsigned long long)w[2] << 32) | w[1];
+    const bool left = (w[0] >> 31) != 0u, right = (w[3] & 1u) != 0u;
     if (r < 0) {
-      htop = m;
-      if (left || right) atomicOr(&hcorner, (left ? 1u : 0u) | (right ? 2u : 0u));
+      sh.htop = m;
+      if (left || right) atomicOr(&sh.hcorner, (left ? 1u : 0u) | (right ? 2u : 0u));
     } else if (r >= kBlkY) {
-      hbot = m;
-      if (left || right) atomicOr(&hcorner, (left ? 4u : 0u) | (right ? 8u : 0u));
-    } else {
-      mrow[r] = m;
-      if (m) atomicAdd(&nsel_sh, __popcll((long long)m));
-      if (left) atomicOr(&hleft, 1ull << r);
-      if (right) atomicOr(&hright, 1ull << r);
+      sh.hbot = m;
+      if (left || right) atomicOr(&sh.hcorner, (left ? 4u : 0u) | (right ? 8u : 0u));
+    } else {   // q = tid: this thread's row
+      mine = m;
+      sh.mrow[r] = m;
+      sh.pw[r][0] = sh.pw[r][1] = 0u;
+      if (left) atomicOr(&sh.hleft, 1ull << r);
+      if (right) atomicOr(&sh.hright, 1ull << r);
     }
   }
-  __syncthreads();
-  // 3. the run list: counts per row, their scan (one thread per row, the
+  // 2. the run list: counts per row, their scan (one thread per row, the
   // first kBlkY / 32 warps), then each row's runs
-  __shared__ int wrun[kBlkY / 32];
-  int rc = 0, rincl = 0;
   if (tid < kBlkY) {
-    rc = __popcll((long long)run_starts(mrow[tid]));
+    rc = __popcll((long long)run_starts(mine));
     rincl = rc;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, rincl, o);
       if (lane >= o) rincl += y;
     }
-    if (lane == 31) wrun[warp] = rincl;
+    if (lane == 31) sh.wrun[warp] = rincl;
+    int n = __popcll((long long)mine);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+    if (lane == 0) atomicAdd(&sh.nsel, n);
   }
   __syncthreads();
+  int nr = 0;
+#pragma unroll
+  for (int w = 0; w < kBlkY / 32; ++w) nr += sh.wrun[w];
+  if (nr > MAXR) return false;
   if (tid < kBlkY) {
-    int before = 0;
-    for (int w = 0; w < warp; ++w) before += wrun[w];
-    const int k0 = before + rincl - rc;
-    runbase[tid] = k0;
-    if (tid == kBlkY - 1) runbase[kBlkY] = before + rincl;
-    const unsigned long long m = mrow[tid];
-    int k = k0;
-    for (unsigned long long st = run_starts(m); st; st &= st - 1, ++k) {
-      const int sb = __ffsll((long long)st) - 1;
-      const int eb = 63 - __clzll((long long)run_bits(m, sb));
-      rinfo[k] = ((uint32_t)tid << 16) | ((uint32_t)sb << 8) | (uint32_t)eb;
+    int k = rincl - rc;
+    for (int w = 0; w < warp; ++w) k += sh.wrun[w];
+    sh.runbase[tid] = k;
+    if (tid == 0) sh.runbase[kBlkY] = nr;
+    for (unsigned long long st = run_starts(mine); st; st &= st - 1, ++k) {
+      const int s0 = __ffsll((long long)st) - 1;
+      const int e0 = 63 - __clzll((long long)run_bits(mine, s0));
+      sh.rinfo[k] = ((uint32_t)tid << 16) | ((uint32_t)s0 << 8) | (uint32_t)e0;
+      sh.par[k] = (short)k;
+      sh.pkey[k] = 0ull;
     }
   }
+  for (int k = tid; k < MAXR / 32; k += NT) sh.bnd[k] = 0u;
   __syncthreads();
-  const int nr = runbase[kBlkY];
-  auto run_index = [&](int row, int sb) {   // run of `row` starting at bit sb
-    const unsigned long long st = run_starts(mrow[row]);
-    return runbase[row] + __popcll((long long)(st & ((1ull << sb) - 1ull)));
+  auto run_index = [&](int row, int s0) {   // run of `row` starting at bit s0
+    const unsigned long long st = run_starts(sh.mrow[row]);
+    return sh.runbase[row] + __popcll((long long)(st & ((1ull << s0) - 1ull)));
   };
-  for (int k = tid; k < nr; k += kBlkThreads) {
-    par[k] = (short)k;
-    pkey[k] = 0ull;
-  }
-  for (int k = tid; k < kBlkMaxRuns / 32; k += kBlkThreads) bnd[k] = 0u;
-  __syncthreads();
-  // 4. unions: each run with the touching runs of the row above
-  const volatile short* vpar = par;
+  // 3. unions: each run with the touching runs of the row above
+  const volatile short* vpar = sh.par;
   auto unite_r = [&](int a, int c) {
     for (int it = 0; it < (1 << 16); ++it) {
       while (vpar[a] != a) a = vpar[a];
@@ -657,21 +665,21 @@ __global__ void __launch_bounds__(kBlkThreads, 6) k_blk_cc(const float* __restri
       if (a == c) return;
       const int hi = a > c ? a : c, lo = a > c ? c : a;
       // 16-bit compare-and-swap through the aligned 32-bit word
-      unsigned* w = reinterpret_cast<unsigned*>(&par[hi & ~1]);
-      const unsigned sh = (hi & 1) ? 16u : 0u;
+      unsigned* w = reinterpret_cast<unsigned*>(&sh.par[hi & ~1]);
+      const unsigned shf = (hi & 1) ? 16u : 0u;
       const unsigned old = *reinterpret_cast<volatile unsigned*>(w);
-      if ((int)(short)(old >> sh) != hi) continue;
-      const unsigned nw = (old & ~(0xffffu << sh)) | ((unsigned)(unsigned short)lo << sh);
+      if ((int)(short)(old >> shf) != hi) continue;
+      const unsigned nw = (old & ~(0xffffu << shf)) | ((unsigned)(unsigned short)lo << shf);
       if (atomicCAS(w, old, nw) == old) return;
     }
     atomicOr(status, kErrCcLimit);
   };
-  for (int k = tid; k < nr; k += kBlkThreads) {
-    const uint32_t ri = rinfo[k];
-    const int row = ri >> 16, sb = (ri >> 8) & 255, eb = ri & 255;
+  for (int k = tid; k < nr; k += NT) {
+    const uint32_t ri = sh.rinfo[k];
+    const int row = ri >> 16, s0 = (ri >> 8) & 255, e0 = ri & 255;
     if (row == 0) continue;
-    const unsigned long long rb = (eb == 63 ? ~0ull : ((2ull << eb) - 1ull)) & ~((1ull << sb) - 1ull);
-    const unsigned long long u = mrow[row - 1];
+    const unsigned long long rb = (e0 == 63 ? ~0ull : ((2ull << e0) - 1ull)) & ~((1ull << s0) - 1ull);
+    const unsigned long long u = sh.mrow[row - 1];
     unsigned long long nb = (rb | (rb << 1) | (rb >> 1)) & u;
     while (nb) {
       const int ub = __ffsll((long long)nb) - 1;
@@ -681,106 +689,153 @@ __global__ void __launch_bounds__(kBlkThreads, 6) k_blk_cc(const float* __restri
     }
   }
   __syncthreads();
-  // 5. per run: its root (read-only), boundary flag, peak key
-  int rootv[(kBlkMaxRuns + kBlkThreads - 1) / kBlkThreads];
+  // 4. per run: its root (read-only), boundary flag, peak key
+  int rootv[kIter];
 #pragma unroll
-  for (int j = 0; j < (kBlkMaxRuns + kBlkThreads - 1) / kBlkThreads; ++j) {
-    const int k = tid + j * kBlkThreads;
+  for (int j = 0; j < kIter; ++j) {
+    const int k = tid + j * NT;
     rootv[j] = -1;
     if (k >= nr) continue;
     int r = k;
-    while (par[r] != r) r = par[r];
+    while (sh.par[r] != r) r = sh.par[r];
     rootv[j] = r;
-    const uint32_t ri = rinfo[k];
-    const int row = ri >> 16, sb = (ri >> 8) & 255, eb = ri & 255;
-    const unsigned long long rb = (eb == 63 ? ~0ull : ((2ull << eb) - 1ull)) & ~((1ull << sb) - 1ull);
+    const uint32_t ri = sh.rinfo[k];
+    const int row = ri >> 16, s0 = (ri >> 8) & 255, e0 = ri & 255;
+    const unsigned long long rb = (e0 == 63 ? ~0ull : ((2ull << e0) - 1ull)) & ~((1ull << s0) - 1ull);
     const unsigned long long dil = rb | (rb << 1) | (rb >> 1);
     bool out = false;
-    if (row == 0) out = out || (dil & htop) || (sb == 0 && (hcorner & 1u)) || (eb == 63 && (hcorner & 2u));
+    if (row == 0)
+      out = out || (dil & sh.htop) || (s0 == 0 && (sh.hcorner & 1u)) || (e0 == 63 && (sh.hcorner & 2u));
     if (row == kBlkY - 1)
-      out = out || (dil & hbot) || (sb == 0 && (hcorner & 4u)) || (eb == 63 && (hcorner & 8u));
+      out = out || (dil & sh.hbot) || (s0 == 0 && (sh.hcorner & 4u)) || (e0 == 63 && (sh.hcorner & 8u));
     // block rows row-1..row+1 as halo-column bits
     const unsigned long long near = row == 0 ? 3ull : (7ull << (row - 1));
-    if (sb == 0) out = out || (hleft & near);
-    if (eb == 63) out = out || (hright & near);
-    if (out) atomicOr(&bnd[r >> 5], 1u << (r & 31));
+    if (s0 == 0) out = out || (sh.hleft & near);
+    if (e0 == 63) out = out || (sh.hright & near);
+    if (out) atomicOr(&sh.bnd[r >> 5], 1u << (r & 31));
     unsigned long long key = 0ull;
     const uint32_t t0 = (uint32_t)((ty0 + row) * Tx + tx0);
     const float* vr = vals + (size_t)g * stride + t0;
 #pragma unroll 4
-    for (int c = sb; c <= eb; ++c) {
+    for (int c = s0; c <= e0; ++c) {
       const unsigned long long kc = peak_key(vr[c], t0 + (uint32_t)c);
       key = kc > key ? kc : key;
     }
-    atomicMax(&pkey[r], key);
+    atomicMax(&sh.pkey[r], key);
   }
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < (kBlkMaxRuns + kBlkThreads - 1) / kBlkThreads; ++j)
-    if (rootv[j] >= 0) par[tid + j * kBlkThreads] = (short)rootv[j];   // straight to the root
-  // 6. roots: an interior component's peak bit; a boundary component's id
+  for (int j = 0; j < kIter; ++j)
+    if (rootv[j] >= 0) sh.par[tid + j * NT] = (short)rootv[j];   // straight to the root
+  // 5. roots: an interior component's peak bit; a boundary component's id
 #pragma unroll
-  for (int j = 0; j < (kBlkMaxRuns + kBlkThreads - 1) / kBlkThreads; ++j) {
-    const int k = tid + j * kBlkThreads;
+  for (int j = 0; j < kIter; ++j) {
+    const int k = tid + j * NT;
     if (rootv[j] != k) continue;
-    const unsigned long long key = pkey[k];
-    if (!((bnd[k >> 5] >> (k & 31)) & 1u)) {
+    const unsigned long long key = sh.pkey[k];
+    if (!((sh.bnd[k >> 5] >> (k & 31)) & 1u)) {
       const uint32_t t = 0xffffffffu - (uint32_t)key;
       const int pty = (int)(t / (uint32_t)Tx), ptx = (int)(t - (uint32_t)pty * (uint32_t)Tx);
       const int ply = pty - ty0, plx = ptx - tx0;
-      atomicOr(&pw[ply][plx >> 5], 1u << (plx & 31));
+      atomicOr(&sh.pw[ply][plx >> 5], 1u << (plx & 31));
     } else {
-      const int slot = atomicAdd(&nbnd_sh, 1);   // < kBlkIds: each owns a ring tile
+      const int slot = atomicAdd(&sh.nbnd, 1);   // < kBlkIds: each owns a ring tile
       const int id = (int)(bidx * kBlkIds + slot);
       b.bpar[id] = id;
       b.bgrp[id] = g;
       b.bkey[id] = key;
       b.rkey[id] = key;
-      pkey[k] = (unsigned long long)id;   // only this thread reads or writes a root's slot here
+      sh.pkey[k] = (unsigned long long)id;   // only this thread reads or writes a root's slot here
     }
   }
   __syncthreads();
-  // 7. edge tiles of boundary components: their label, and each selected
+  // 6. edge tiles of boundary components: their label, and each selected
   // neighbour across the block edge with a larger tile index as a pair; the
   // block's peak words; the counts
   auto selected = [&](int ly, int lx) -> bool {   // -1 <= ly <= kBlkY, -1 <= lx <= kBlkX
     if (ly >= 0 && ly < kBlkY) {
-      if (lx >= 0 && lx < kBlkX) return (mrow[ly] >> lx) & 1ull;
-      return ((lx < 0 ? hleft : hright) >> ly) & 1ull;
+      if (lx >= 0 && lx < kBlkX) return (sh.mrow[ly] >> lx) & 1ull;
+      return ((lx < 0 ? sh.hleft : sh.hright) >> ly) & 1ull;
     }
-    if (lx >= 0 && lx < kBlkX) return ((ly < 0 ? htop : hbot) >> lx) & 1ull;
-    return (hcorner >> ((ly < 0 ? 0 : 2) + (lx < 0 ? 0 : 1))) & 1u;
+    if (lx >= 0 && lx < kBlkX) return ((ly < 0 ? sh.htop : sh.hbot) >> lx) & 1ull;
+    return (sh.hcorner >> ((ly < 0 ? 0 : 2) + (lx < 0 ? 0 : 1))) & 1u;
   };
-  if (tid < kBlkRing) {
-    int ly, lx;
-    ring_pos(tid, &ly, &lx);
-    if (selected(ly, lx)) {
-      const int r = par[run_index(ly, run_of(mrow[ly], lx))];
-      if ((bnd[r >> 5] >> (r & 31)) & 1u) {
-        const int64_t t = (int64_t)(ty0 + ly) * Tx + (tx0 + lx);
-        b.glab[(size_t)g * stride + t] = (int)pkey[r];
+  if (sh.nbnd > 0) {
+    for (int q = tid; q < kBlkRing; q += NT) {
+      int ly, lx;
+      ring_pos(q, &ly, &lx);
+      if (!selected(ly, lx)) continue;
+      const int r = sh.par[run_index(ly, run_of(sh.mrow[ly], lx))];
+      if (!((sh.bnd[r >> 5] >> (r & 31)) & 1u)) continue;
+      const int64_t t = (int64_t)(ty0 + ly) * Tx + (tx0 + lx);
+      b.glab[(size_t)g * stride + t] = (int)sh.pkey[r];
 #pragma unroll
-        for (int d = 0; d < 8; ++d) {
-          int dy, dx;
-          dir_offset(d, &dy, &dx);
-          const int ny = ly + dy, nx = lx + dx;
-          const bool outside = ny < 0 || ny >= kBlkY || nx < 0 || nx >= kBlkX;
-          if (!outside || !selected(ny, nx)) continue;
-          if (dy * Tx + dx <= 0) continue;   // the other tile records it
-          const int k = atomicAdd(&npair_sh, 1);   // < kBlkPairs: at most 4 per ring tile
-          b.pairs[bidx * kBlkPairs + k] =
-              ((unsigned long long)g << 40) | ((unsigned long long)t << 3) | (unsigned)d;
-        }
+      for (int d = 0; d < 8; ++d) {
+        int dy, dx;
+        dir_offset(d, &dy, &dx);
+        const int ny = ly + dy, nx = lx + dx;
+        const bool outside = ny < 0 || ny >= kBlkY || nx < 0 || nx >= kBlkX;
+        if (!outside || !selected(ny, nx)) continue;
+        if (dy * Tx + dx <= 0) continue;   // the other tile records it
+        const int k = atomicAdd(&sh.npair, 1);   // < kBlkPairs: at most 4 per ring tile
+        b.pairs[bidx * kBlkPairs + k] =
+            ((unsigned long long)g << 40) | ((unsigned long long)t << 3) | (unsigned)d;
       }
     }
   }
-  if (tid < 2 * kBlkY) {
-    const int ly = tid >> 1, wx = tid & 1;
+  for (int q = tid; q < 2 * kBlkY; q += NT) {
+    const int ly = q >> 1, wx = q & 1;
     const int ty = ty0 + ly, w = tx0 / 32 + wx;
-    if (ty < Ty && w < b.words) b.pbits[((size_t)g * Ty + ty) * b.words + w] = pw[ly][wx];
+    if (ty < Ty && w < b.words) b.pbits[((size_t)g * Ty + ty) * b.words + w] = sh.pw[ly][wx];
   }
   __syncthreads();
-  if (tid == 0) b.bstat[bidx] = make_int4(nbnd_sh, npair_sh, nsel_sh, 0);
+  if (tid == 0) b.bstat[bidx] = make_int4(sh.nbnd, sh.npair, sh.nsel, 0);
+  return true;
+}
+
+// A block holds a hundred or two runs where a few per cent of the tiles are
+// selected, and its labelling is a chain of short dependent steps: what counts
+// is how many blocks an SM has in hand.  Two warps and shared memory for
+// kBlkFewRuns runs let 20 blocks share an SM, where 256 threads and room for
+// the most runs a block can have (2048) let six.  A block with more runs is
+// marked (bstat.w) and left to k_blk_cc_full, launched next.  Bound by issue and
+// the divergence of its loops over runs.  30 sliding maps of 16.8 M pixels 1378
+// -> 688 us, 6 maps of 24.2 M tiles 528 -> 420 us, 62 maps of 672 k 114 -> 108.
+constexpr int kBlkFewThreads = 64;
+constexpr int kBlkFewRuns = 512;
+
+__global__ void __launch_bounds__(kBlkFewThreads, 20) k_blk_cc(const float* __restrict__ vals,
+                                                               int64_t stride, int Tx, int Ty,
+                                                               BlockScratch b, unsigned* status) {
+  pdl_begin();
+  __shared__ BlkShared<kBlkFewThreads, kBlkFewRuns> sh;
+  const int64_t bidx = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  if (!blk_label(sh, vals, stride, Tx, Ty, b, bidx, (int)blockIdx.z, (int)blockIdx.x,
+                 (int)blockIdx.y, status) &&
+      threadIdx.x == 0)
+    b.bstat[bidx] = make_int4(0, 0, 0, 1);
+}
+
+__global__ void __launch_bounds__(kBlkThreads) k_blk_cc_full(const float* __restrict__ vals,
+                                                             int64_t stride, int Tx, int Ty,
+                                                             int64_t nblocks, BlockScratch b,
+                                                             unsigned* status) {
+  pdl_begin();
+  __shared__ BlkShared<kBlkThreads, kBlkMaxRuns> sh;
+  const int nbx = (Tx + kBlkX - 1) / kBlkX, nby = (Ty + kBlkY - 1) / kBlkY;
+  for (int64_t b0 = (int64_t)blockIdx.x * kBlkThreads; b0 < nblocks;
+       b0 += (int64_t)gridDim.x * kBlkThreads) {
+    const int64_t i = b0 + threadIdx.x;
+    if (!__syncthreads_or(i < nblocks && b.bstat[i].w)) continue;
+    for (int k = 0; k < kBlkThreads && b0 + k < nblocks; ++k) {
+      const int64_t bidx = b0 + k;
+      if (!b.bstat[bidx].w) continue;   // the same word for every thread
+      __syncthreads();                  // nobody reads it any more, nor the last block's memory
+      blk_label(sh, vals, stride, Tx, Ty, b, bidx, (int)(bidx / ((int64_t)nbx * nby)),
+                (int)(bidx % nbx), (int)(bidx / nbx % nby), status);
+      __syncthreads();
+    }
+  }
 }
 
 // Unions of boundary components across block edges: one warp per block joins
@@ -1026,8 +1081,12 @@ cudaError_t launch_block_select(const float* vals, int groups, int64_t stride, i
                              dim3(kMaskThreads), 0, st, vals, stride, Tx, Ty, nrows, thr, b);
   const dim3 grid((Tx + kBlkX - 1) / kBlkX, (Ty + kBlkY - 1) / kBlkY, groups);
   if (e == cudaSuccess)
-    e = launch_pdl(k_blk_cc, grid, dim3(kBlkThreads), 0, st, vals, stride, Tx, Ty, b, status);
-  const unsigned wgrid = (unsigned)std::min<int64_t>((nblocks + 7) / 8, 152 * 16);   // a warp per block
+    e = launch_pdl(k_blk_cc, grid, dim3(kBlkFewThreads), 0, st, vals, stride, Tx, Ty, b, status);
+  if (e == cudaSuccess)
+    e = launch_pdl(k_blk_cc_full,
+                   dim3((unsigned)std::min<int64_t>((nblocks + kBlkThreads - 1) / kBlkThreads, 152 * 4)),
+                   dim3(kBlkThreads), 0, st, vals, stride, Tx, Ty, nblocks, b, status);
+  const unsigned wgrid = (unsigned)std::min<int64_t>((nblocks + 7) / 8, 152 * 64);   // a warp per block
   if (e == cudaSuccess)
     e = launch_pdl(k_blk_merge, dim3(wgrid), dim3(256), 0, st, stride, Tx, nblocks, b, status);
   if (e == cudaSuccess) e = launch_pdl(k_blk_resolve, dim3(wgrid), dim3(256), 0, st, nblocks, b);
@@ -1047,7 +1106,7 @@ cudaError_t launch_block_select(const float* vals, int groups, int64_t stride, i
   if (e == cudaSuccess)
     e = launch_pdl(k_blk_check, dim3(1), dim3(1024), 0, st, nblocks, b, cap, status, want);
   if (e != cudaSuccess) return e;
-  count_launches(peaks ? 9 : 8);
+  count_launches(peaks ? 10 : 9);
   return cudaGetLastError();
 }
 
@@ -1452,98 +1511,137 @@ __global__ void __launch_bounds__(kGroupWarps * 32) k_group_sort(CandArgs a, con
   }
 }
 
-// Image branch with the march's in-tile arg-max, w <= kRowsMaxW and rows of at
-// most 32 bitmap words (Tx <= 1024), straight from the peak bitmap: one warp
-// per tile row, one word per lane, writes the row's candidates in (snapshot,
-// y, x) order.  Inside a tile row that order is (dy, tx), so a peak's place is
-// the row's offset (from the scan of the rows' peak counts), the row's peaks
-// in lower in-tile rows, and the peaks of its own in-tile row at smaller tx
-// (warp scans of each lane's count per in-tile row).  Each lane reads the
-// arg-max byte and value of its first kRowsBatch peaks together and keeps
-// them; a lane with more reads the rest again.  The same candidates as
-// k_group_sort<true> on the compacted peak list, without that list.
+// Image branch straight from the peak bitmap, w <= kRowsMaxW: one warp per
+// tile row writes the row's candidates in (snapshot, y, x) order, a bitmap
+// word per lane, 32 words at a time.  Inside a tile row that order is (dy,
+// tx), so a peak's place is the row's offset (from the scan of the rows' peak
+// counts), the row's peaks in lower in-tile rows, and the peaks of its own
+// in-tile row at smaller tx (earlier words, then warp scans of each lane's
+// count per in-tile row).  Rows of more than 32 words (WIDE) are counted once
+// over all words first.  The in-tile row and column come from the march's
+// arg-max; in sliding mode and at w = 1 a tile is its pixel and there is
+// nothing to read.  Each lane reads the arg-max byte and value of its first
+// kRowsBatch peaks together and keeps them; a lane with more reads the rest
+// again.  No peak list, recomputed arg-max or sort is needed: 30 sliding maps
+// of 16.8 M pixels, 1.5 M candidates, 742 -> 160 us (k_pbits_write, k_emit_image
+// and k_group_sort before); 6 maps of 24.2 M tiles, 7.3 M candidates, 382 -> 284.
 constexpr int kRowsMaxW = 8;
 constexpr int kRowsBatch = 4;
-__global__ void __launch_bounds__(kPbThreads, 4) k_emit_rows(CandArgs a, const float* __restrict__ vals,
+template <bool WIDE, int MAXW>
+__global__ void __launch_bounds__(kPbThreads, MAXW == 1 ? 6 : 4) k_emit_rows(CandArgs a, const float* __restrict__ vals,
                                                           int64_t nrows, BlockScratch b,
                                                           int64_t cap, const int* base_) {
   pdl_begin();
   const int lane = threadIdx.x & 31;
   const int64_t r = ((int64_t)blockIdx.x * kPbThreads + threadIdx.x) >> 5;
-  if (r >= nrows) return;
-  const int w = a.w;
+  if (r >= nrows || (WIDE && b.rowcnt[r] == 0)) return;
+  const int w = MAXW == 1 ? 1 : a.w;
   const int g = (int)(r / a.Ty), ty = (int)(r - (int64_t)g * a.Ty);
   const int t0 = ty * a.Tx;
   const uint32_t* row = b.pbits + (size_t)r * b.words;
-  const uint8_t* ag = a.arg + (size_t)g * a.stride + t0;
+  const uint8_t* ag = a.arg ? a.arg + (size_t)g * a.stride + t0 : nullptr;
   const float* vg = vals + (size_t)g * a.stride + t0;
   const int64_t roff = row_offset(b, r);
   const int64_t base = *base_;
-  // one word per lane: each lane's first kRowsBatch peaks are read once
-  // (arg-max byte and value together) and kept; a lane with more reads the
-  // rest again
-  const uint32_t word = lane < b.words ? row[lane] : 0u;
-  int idx[kRowsBatch], tx[kRowsBatch];
-  float v[kRowsBatch];
-  uint32_t m = word;
+  auto arg_of = [&](int t) -> int { return MAXW == 1 ? 0 : ag[t]; };
+  // place of the next peak of each in-tile row over the words so far
+  int next[MAXW];
 #pragma unroll
-  for (int k = 0; k < kRowsBatch; ++k) {
-    idx[k] = -1;
-    tx[k] = 0;
-    v[k] = 0.f;
-    if (m) {
-      tx[k] = lane * 32 + __ffs(m) - 1;
-      m &= m - 1;
-      idx[k] = ag[tx[k]];
-      v[k] = vg[tx[k]];
+  for (int d = 0; d < MAXW; ++d) next[d] = 0;
+  if (WIDE && MAXW > 1) {
+    int cnt[MAXW];
+#pragma unroll
+    for (int d = 0; d < MAXW; ++d) cnt[d] = 0;
+    for (int wx = lane; wx < b.words; wx += 32)
+      for (uint32_t q = row[wx]; q; q &= q - 1) {
+        const int dy = arg_of(wx * 32 + __ffs(q) - 1) / w;
+#pragma unroll
+        for (int d = 0; d < MAXW; ++d) cnt[d] += dy == d;
+      }
+    int run = 0;
+#pragma unroll
+    for (int d = 0; d < MAXW; ++d) {
+      next[d] = run;
+      int c = cnt[d];
+#pragma unroll
+      for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      run += c;
     }
   }
-  const uint32_t rest = m;
-  int mine[kRowsMaxW];
+  for (int w0 = 0; w0 < b.words; w0 += 32) {
+    const int wx = w0 + lane;
+    const uint32_t word = wx < b.words ? row[wx] : 0u;
+    int idx[kRowsBatch], tx[kRowsBatch];
+    float v[kRowsBatch];
+    uint32_t m = word;
 #pragma unroll
-  for (int d = 0; d < kRowsMaxW; ++d) mine[d] = 0;
-#pragma unroll
-  for (int k = 0; k < kRowsBatch; ++k) {
-    const int dy = idx[k] >= 0 ? idx[k] / w : -1;
-#pragma unroll
-    for (int d = 0; d < kRowsMaxW; ++d) mine[d] += dy == d;
-  }
-  for (uint32_t q = rest; q; q &= q - 1) {
-    const int dy = ag[lane * 32 + __ffs(q) - 1] / w;
-#pragma unroll
-    for (int d = 0; d < kRowsMaxW; ++d) mine[d] += dy == d;
-  }
-  // place of this lane's first peak of each in-tile row: the row's peaks
-  // in lower in-tile rows, then the lower lanes' peaks of that row
-  int excl[kRowsMaxW];
-  int run = 0;
-#pragma unroll
-  for (int d = 0; d < kRowsMaxW; ++d) {
-    int incl = mine[d];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
+    for (int k = 0; k < kRowsBatch; ++k) {
+      idx[k] = -1;
+      tx[k] = 0;
+      v[k] = 0.f;
+      if (m) {
+        tx[k] = wx * 32 + __ffs(m) - 1;
+        m &= m - 1;
+        idx[k] = arg_of(tx[k]);
+        v[k] = vg[tx[k]];
+      }
     }
-    excl[d] = run + incl - mine[d];
-    run += __shfl_sync(0xffffffffu, incl, 31);
-  }
-  auto put = [&](int t, int i, float val) {
-    const int dy = i / w, dx = i - dy * w;
-    int j = 0;
+    const uint32_t rest = m;
+    int mine[MAXW];
 #pragma unroll
-    for (int d = 0; d < kRowsMaxW; ++d)
-      if (dy == d) j = excl[d]++;
-    const int64_t n = roff + j;   // place among the image candidates
-    const int64_t pos = base + n;
-    if (n < cap && pos < a.cap) a.out[pos] = image_candidate(a, SelItem{g, t0 + t, val}, t, ty, w, dx, dy);
-  };
+    for (int d = 0; d < MAXW; ++d) mine[d] = 0;
 #pragma unroll
-  for (int k = 0; k < kRowsBatch; ++k)
-    if (idx[k] >= 0) put(tx[k], idx[k], v[k]);
-  for (uint32_t q = rest; q; q &= q - 1) {
-    const int t = lane * 32 + __ffs(q) - 1;
-    put(t, ag[t], vg[t]);
+    for (int k = 0; k < kRowsBatch; ++k) {
+      const int dy = idx[k] >= 0 ? idx[k] / w : -1;
+#pragma unroll
+      for (int d = 0; d < MAXW; ++d) mine[d] += dy == d;
+    }
+    for (uint32_t q = rest; q; q &= q - 1) {
+      const int dy = arg_of(wx * 32 + __ffs(q) - 1) / w;
+#pragma unroll
+      for (int d = 0; d < MAXW; ++d) mine[d] += dy == d;
+    }
+    // place of this lane's first peak of each in-tile row: the row's peaks in
+    // lower in-tile rows, the earlier words' and the lower lanes' of that row
+    int excl[MAXW];
+    int run = 0;
+#pragma unroll
+    for (int d = 0; d < MAXW; ++d) {
+      excl[d] = 0;
+      int incl = mine[d];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const int tot = __shfl_sync(0xffffffffu, incl, 31);
+      if (WIDE) {
+        excl[d] = next[d] + incl - mine[d];
+        next[d] += tot;
+      } else {
+        excl[d] = run + incl - mine[d];
+        run += tot;
+      }
+    }
+    auto put = [&](int t, int i, float val) {
+      const int dy = i / w, dx = i - dy * w;
+      int j = 0;
+#pragma unroll
+      for (int d = 0; d < MAXW; ++d)
+        if (dy == d) j = excl[d]++;
+      const int64_t n = roff + j;   // place among the image candidates
+      const int64_t pos = base + n;
+      if (n < cap && pos < a.cap)
+        a.out[pos] = image_candidate(a, SelItem{g, t0 + t, val}, t, ty, w, dx, dy);
+    };
+#pragma unroll
+    for (int k = 0; k < kRowsBatch; ++k)
+      if (idx[k] >= 0) put(tx[k], idx[k], v[k]);
+    for (uint32_t q = rest; q; q &= q - 1) {
+      const int t = wx * 32 + __ffs(q) - 1;
+      put(t, arg_of(t), vg[t]);
+    }
+    if (!WIDE) break;
   }
 }
 
@@ -1594,12 +1692,21 @@ cudaError_t launch_emit_peaks(const CandArgs& a, const SelItem* peaks, const int
 
 cudaError_t launch_emit_rows(const CandArgs& a, const float* vals, int groups, const BlockScratch& b,
                              int64_t cap, int* base, cudaStream_t st) {
-  if (!a.arg || a.w < 1 || a.w > kRowsMaxW || b.words > 32 ||
+  if ((!a.arg && a.w != 1) || a.w < 1 || a.w > kRowsMaxW ||
       ((int64_t)groups * a.Ty + kRowsPerCta - 1) / kRowsPerCta > b.nblk)
     return cudaErrorInvalidValue;
   const int64_t nrows = (int64_t)groups * a.Ty;
-  cudaError_t e = launch_pdl(k_emit_rows, dim3((unsigned)((nrows * 32 + kPbThreads - 1) / kPbThreads)),
-                             dim3(kPbThreads), 0, st, a, vals, nrows, b, cap, (const int*)base);
+  const dim3 grid((unsigned)((nrows * 32 + kPbThreads - 1) / kPbThreads));
+  cudaError_t e;
+  if (a.w == 1)
+    e = launch_pdl(k_emit_rows<true, 1>, grid, dim3(kPbThreads), 0, st, a, vals, nrows, b, cap,
+                   (const int*)base);
+  else if (b.words > 32)
+    e = launch_pdl(k_emit_rows<true, kRowsMaxW>, grid, dim3(kPbThreads), 0, st, a, vals, nrows, b,
+                   cap, (const int*)base);
+  else
+    e = launch_pdl(k_emit_rows<false, kRowsMaxW>, grid, dim3(kPbThreads), 0, st, a, vals, nrows, b,
+                   cap, (const int*)base);
   if (e == cudaSuccess)
     e = launch_pdl(k_add_count, dim3(1), dim3(1), 0, st, a.nout, (const int*)&b.counters[2]);
   count_launches(2);

@@ -1007,10 +1007,10 @@ static cudaError_t enqueue_post(fitrig_plan_t p, cudaStream_t st, bool timed) {
   // statistics, so they run on the side stream beside the spectrum and the
   // frequency branch; the two join before the image candidates are written
   // (frequency candidates, snapshot -1, lead the sorted list).
-  // with the march's in-tile arg-max, a small window and tile rows of at most
-  // 1024 tiles the image candidates come straight from the peak bitmap,
+  // with the march's in-tile arg-max and a small window, or with 1 x 1 tiles
+  // (sliding mode), the image candidates come straight from the peak bitmap,
   // already in (snapshot, y, x) order
-  const bool rows_emit = image && p->d_arg && ca.w <= 8 && p->Tx <= 1024;
+  const bool rows_emit = image && ((p->d_arg && ca.w <= 8) || ca.w == 1);
   // Maps too large for the plan's own split scratch borrow the candidates'
   // second buffer, which nothing uses before the image candidates are formed
   // (after the branches join): the automatic capacity of 4 Mi + tiles / 12
