@@ -495,20 +495,210 @@ __global__ void __launch_bounds__(kLongWarps * 32) k_dft_long(const float* __res
   warp_spectrum_best(mk, K, hmax, lane, eta + t, bin + t);
 }
 
+// Composite lengths of the long path: one step of Cooley and Tukey's splitting
+// (Math. Comp. 19, 1965) with n = P M, X_q = sum_p W_n^(p q) S_p[q mod M], S_p
+// the length-M DFT of y_p, y_(p+P), ..  The sub-series are real, so S_p[M - k]
+// is the conjugate of S_p[k] and only k <= M/2 is summed, from folded pairs as
+// in the direct kernels; a lane holds two bins of kMixP sub-series, so one
+// table entry feeds 4 kMixP multiply-adds and one pair of broadcast loads four.
+// n = 1498 = 14 x 107: about 9 k instructions per tile and warp against the
+// direct kernel's 116 k; every twiddle is a table entry (the direct kernel
+// advances a phasor), so the rounding error is smaller too.  4096 series of
+// 1498 points, harmonic sums to 8: 988 -> 138 us; 16,384 of 300 / 1001 / 4095:
+// 208 / 1298 / 38383 -> 70 / 218 / 4121 us; 998 = 2 x 499: 1300 -> 1056.  Bound by
+// the shared-memory loads of the pairs and table entries.  One warp per tile;
+// the table (full circle) and the WARPS tiles' series and sub-spectra are in
+// shared memory.
+constexpr int kMixP = 8;
+constexpr int kMixK = 2;
+
+__host__ __device__ constexpr int mixed_lds(int n, int P) { return P * (n / P / 2 + 1); }
+
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32) k_dft_mixed(const float* __restrict__ vp, int n, int P,
+                                                          int64_t T, int64_t vs,
+                                                          const float2* __restrict__ tw,
+                                                          const float* __restrict__ wts, int hmax,
+                                                          float* eta, int* bin) {
+  extern __shared__ float2 msm[];
+  const int K = n / 2, H = (n - 1) / 2, M = n / P, MB = M / 2 + 1, HM = (M - 1) / 2;
+  const int ldy = long_ldy(n), lds = mixed_lds(n, P);
+  float2* tb = msm;                                           // [n] (cos, sin)(2 pi a / n)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float2* S = tb + n + warp * lds;                            // [P][MB]
+  float* ys = reinterpret_cast<float*>(tb + n + WARPS * lds);   // [WARPS][ldy]
+  const int64_t t0 = (int64_t)blockIdx.x * WARPS;
+  for (int i = threadIdx.x; i < n * WARPS; i += WARPS * 32) {
+    const int q = i / WARPS, c = i - q * WARPS;
+    const int64_t t = t0 + c;
+    float v = t < T ? vp[(size_t)q * vs + t] : 0.f;
+    if (wts) v *= wts[q];
+    ys[c * ldy + q] = v;
+  }
+  for (int a = threadIdx.x; a < n; a += WARPS * 32) {
+    float2 e;
+    if (a == 0) e = make_float2(1.f, 0.f);
+    else if (2 * a == n) e = make_float2(-1.f, 0.f);
+    else if (a <= H) e = tw[a - 1];
+    else {
+      e = tw[n - a - 1];
+      e.y = -e.y;
+    }
+    tb[a] = e;
+  }
+  __syncthreads();
+  const int64_t t = t0 + warp;
+  if (t >= T) return;
+  float* y = ys + warp * ldy;
+  float sum = 0.f;
+  bool ok = true;
+  for (int q = lane; q < n; q += 32) {
+    const float v = y[q];
+    ok = ok && isfinite(v);
+    sum += v;
+  }
+  ok = __all_sync(0xffffffffu, ok);
+#pragma unroll
+  for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  if (!ok) {
+    if (lane == 0) {
+      eta[t] = NAN;
+      bin[t] = -1;
+    }
+    return;
+  }
+  const float mean = sum / (float)n;
+  const bool even = (M & 1) == 0;
+  __syncwarp();
+  // the folded pairs of every sub-series: y_(p + P j), j = 1..HM, lie at i + P
+  for (int i = lane; i < P * HM; i += 32) {
+    const int p = i % P, hi = p + P * (M - 1 - i / P);
+    const float a = y[i + P] - mean, b = y[hi] - mean;
+    y[i + P] = a + b;   // e
+    y[hi] = a - b;      // o
+  }
+  for (int p = lane; p < P; p += 32) {
+    y[p] -= mean;
+    if (even) y[p + P * (M / 2)] -= mean;
+  }
+  __syncwarp();
+  for (int kb = 0; kb < MB; kb += 32 * kMixK) {
+    int kk[kMixK];
+#pragma unroll
+    for (int b = 0; b < kMixK; ++b) kk[b] = min(kb + lane + 32 * b, MB - 1);
+    for (int p0 = 0; p0 < P; p0 += kMixP) {
+      float re[kMixK][kMixP], im[kMixK][kMixP];
+#pragma unroll
+      for (int i = 0; i < kMixP; ++i) {
+        const int p = min(p0 + i, P - 1);
+        const float y0 = y[p], ym = even ? y[p + P * (M / 2)] : 0.f;
+#pragma unroll
+        for (int b = 0; b < kMixK; ++b) {
+          re[b][i] = y0 + ((kk[b] & 1) ? -ym : ym);
+          im[b][i] = 0.f;
+        }
+      }
+      int a[kMixK];
+#pragma unroll
+      for (int b = 0; b < kMixK; ++b) a[b] = 0;
+      const float* ye = y + p0;
+      const float* yo = y + p0 + P * M;
+      for (int j = 1; j <= HM; ++j) {
+        ye += P;
+        yo -= P;
+        float2 c[kMixK];
+#pragma unroll
+        for (int b = 0; b < kMixK; ++b) {
+          a[b] += kk[b];
+          if (a[b] >= M) a[b] -= M;
+          c[b] = tb[a[b] * P];
+        }
+#pragma unroll
+        for (int i = 0; i < kMixP; ++i) {
+          if (p0 + i >= P) break;   // (uniform)
+          const float e = ye[i], o = yo[i];
+#pragma unroll
+          for (int b = 0; b < kMixK; ++b) {
+            re[b][i] = fmaf(e, c[b].x, re[b][i]);
+            im[b][i] = fmaf(o, c[b].y, im[b][i]);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kMixP; ++i)
+        if (p0 + i < P) {
+#pragma unroll
+          for (int b = 0; b < kMixK; ++b)
+            if (kb + lane + 32 * b < MB) S[(p0 + i) * MB + kk[b]] = make_float2(re[b][i], -im[b][i]);
+        }
+    }
+  }
+  __syncwarp();
+  float* mk = y;   // the series is spent: |X_q|^2 at mk[q]
+  for (int q = 1 + lane; q <= K; q += 32) {
+    int k = q % M;
+    const bool mirror = k >= MB;
+    if (mirror) k = M - k;
+    const float sg = mirror ? -1.f : 1.f;   // conjugate of S_p[M - k]
+    float2 x = S[k];
+    x.y *= sg;
+    int a = 0;
+    for (int p = 1; p < P; ++p) {
+      a += q;
+      if (a >= n) a -= n;
+      const float2 w = tb[a];
+      float2 v = S[p * MB + k];
+      v.y *= sg;
+      x.x = fmaf(w.x, v.x, fmaf(w.y, v.y, x.x));
+      x.y = fmaf(w.x, v.y, fmaf(-w.y, v.x, x.y));
+    }
+    mk[q] = x.x * x.x + x.y * x.y;
+  }
+  __syncwarp();
+  warp_spectrum_best(mk, K, hmax, lane, eta + t, bin + t);
+}
+
+// The divisor P of n whose splitting costs least, in instructions per warp
+// and tile, or 0 when the direct kernel (six multiply-adds and two loads per
+// pair and four bins) costs less: primes, and twice a prime below about 70.
+static int mixed_split(int n) {
+  const int K = n / 2, H = (n - 1) / 2;
+  int best = 0;
+  int64_t cost = (int64_t)((K + 32 * kLongB - 1) / (32 * kLongB)) * H * (6 * kLongB + 2) * 4 / 5;
+  for (int P = 2; P <= n / 3; ++P) {
+    if (n % P) continue;
+    const int M = n / P, MB = M / 2 + 1;
+    const int64_t sub = (int64_t)((MB + 32 * kMixK - 1) / (32 * kMixK)) * (M / 2) *
+                        ((P + kMixP - 1) / kMixP * 5 * kMixK + P * (2 + 2 * kMixK));
+    const int64_t c = sub + (int64_t)((K + 31) / 32) * P * 10 + n / 2;
+    if (c < cost) {
+      cost = c;
+      best = P;
+    }
+  }
+  return best;
+}
+
 // Powers of two, kFftMinN <= n <= kLongMaxN: a radix FFT per tile instead of
 // the O(n^2) direct sum.  One warp per tile; a CTA stages the series of
 // TILES consecutive tiles by asynchronous global -> shared copies (each cube
 // row a TILES x 4-byte segment).  The real series y_0..y_(n-1), mean removed,
 // is read as the complex series z_j = y_(2j) + i y_(2j+1) of N = n/2 points
 // (the staging buffer already holds it in that order), transformed by a
-// Stockham autosort FFT (radix-4 passes, one radix-2 pass when log2 N is odd)
-// that alternates between the staging buffer and a second warp buffer, and
-// the real spectrum is recovered as
+// Stockham autosort FFT (radix-8 passes, one radix-4 or radix-2 pass for the
+// rest of log2 N) that alternates between the staging buffer and a second warp
+// buffer, and the real spectrum is recovered as
 //   X_k = (Z_k + conj Z_(N-k)) / 2 - (i/2) e^(-2 pi i k/n) (Z_k - conj Z_(N-k)),
 //   X_(n/2) = Re Z_0 - Im Z_0,
 // whose squared magnitudes feed the same maximum / harmonic-sum reduction as
 // the direct kernels.  Every twiddle is an entry of the host's FP64 table of
 // (cos, sin)(2 pi a / n), a = 0..n-1, rounded once to FP32.
+// Bound by shared memory: what counts is the number of passes (three instead
+// of five at n = 1024) and bank conflicts.  Both buffers leave one entry in
+// nine unused, so that a radix-8 pass's stores, eight entries apart, meet
+// none, and the tiles' buffers are shifted against each other for the loads.
+// 16,384 series of 512 / 1024 / 2048 / 4096 points: 57 / 118 / 257 / 712 us with
+// radix-4 passes and neither, 43 / 81 / 237 / 613 now.
 constexpr int kFftMinN = 128;
 
 __host__ __device__ constexpr bool fft_length(int n) {
@@ -519,6 +709,69 @@ __device__ __forceinline__ float2 cmul_conj(float2 a, float2 w) {   // a * conj(
   return make_float2(fmaf(a.x, w.x, a.y * w.y), fmaf(a.y, w.x, -a.x * w.y));
 }
 
+__host__ __device__ constexpr int fft_at(int i) { return i + (i >> 3); }   // place of entry i
+__host__ __device__ constexpr int fft_buf(int N) { return N + N / 8; }
+// Entries of a tile's two buffers, with a shift of 32 / tiles words between
+// tiles: a load instruction writes 32 / tiles points of every tile of the CTA.
+__host__ __device__ constexpr int fft_tile(int N, int tiles) { return 2 * fft_buf(N) + 16 / tiles; }
+
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 mul_mi(float2 a) { return make_float2(a.y, -a.x); }   // -i a
+
+// Forward DFTs of R points in registers.
+template <int R>
+__device__ __forceinline__ void dft_r(float2 (&a)[R]) {
+  if constexpr (R == 2) {
+    const float2 t = a[0];
+    a[0] = cadd(t, a[1]);
+    a[1] = csub(t, a[1]);
+  } else if constexpr (R == 4) {
+    const float2 b0 = cadd(a[0], a[2]), b1 = csub(a[0], a[2]);
+    const float2 b2 = cadd(a[1], a[3]), b3 = mul_mi(csub(a[1], a[3]));
+    a[0] = cadd(b0, b2);
+    a[1] = cadd(b1, b3);
+    a[2] = csub(b0, b2);
+    a[3] = csub(b1, b3);
+  } else {
+    static_assert(R == 8, "radix");
+    float2 e[4] = {a[0], a[2], a[4], a[6]}, o[4] = {a[1], a[3], a[5], a[7]};
+    dft_r<4>(e);
+    dft_r<4>(o);
+    constexpr float h = 0.70710678118654752f;   // W_8 = (1 - i) / sqrt 2
+    o[1] = make_float2(h * (o[1].x + o[1].y), h * (o[1].y - o[1].x));
+    o[2] = mul_mi(o[2]);
+    o[3] = make_float2(h * (o[3].y - o[3].x), -h * (o[3].x + o[3].y));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      a[k] = cadd(e[k], o[k]);
+      a[k + 4] = csub(e[k], o[k]);
+    }
+  }
+}
+
+// One Stockham pass of radix R over the warp's N points (Ns points done).
+template <int R, bool FIRST>
+__device__ __forceinline__ void fft_pass(const float2* src, float2* dst, int N, int Ns, int n,
+                                         float mean, const float2* __restrict__ fw, int lane) {
+  const int Q = N / R, step = n / (R * Ns);
+  for (int j = lane; j < Q; j += 32) {
+    const int k = j & (Ns - 1);
+    float2 a[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      a[r] = src[fft_at(j + r * Q)];
+      if (FIRST) a[r] = make_float2(a[r].x - mean, a[r].y - mean);   // (all twiddles are 1)
+      else if (r > 0) a[r] = cmul_conj(a[r], __ldg(fw + r * k * step));   // W_(R Ns)^(r k)
+    }
+    dft_r<R>(a);
+    const int base = (j - k) * R + k;
+#pragma unroll
+    for (int r = 0; r < R; ++r) dst[fft_at(base + r * Ns)] = a[r];
+  }
+  __syncwarp();
+}
+
 template <int TILES>
 __global__ void __launch_bounds__(TILES * 32) k_fft_pow2(const float* __restrict__ vp, int n,
                                                          int logN, int64_t T, int64_t vs,
@@ -526,12 +779,13 @@ __global__ void __launch_bounds__(TILES * 32) k_fft_pow2(const float* __restrict
                                                          const float* __restrict__ wts, int hmax,
                                                          float* eta, int* bin) {
   extern __shared__ float2 fsm[];
-  const int N = n >> 1;
+  const int N = n >> 1, NB = fft_buf(N);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t0 = (int64_t)blockIdx.x * TILES;
+  auto at = [](int q) { return 2 * fft_at(q >> 1) + (q & 1); };   // series point q as a float
   for (int i = threadIdx.x; i < n * TILES; i += TILES * 32) {
     const int q = i / TILES, c = i - q * TILES;
-    float* dst = reinterpret_cast<float*>(fsm + (size_t)c * 2 * N) + q;
+    float* dst = reinterpret_cast<float*>(fsm + (size_t)c * fft_tile(N, TILES)) + at(q);
     if (t0 + c < T) {
       asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)),
                    "l"(vp + (size_t)q * vs + t0 + c)
@@ -544,16 +798,16 @@ __global__ void __launch_bounds__(TILES * 32) k_fft_pow2(const float* __restrict
   __syncthreads();
   const int64_t t = t0 + warp;
   if (t >= T) return;
-  float2* src = fsm + (size_t)warp * 2 * N;   // z_j = (y_2j, y_2j+1)
-  float2* dst = src + N;
+  float2* src = fsm + (size_t)warp * fft_tile(N, TILES);   // z_j = (y_2j, y_2j+1)
+  float2* dst = src + NB;
   float* y = reinterpret_cast<float*>(src);
   float sum = 0.f;
   bool ok = true;
   for (int q = lane; q < n; q += 32) {
-    float v = y[q];
+    float v = y[at(q)];
     if (wts) {
       v *= wts[q];
-      y[q] = v;
+      y[at(q)] = v;
     }
     ok = ok && isfinite(v);
     sum += v;
@@ -569,45 +823,30 @@ __global__ void __launch_bounds__(TILES * 32) k_fft_pow2(const float* __restrict
     return;
   }
   const float mean = sum / (float)n;
-  for (int q = lane; q < n; q += 32) y[q] -= mean;
   __syncwarp();
-  int Ns = 1;
-  for (int pass = 0; pass < (logN >> 1); ++pass) {
-    const int Q = N >> 2, step = n / (4 * Ns);
-    for (int j = lane; j < Q; j += 32) {
-      const int k = j & (Ns - 1);
-      const int e = k * step;   // W_(4 Ns)^(r k) = W_n^(r e), r e < 3n/4
-      const float2 a0 = src[j];
-      const float2 a1 = cmul_conj(src[j + Q], __ldg(fw + e));
-      const float2 a2 = cmul_conj(src[j + 2 * Q], __ldg(fw + 2 * e));
-      const float2 a3 = cmul_conj(src[j + 3 * Q], __ldg(fw + 3 * e));
-      const float2 b0 = make_float2(a0.x + a2.x, a0.y + a2.y);
-      const float2 b1 = make_float2(a0.x - a2.x, a0.y - a2.y);
-      const float2 b2 = make_float2(a1.x + a3.x, a1.y + a3.y);
-      const float2 b3 = make_float2(a1.y - a3.y, a3.x - a1.x);   // -i (a1 - a3)
-      const int base = ((j - k) << 2) + k;
-      dst[base] = make_float2(b0.x + b2.x, b0.y + b2.y);
-      dst[base + Ns] = make_float2(b1.x + b3.x, b1.y + b3.y);
-      dst[base + 2 * Ns] = make_float2(b0.x - b2.x, b0.y - b2.y);
-      dst[base + 3 * Ns] = make_float2(b1.x - b3.x, b1.y - b3.y);
-    }
-    __syncwarp();
+  auto swap = [&]() {
     float2* tmp = src;
     src = dst;
     dst = tmp;
-    Ns <<= 2;
-  }
-  if (logN & 1) {   // last pass radix 2: Ns = N / 2, twiddle W_N^j = W_n^(2j)
-    for (int j = lane; j < Ns; j += 32) {
-      const float2 a0 = src[j];
-      const float2 a1 = cmul_conj(src[j + Ns], __ldg(fw + 2 * j));
-      dst[j] = make_float2(a0.x + a1.x, a0.y + a1.y);
-      dst[j + Ns] = make_float2(a0.x - a1.x, a0.y - a1.y);
+  };
+  fft_pass<8, true>(src, dst, N, 1, n, mean, fw, lane);   // N >= 64
+  swap();
+  int Ns = 8;
+  for (int left = logN - 3; left > 0;) {
+    if (left >= 3) {
+      fft_pass<8, false>(src, dst, N, Ns, n, 0.f, fw, lane);
+      Ns <<= 3;
+      left -= 3;
+    } else if (left == 2) {
+      fft_pass<4, false>(src, dst, N, Ns, n, 0.f, fw, lane);
+      Ns <<= 2;
+      left = 0;
+    } else {
+      fft_pass<2, false>(src, dst, N, Ns, n, 0.f, fw, lane);
+      Ns <<= 1;
+      left = 0;
     }
-    __syncwarp();
-    float2* tmp = src;
-    src = dst;
-    dst = tmp;
+    swap();
   }
   float* mk = reinterpret_cast<float*>(dst);   // |X_k|^2 at mk[k], k = 1..N
   for (int k = 1 + lane; k <= N; k += 32) {
@@ -617,7 +856,7 @@ __global__ void __launch_bounds__(TILES * 32) k_fft_pow2(const float* __restrict
       const float x = z0.x - z0.y;
       m2 = x * x;
     } else {
-      const float2 zk = src[k], zc = src[N - k];
+      const float2 zk = src[fft_at(k)], zc = src[fft_at(N - k)];
       const float er = 0.5f * (zk.x + zc.x), ei = 0.5f * (zk.y - zc.y);
       const float orr = 0.5f * (zk.y + zc.y), oi = 0.5f * (zc.x - zk.x);
       const float2 w = __ldg(fw + k);   // (cos, sin)(2 pi k / n); forward uses conj
@@ -677,11 +916,31 @@ static cudaError_t launch_long(const float* vp, int n, int64_t T, int64_t vs,
   return cudaGetLastError();
 }
 
+template <int WARPS>
+static cudaError_t launch_mixed_t(const float* vp, int n, int P, int64_t T, int64_t vs,
+                                  const float2* tw, const float* wts, int hmax, float* eta,
+                                  int* bin, cudaStream_t st) {
+  const size_t sm = sizeof(float2) * ((size_t)n + (size_t)WARPS * mixed_lds(n, P)) +
+                    sizeof(float) * (size_t)WARPS * long_ldy(n);
+  static size_t configured = 0;
+  if (sm > 48 * 1024 && sm > configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_dft_mixed<WARPS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    configured = sm;
+  }
+  const int64_t blocks = (T + WARPS - 1) / WARPS;
+  k_dft_mixed<WARPS><<<(unsigned)blocks, WARPS * 32, sm, st>>>(vp, n, P, T, vs, tw, wts, hmax, eta,
+                                                              bin);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
 template <int TILES>
 static cudaError_t launch_fft_t(const float* vp, int n, int64_t T, int64_t vs, const float2* fw,
                                 const float* wts, int hmax, float* eta, int* bin,
                                 cudaStream_t st) {
-  const size_t sm = (size_t)TILES * n * sizeof(float2);   // two N-point buffers per tile
+  const size_t sm = (size_t)TILES * fft_tile(n / 2, TILES) * sizeof(float2);
   static size_t configured = 0;
   if (sm > 48 * 1024 && sm > configured) {
     cudaError_t e = cudaFuncSetAttribute(k_fft_pow2<TILES>,
@@ -698,6 +957,10 @@ static cudaError_t launch_fft_t(const float* vp, int n, int64_t T, int64_t vs, c
   return cudaGetLastError();
 }
 
+static cudaError_t launch_odd_length(const float* vp, int n, int64_t T, int64_t vs,
+                                     const float2* twiddle, const float* wts, int hmax, float* eta,
+                                     int* bin, bool direct, cudaStream_t st);
+
 cudaError_t launch_spectrum_method(const float* vp, int n, int64_t T, int64_t vs,
                                    const float2* twiddle, const float* wts, int hmax, float* eta,
                                    int* bin, int method, cudaStream_t st) {
@@ -710,18 +973,21 @@ cudaError_t launch_spectrum_method(const float* vp, int n, int64_t T, int64_t vs
                              : launch_fft_t<4>(vp, n, T, vs, twiddle, wts, hmax, eta, bin, st);
   }
   if (method == kSpectrumRadix) return cudaErrorInvalidValue;
-  return launch_spectrum(vp, n, T, vs, twiddle, wts, hmax, eta, bin, st);
+  return launch_odd_length(vp, n, T, vs, twiddle, wts, hmax, eta, bin, method == kSpectrumDirect, st);
 }
 
 cudaError_t launch_spectrum(const float* vp, int n, int64_t T, int64_t vs,
                             const float2* twiddle, const float* wts, int hmax, float* eta,
                             int* bin, cudaStream_t st) {
+  return launch_spectrum_method(vp, n, T, vs, twiddle, wts, hmax, eta, bin, kSpectrumAuto, st);
+}
+
+// Every length that is not the radix kernel's; `direct`: without the splitting.
+static cudaError_t launch_odd_length(const float* vp, int n, int64_t T, int64_t vs,
+                                     const float2* twiddle, const float* wts, int hmax, float* eta,
+                                     int* bin, bool direct, cudaStream_t st) {
   const int64_t blocks = (T + kDftThreads - 1) / kDftThreads;
   const int H = (n - 1) / 2, K = n / 2;
-  if (n < 2 || n > kLongMaxN || hmax < 1) return cudaErrorInvalidValue;
-  if (T == 0) return cudaSuccess;
-  if (fft_length(n))
-    return launch_spectrum_method(vp, n, T, vs, twiddle, wts, hmax, eta, bin, kSpectrumAuto, st);
   const bool harm = hmax > 1;
   if ((n & 1) == 0 && n <= 66) {
     const int m = n / 2, Hm = (m - 1) / 2, Kh = m / 2;
@@ -740,7 +1006,15 @@ cudaError_t launch_spectrum(const float* vp, int n, int64_t T, int64_t vs,
     count_launches(1);
     return cudaGetLastError();
   }
-  if (n > 256 || hmax > 1) return launch_long(vp, n, T, vs, twiddle, wts, hmax, eta, bin, st);
+  if (n > 256 || hmax > 1) {
+    const int P = direct ? 0 : mixed_split(n);
+    // eight tiles per CTA fill 32-byte segments of the cube's rows; four where
+    // eight tiles' series, sub-spectra and the table exceed half an SM's memory
+    if (P && n <= 1664)
+      return launch_mixed_t<8>(vp, n, P, T, vs, twiddle, wts, hmax, eta, bin, st);
+    if (P) return launch_mixed_t<4>(vp, n, P, T, vs, twiddle, wts, hmax, eta, bin, st);
+    return launch_long(vp, n, T, vs, twiddle, wts, hmax, eta, bin, st);
+  }
   const size_t smem = (size_t)n * kDftThreads * sizeof(float);
   static size_t configured = 0;
   if (smem > 48 * 1024 && smem > configured) {

@@ -1458,11 +1458,8 @@ FITRIG_API int fitrig_spectrum_map(const float* dev_cube, int32_t n, int64_t T, 
   if (e == cudaSuccess) {
     const int m = method == FITRIG_SPECTRUM_DIRECT ? kSpectrumDirect
                   : method == FITRIG_SPECTRUM_RADIX ? kSpectrumRadix : kSpectrumAuto;
-    if (method == FITRIG_SPECTRUM_DIRECT && !pow2)   // the table is already the direct kernels'
-      e = launch_spectrum(dev_cube, n, T, stride, d_tw, nullptr, harmonics, dev_eta, dev_bin, st);
-    else
-      e = launch_spectrum_method(dev_cube, n, T, stride, d_tw, nullptr, harmonics, dev_eta,
-                                 dev_bin, m, st);
+    e = launch_spectrum_method(dev_cube, n, T, stride, d_tw, nullptr, harmonics, dev_eta, dev_bin,
+                               m, st);
   }
   if (e == cudaSuccess) e = cudaEventRecord(e1, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
