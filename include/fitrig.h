@@ -236,6 +236,9 @@ FITRIG_API int fitrig_plan_set(fitrig_plan_t plan, int option, int64_t value);
  * copied in four row bands on internal side streams (ordered after the work
  * already on the plan's stream; the plan's stream waits for them), so that
  * several copy engines share the transfer; pinned host memory is fastest.
+ * Contiguous host rows that do not fill the device pitch (a row is not a
+ * multiple of 128 bytes) go through a 32 MB device buffer of the plan, from
+ * 4 MB on, allocated at the first such push (without it if there is no room).
  */
 FITRIG_API int fitrig_push_snapshot(fitrig_plan_t plan, const void* data, int dtype,
                                     int on_device, int64_t row_pitch_elems);
@@ -246,10 +249,8 @@ FITRIG_API int fitrig_push_snapshot(fitrig_plan_t plan, const void* data, int dt
  * `snap_stride_elems` elements after snapshot i-1 (0 means row_pitch * ny) and
  * holds ny rows of `row_pitch_elems` elements (0 means nx).  A host buffer is
  * borrowed until the call returns (one synchronisation at the end, not one per
- * snapshot).  When the host snapshots are contiguous rows of the storage type
- * and the plan's rows are unpadded (nx * element size a multiple of 128 bytes),
- * the block goes as one transfer split into four row bands on the side
- * streams.  With FITRIG_OPT_ACCUMULATE = K they are raw snapshots (K per slot).
+ * snapshot).  When the snapshots follow each other without a gap in the storage
+ * type, the block goes as one transfer of count * ny rows.  With FITRIG_OPT_ACCUMULATE = K they are raw snapshots (K per slot).
  * EINVAL for count < 0 or a stride shorter than one snapshot; ESTATE (nothing
  * pushed) when they do not fit into the remaining slots.
  */

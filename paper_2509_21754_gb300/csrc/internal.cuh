@@ -447,6 +447,10 @@ cudaError_t launch_spectrum_method(const float* vp, int n, int64_t T, int64_t vs
 // Ingest conversion (fp32 <-> bf16/fp16).
 cudaError_t launch_convert(const void* src, int src_type, int64_t src_pitch, void* dst,
                            int dst_type, int64_t dst_pitch, int ny, int nx, cudaStream_t st);
+// `rows` rows of `width` bytes (a multiple of 2), spitch bytes apart in device
+// memory, to dst, dpitch bytes apart.
+cudaError_t launch_repitch(const void* src, size_t spitch, void* dst, size_t dpitch, size_t width,
+                           int64_t rows, cudaStream_t st);
 // Difference coding of one pushed snapshot (FITRIG_CODING_DELTA): with
 // `first` the snapshot goes to the FP32 key frame (pitch key_pitch) and to the
 // coder's running decoded snapshot `state` (ny x nx dense); otherwise

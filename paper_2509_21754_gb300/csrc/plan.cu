@@ -49,6 +49,86 @@ int elem_bytes(int t) { return t == FITRIG_F32 ? 4 : 2; }
 
 std::atomic<long long> g_launches{0};
 
+// Host-to-device copies of rows that do not fill the device pitch.  The copy
+// engines move such rows at half the link's rate (6200-byte rows: 102 GB/s
+// however many streams share them, against 210 GB/s for one linear copy), so
+// contiguous host rows go to a ring of staging slots as linear copies on two
+// streams of their own, and a kernel on the caller's stream sets them at their
+// pitch while the next slot is filled: 20 snapshots of 2600 x 3100 BF16 from
+// pinned memory with the detect 3.65 -> 2.27 ms.
+struct Ingest {
+  static constexpr int kSlots = 4;
+  static constexpr size_t kSlot = (size_t)8 << 20;   // 40 us of copying each
+  static constexpr size_t kLeast = (size_t)4 << 20;  // below, the launches cost what is gained
+  char* buf = nullptr;
+  cudaStream_t cs[2] = {};   // alternate, so that one's copy covers the other's wait and launch
+  cudaEvent_t start = nullptr, full[kSlots] = {}, freed[kSlots] = {};
+  int next = 0;
+  bool failed = false;   // no memory for it: such copies stay pitched ones
+
+  bool ready() {
+    if (buf) return true;
+    if (failed) return false;
+    bool ok = cudaMalloc(&buf, kSlots * kSlot) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&cs[0], cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&cs[1], cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&start, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; ok && i < kSlots; ++i)
+      ok = cudaEventCreateWithFlags(&full[i], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&freed[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+      (void)cudaGetLastError();
+      release();
+      failed = true;
+    }
+    return ok;
+  }
+
+  void release() {
+    for (cudaStream_t c : cs)
+      if (c) cudaStreamSynchronize(c);
+    if (buf) cudaFree(buf);
+    for (cudaStream_t c : cs)
+      if (c) cudaStreamDestroy(c);
+    if (start) cudaEventDestroy(start);
+    for (int i = 0; i < kSlots; ++i) {
+      if (full[i]) cudaEventDestroy(full[i]);
+      if (freed[i]) cudaEventDestroy(freed[i]);
+      full[i] = freed[i] = nullptr;
+    }
+    buf = nullptr;
+    cs[0] = cs[1] = nullptr;
+    start = nullptr;
+  }
+
+  static bool suits(size_t dpitch, size_t spitch, size_t width, size_t bytes) {
+    return spitch == width && dpitch != width && width <= kSlot && bytes >= kLeast;
+  }
+
+  // `rows` contiguous host rows to dst (pitch dpitch), ordered on st: the
+  // copies start after the work already on st, and st waits for them.
+  cudaError_t rows(char* dst, size_t dpitch, const char* src, size_t width, int64_t rows,
+                   cudaStream_t st) {
+    cudaError_t e = cudaEventRecord(start, st);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(cs[i], start, 0);
+    const int64_t per = (int64_t)(kSlot / width);
+    for (int64_t r = 0; r < rows && e == cudaSuccess; r += per) {
+      const int64_t n = std::min(per, rows - r);
+      char* slot = buf + (size_t)next * kSlot;
+      const cudaStream_t c = cs[next & 1];
+      e = cudaStreamWaitEvent(c, freed[next], 0);   // (a slot never used yet: no wait)
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(slot, src + (size_t)r * width, width * (size_t)n, cudaMemcpyHostToDevice, c);
+      if (e == cudaSuccess) e = cudaEventRecord(full[next], c);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(st, full[next], 0);
+      if (e == cudaSuccess) e = launch_repitch(slot, width, dst + (size_t)r * dpitch, dpitch, width, n, st);
+      if (e == cudaSuccess) e = cudaEventRecord(freed[next], st);
+      next = (next + 1) % kSlots;
+    }
+    return e;
+  }
+};
+
 }  // namespace
 
 void fitrig::count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
@@ -149,6 +229,7 @@ struct fitrig_plan_s {
   // host-to-device pushes are split over these streams (several copy engines)
   cudaStream_t copy_st[4] = {};
   cudaEvent_t copy_ev[5] = {};
+  Ingest ingest;   // rows that do not fill the pitch (allocated at their first push)
   // a detect repeated on the same state replays a captured graph of its
   // stream work (see fitrig_detect); the state is (pushed, zrot, generation
   // of the selection lists)
@@ -715,6 +796,8 @@ static cudaError_t copy_rows_h2d(fitrig_plan_t p, void* dst, size_t dpitch, cons
                                  size_t spitch, size_t width, int64_t ny, cudaStream_t st) {
   const size_t bytes = width * (size_t)ny;
   const bool linear = dpitch == width && spitch == width;
+  if (Ingest::suits(dpitch, spitch, width, bytes) && p->ingest.ready())
+    return p->ingest.rows(static_cast<char*>(dst), dpitch, static_cast<const char*>(src), width, ny, st);
   int nb = bytes >= ((size_t)32 << 20) ? 4 : 1;
   if (nb > 1 && !p->copy_st[0]) {
     for (int i = 0; i < 4; ++i) {
@@ -806,8 +889,7 @@ static int push_one(fitrig_plan_t p, const void* data, int dtype, int on_device,
   }
   if (dtype == p->storage) {
     if (on_device)
-      CK(cudaMemcpy2DAsync(dst, p->pitch * eb, data, rp * ib, (size_t)p->nx * ib, p->ny,
-                           cudaMemcpyDeviceToDevice, st));
+      CK(launch_repitch(data, rp * ib, dst, p->pitch * eb, (size_t)p->nx * ib, p->ny, st));
     else
       CK(copy_rows_h2d(p, dst, (size_t)p->pitch * eb, data, (size_t)rp * ib, (size_t)p->nx * ib,
                        p->ny, st));
@@ -868,15 +950,21 @@ FITRIG_API int fitrig_push_snapshots(fitrig_plan_t p, const void* data, int32_t 
   if (rc != FITRIG_OK) return rc;
   cudaStream_t st = plan_stream(p);
   const int eb = elem_bytes(p->storage);
-  // (a difference-coded plan takes its first snapshot as the key frame)
-  const bool contiguous = !on_device && k == 1 && dtype == p->storage && rp == p->nx &&
-                          p->pitch == p->nx && ss == rp * p->ny &&
-                          !(p->coding == FITRIG_CODING_DELTA && p->pushed == 0);
-  if (contiguous) {
-    // host rows and device slots line up: one transfer of count * ny rows
+  // Snapshots one after another, of the storage type: the slots' rows follow
+  // each other at the pitch too, so the block is one copy of count * ny rows
+  // (a difference-coded plan takes its first snapshot as the key frame).
+  const bool one_copy = k == 1 && dtype == p->storage && ss == rp * p->ny &&
+                        !(p->coding == FITRIG_CODING_DELTA && p->pushed == 0);
+  if (one_copy) {
     char* dst = p->d_stack + p->slice_bytes * p->pushed;
-    const size_t row = (size_t)p->nx * eb;
-    CK(copy_rows_h2d(p, dst, row, data, row, row, (int64_t)count * p->ny, st));
+    const size_t row = (size_t)p->nx * eb, dp = (size_t)p->pitch * eb, sp = (size_t)rp * eb;
+    const int64_t rows = (int64_t)count * p->ny;
+    if (!on_device)
+      CK(copy_rows_h2d(p, dst, dp, data, sp, row, rows, st));
+    else if (dp == row && sp == row)
+      CK(cudaMemcpyAsync(dst, data, row * (size_t)rows, cudaMemcpyDeviceToDevice, st));
+    else
+      CK(launch_repitch(data, sp, dst, dp, row, rows, st));
     p->pushed += count;
     p->detected = false;
     if (p->coding == FITRIG_CODING_DELTA) p->dstate_stale = true;
@@ -1780,6 +1868,8 @@ struct fitrig_server_s {
   std::vector<ServerField*> fields;   // index = field id
   std::deque<int> waiting;            // FIFO of queued field ids
   int active = 0;
+  Ingest ingest;                      // all fields' rows that do not fill the pitch (under mtx;
+                                      // 32 MB beside the budget, allocated at the first such push)
   std::mutex rmtx;                    // results only (never held across CUDA calls)
   std::deque<ServerResult> results;
 };
@@ -2010,8 +2100,16 @@ FITRIG_API int fitrig_server_push(fitrig_server_t s, int32_t field, const void* 
     const bool unit = f->received + 1 >= 3;   // this snapshot completes a unit
     if (unit) CK(launch_stamp(f->d_stamps + 0, st));
     if (dtype == p->storage) {
-      CK(cudaMemcpy2DAsync(dst, p->pitch * eb, data, (size_t)p->nx * ib, (size_t)p->nx * ib, p->ny,
-                           cudaMemcpyDefault, st));
+      const size_t row = (size_t)p->nx * ib, dp = (size_t)p->pitch * eb;
+      cudaPointerAttributes at{};
+      const bool staged = Ingest::suits(dp, row, row, row * (size_t)p->ny) &&
+                          cudaPointerGetAttributes(&at, data) == cudaSuccess &&
+                          (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeUnregistered) &&
+                          s->ingest.ready();
+      if (staged)
+        CK(s->ingest.rows(dst, dp, static_cast<const char*>(data), row, p->ny, st));
+      else
+        CK(cudaMemcpy2DAsync(dst, dp, data, row, row, p->ny, cudaMemcpyDefault, st));
     } else {
       if (!p->d_staging) CK(dmalloc(p, &p->d_staging, (size_t)p->nx * p->ny * 4));
       CK(cudaMemcpyAsync(p->d_staging, data, (size_t)p->nx * p->ny * ib, cudaMemcpyDefault, st));
@@ -2254,6 +2352,7 @@ FITRIG_API int fitrig_server_destroy(fitrig_server_t s) {
       delete f;
     }
     s->fields.clear();
+    s->ingest.release();
   }
   delete s;
   return FITRIG_OK;
@@ -2291,6 +2390,7 @@ FITRIG_API int fitrig_plan_destroy(fitrig_plan_t p) {
   free_all(p);
   for (int i = 0; i < 2 * FITRIG_KERNEL_COUNT; ++i)
     if (p->ev[i]) cudaEventDestroy(p->ev[i]);
+  p->ingest.release();
   for (cudaStream_t c : p->copy_st)
     if (c) cudaStreamDestroy(c);
   for (cudaEvent_t c : p->copy_ev)
