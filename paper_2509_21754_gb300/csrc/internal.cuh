@@ -300,8 +300,20 @@ void noise_split_carve(void* base, int groups, int64_t stride, NoiseScratch* s);
 // (for the count of invalid ones).
 cudaError_t launch_noise(const float* vals, int groups, int64_t stride, int64_t n, int mode,
                          const NoiseScratch& s, double* centre_scale, cudaStream_t st);
-// thr32[g] = largest float <= centre + tau*scale (+inf if degenerate), and
-// inv_scale[g] = 1/scale (0 if degenerate)
+// The threshold of one group: the largest float <= centre + tau*scale (+inf if
+// degenerate), so that (float v > it) <=> ((double)v > centre + tau*scale), and
+// *inv_scale = 1/scale (0 if degenerate; null: not wanted).
+__device__ __forceinline__ float group_threshold(const double* cs, int g, double tau,
+                                                 double* inv_scale) {
+  const double c = cs[2 * g], s = cs[2 * g + 1];
+  if (!(s > 0.0) || !isfinite(c) || !isfinite(s)) {
+    if (inv_scale) *inv_scale = 0.0;
+    return INFINITY;   // degenerate spread: nothing is selected
+  }
+  if (inv_scale) *inv_scale = 1.0 / s;
+  return __double2float_rd(c + tau * s);
+}
+// thr32[g] and inv_scale[g] of every group
 cudaError_t launch_thresholds(const double* centre_scale, int groups, double tau, float* thr,
                               double* inv_scale, cudaStream_t st);
 
@@ -338,7 +350,6 @@ cudaError_t launch_select(const float* vals, int groups, int64_t stride, const f
                           const SelectScratch& s, unsigned* status, cudaStream_t st);
 cudaError_t launch_count_selected(const float* vals, int groups, int64_t stride, const float* thr,
                                   int nblk, int* wcnt, long long* total, cudaStream_t st);
-cudaError_t launch_clamp_count(int* n, int cap, unsigned* status, cudaStream_t st);
 cudaError_t launch_components(int Tx, int Ty, int64_t T, const SelectScratch& s,
                               unsigned* status, cudaStream_t st);
 
@@ -371,15 +382,17 @@ struct BlockScratch {
 // `stride` (carved by block_scratch_carve in the same order).
 size_t block_scratch_bytes(int groups, int Tx, int Ty, int64_t stride);
 void block_scratch_carve(void* base, int groups, int Tx, int Ty, int64_t stride, BlockScratch* b);
-// Threshold (v > thr[g]), 8-connected components and their peaks over groups
+// Threshold (v > group_threshold(cs, g, tau); 1/scale of each group to inv), 8-connected
+// components and their peaks over groups
 // x Ty x Tx tiles at vals[g * stride + ty * Tx + tx]; writes the peaks, in
 // (group, t) order, as SelItem{g, t, v} to peaks[0..min(n, cap)) with n in
 // b.counters[2] (with peaks == nullptr the list is left to launch_emit_rows:
 // the peak bitmap and the rows' offsets stay in b); flags kErrCapacity (and
 // *want = selected count) when more than `cap` tiles are selected.
 cudaError_t launch_block_select(const float* vals, int groups, int64_t stride, int Tx, int Ty,
-                                const float* thr, const BlockScratch& b, SelItem* peaks,
-                                int64_t cap, unsigned* status, unsigned* want, cudaStream_t st);
+                                const double* cs, double tau, double* inv, const BlockScratch& b,
+                                SelItem* peaks, int64_t cap, unsigned* status, unsigned* want,
+                                cudaStream_t st);
 
 struct CandArgs {
   int nx, ny, w, Tx, Ty;
@@ -413,16 +426,18 @@ cudaError_t launch_emit_candidates(const CandArgs& a, const SelectScratch& s, in
                                    fitrig_candidate* tmp, unsigned* status, cudaStream_t st);
 
 // The candidates of an ordered peak list (launch_block_select), as
-// launch_emit_candidates does from its own list.
+// launch_emit_candidates does from its own list: a frequency branch's at [0,
+// npeak), an image branch's after the first *base (null: 0).  Sets *a.nout to
+// the number of candidates so far, at most a.cap (more: kErrCapacity).
 cudaError_t launch_emit_peaks(const CandArgs& a, const SelItem* peaks, const int* npeak,
-                              int* base, fitrig_candidate* tmp, cudaStream_t st);
+                              const int* base, fitrig_candidate* tmp, unsigned* status,
+                              cudaStream_t st);
 // The image candidates of a launch_block_select run without a peak list
 // (peaks == nullptr), from its peak bitmap: needs a.w <= 8 and a.arg, or a.w
 // == 1; the same candidates, in the same places, as launch_emit_peaks on the
 // list.
-// Adds the peak count to *a.nout.
 cudaError_t launch_emit_rows(const CandArgs& a, const float* vals, int groups, const BlockScratch& b,
-                             int64_t cap, int* base, cudaStream_t st);
+                             int64_t cap, const int* base, unsigned* status, cudaStream_t st);
 cudaError_t launch_export_candidates(const fitrig_candidate* src, const int* n,
                                      fitrig_candidate* dst, int cap, cudaStream_t st);
 

@@ -69,8 +69,9 @@ __device__ __forceinline__ void kahan_add(float term, float& s, float& comp) {
 template <bool VEC>
 __global__ void __launch_bounds__(kNoiseThreads) k_sum_pass(const float* __restrict__ vals,
                                                             int64_t stride, int nblk, int sq,
-                                                            const float* __restrict__ shift,
+                                                            const float* shift,
                                                             double* part, int* cnt) {
+  pdl_begin();
   __shared__ double sh[kNoiseThreads];
   __shared__ int shc[kNoiseThreads];
   const int g = blockIdx.y;
@@ -120,17 +121,27 @@ __global__ void __launch_bounds__(kNoiseThreads) k_sum_pass(const float* __restr
 }
 
 // stage 0: mean -> cs[2g], shift[g] = (float)mean.  stage 1: population std.
+// One warp per group adds the blocks' partials, lane l those of blocks l, l +
+// 32, .. and then across the lanes (a fixed order; one thread's chain of 608
+// FP64 additions took 43 us).
 __global__ void k_sum_final(int groups, int64_t n, int nblk, int stage, const double* part,
                             const int* cnt, float* shift, double* cs,
                             unsigned long long* invalid) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_begin();
+  const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (g >= groups) return;
   double s = 0.0;
   long long c = 0;
-  for (int b = 0; b < nblk; ++b) {
+  for (int b = lane; b < nblk; b += 32) {
     s += part[(size_t)g * nblk + b];
     c += cnt[(size_t)g * nblk + b];
   }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    c += __shfl_xor_sync(0xffffffffu, c, o);
+  }
+  if (lane != 0) return;
   if (stage == 0) {
     if (invalid && c < n) atomicAdd(invalid, (unsigned long long)(n - c));
     const double mean = c > 0 ? s / (double)c : NAN;
@@ -1977,15 +1988,16 @@ cudaError_t launch_noise(const float* vals, int groups, int64_t stride, int64_t 
   const bool vec = (reinterpret_cast<uintptr_t>(vals) % 16 == 0) && (stride % 4 == 0);
   if (mode == FITRIG_NOISE_MEANSTD) {
     for (int stage = 0; stage < 2; ++stage) {
-      if (vec)
-        k_sum_pass<true><<<grid, kNoiseThreads, 0, st>>>(vals, stride, nblk, stage, s.shift,
-                                                         s.part, s.cnt);
-      else
-        k_sum_pass<false><<<grid, kNoiseThreads, 0, st>>>(vals, stride, nblk, stage, s.shift,
-                                                          s.part, s.cnt);
-      k_sum_final<<<(groups + 127) / 128, 128, 0, st>>>(groups, n, nblk, stage, s.part, s.cnt,
-                                                        s.shift, cs,
-                                                        stage == 0 ? s.invalid : nullptr);
+      cudaError_t e =
+          vec ? launch_pdl(k_sum_pass<true>, grid, dim3(kNoiseThreads), 0, st, vals, stride, nblk, stage,
+                           (const float*)s.shift, s.part, s.cnt)
+              : launch_pdl(k_sum_pass<false>, grid, dim3(kNoiseThreads), 0, st, vals, stride, nblk,
+                           stage, (const float*)s.shift, s.part, s.cnt);
+      if (e == cudaSuccess)
+        e = launch_pdl(k_sum_final, dim3((groups + 7) / 8), dim3(256), 0, st, groups, n, nblk, stage,
+                       (const double*)s.part, (const int*)s.cnt, s.shift, cs,
+                       stage == 0 ? s.invalid : (unsigned long long*)nullptr);
+      if (e != cudaSuccess) return e;
     }
     count_launches(4);
     return cudaGetLastError();
@@ -2043,15 +2055,7 @@ __global__ void k_thresholds(const double* cs, int groups, double tau, float* th
   pdl_begin();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= groups) return;
-  const double c = cs[2 * g], s = cs[2 * g + 1];
-  if (!(s > 0.0) || !isfinite(c) || !isfinite(s)) {
-    thr[g] = INFINITY;   // degenerate spread: nothing is selected
-    inv_scale[g] = 0.0;
-    return;
-  }
-  // largest float <= c + tau*s, so (float v > thr) <=> ((double)v > c + tau*s)
-  thr[g] = __double2float_rd(c + tau * s);
-  inv_scale[g] = 1.0 / s;
+  thr[g] = group_threshold(cs, g, tau, inv_scale + g);
 }
 
 cudaError_t launch_thresholds(const double* cs, int groups, double tau, float* thr,

@@ -75,12 +75,11 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_count(const float* __restri
   if (lane == 0) wcnt[((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5] = cnt;
 }
 
-// Exclusive scan of per-warp (or per-block) counts (one block of 1024 threads).
-__global__ void __launch_bounds__(1024) k_scan_blocks(int nblk, const int* blkcnt, int* blkoff,
-                                                      int* total, int64_t cap,
-                                                      unsigned* status, unsigned* want) {
-  pdl_begin();
-  __shared__ long long sh[1024];
+// Exclusive scan of per-warp (or per-block) counts (one block of 1024 threads;
+// sh: its shared memory).
+__device__ __forceinline__ void scan_counts(int nblk, const int* blkcnt, int* blkoff, int* total,
+                                            int64_t cap, unsigned* status, unsigned* want,
+                                            long long* sh) {
   const int per = (nblk + 1023) / 1024;
   const int b0 = threadIdx.x * per;
   long long local = 0;
@@ -106,6 +105,13 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(int nblk, const int* blkcn
       if (want) atomicMax(want, (unsigned)(tot < 0xffffffffll ? tot : 0xffffffffll));
     }
   }
+}
+
+__global__ void __launch_bounds__(1024) k_scan_blocks(int nblk, const int* blkcnt, int* blkoff,
+                                                      int* total, int64_t cap,
+                                                      unsigned* status, unsigned* want) {
+  __shared__ long long sh[1024];
+  scan_counts(nblk, blkcnt, blkoff, total, cap, status, want, sh);
 }
 
 template <bool VEC>
@@ -249,21 +255,6 @@ cudaError_t launch_count_selected(const float* vals, int groups, int64_t stride,
     k_sel_count<false><<<nblk, kSelThreads, 0, st>>>(vals, groups, stride, thr, chunk, wcnt);
   k_sum_counts<<<1, 256, 0, st>>>(nw, wcnt, total);
   count_launches(2);
-  return cudaGetLastError();
-}
-
-__global__ void k_clamp_count(int* n, int cap, unsigned* status) {
-  pdl_begin();
-  if (*n > cap) {
-    *n = cap;
-    atomicOr(status, kErrCapacity);
-  }
-}
-
-cudaError_t launch_clamp_count(int* n, int cap, unsigned* status, cudaStream_t st) {
-  const cudaError_t e = launch_pdl(k_clamp_count, dim3(1), dim3(1), 0, st, n, cap, status);
-  if (e != cudaSuccess) return e;
-  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -515,21 +506,25 @@ __device__ __forceinline__ uint64_t run_bits(uint64_t m, int s) {
 constexpr int kBlkMaxRuns = kBlkT / 2;   // runs of a block (alternating bits at most)
 
 // Selected-tile bitmap: bit (tx & 31) of word tx / 32 of row (g, ty) is
-// v > thr[g] (never for NaN: an invalid tile); bits past the row's end are 0.
+// v > the group's threshold (never for NaN: an invalid tile); bits past the row's end are 0.
 // One warp per row: all of the row's loads (coalesced, up to 32 per lane) are
 // issued before its ballots.
 constexpr int kMaskThreads = 256;
 __global__ void __launch_bounds__(kMaskThreads) k_blk_mask(const float* __restrict__ vals,
                                                            int64_t stride, int Tx, int Ty,
                                                            int64_t nrows,
-                                                           const float* __restrict__ thr,
+                                                           const double* __restrict__ cs,
+                                                           double tau, double* inv,
                                                            BlockScratch b) {
   pdl_begin();
   const int lane = threadIdx.x & 31;
   const int64_t r = ((int64_t)blockIdx.x * kMaskThreads + threadIdx.x) >> 5;
   if (r >= nrows) return;
   const int g = (int)(r / Ty), ty = (int)(r - (int64_t)g * Ty);
-  const float th = thr[g];
+  // (a launch of its own for the thresholds was one more step of the chain)
+  float th = 0.f;
+  if (lane == 0) th = group_threshold(cs, g, tau, ty == 0 ? inv + g : nullptr);
+  th = __shfl_sync(0xffffffffu, th, 0);
   const float* row = vals + (size_t)g * stride + (int64_t)ty * Tx;
   uint32_t* out = b.sbits + (size_t)r * b.words;
   for (int w0 = 0; w0 < b.words; w0 += 32) {
@@ -846,13 +841,13 @@ __device__ __forceinline__ bool valid_id(const BlockScratch& b, int64_t nblocks,
   return blk < nblocks && (id - blk * kBlkIds) < b.bstat[blk].x;
 }
 
-__global__ void k_blk_merge(int64_t stride, int Tx, int64_t nblocks, BlockScratch b,
-                            unsigned* status) {
-  pdl_begin();
+// (the loads of words that other warps change go past the L1 cache, so that
+// the steps may also follow each other inside one CTA)
+__device__ __forceinline__ void blk_merge(int64_t stride, int Tx, int64_t nblocks,
+                                          const BlockScratch& b, unsigned* status, int64_t w0,
+                                          int64_t nw) {
   const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t blk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; blk < nblocks;
-       blk += nw) {
+  for (int64_t blk = w0; blk < nblocks; blk += nw) {
     const int np = b.bstat[blk].y;
     for (int k = lane; k < np; k += 32) {
       const unsigned long long pk = b.pairs[blk * kBlkPairs + k];
@@ -871,12 +866,10 @@ __global__ void k_blk_merge(int64_t stride, int Tx, int64_t nblocks, BlockScratc
 }
 
 // Merged peak keys: every boundary component raises its root's key.
-__global__ void k_blk_resolve(int64_t nblocks, BlockScratch b) {
-  pdl_begin();
+__device__ __forceinline__ void blk_resolve(int64_t nblocks, const BlockScratch& b, int64_t w0,
+                                            int64_t nw) {
   const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t blk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; blk < nblocks;
-       blk += nw) {
+  for (int64_t blk = w0; blk < nblocks; blk += nw) {
     const int n = b.bstat[blk].x;
     for (int k = lane; k < n; k += 32) {
       const int id = (int)(blk * kBlkIds + k);
@@ -887,21 +880,40 @@ __global__ void k_blk_resolve(int64_t nblocks, BlockScratch b) {
 }
 
 // Each merged component's peak bit.
-__global__ void k_blk_mark(int Tx, int Ty, int64_t nblocks, BlockScratch b) {
-  pdl_begin();
+__device__ __forceinline__ void blk_mark(int Tx, int Ty, int64_t nblocks, const BlockScratch& b,
+                                         int64_t w0, int64_t nw) {
   const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t blk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; blk < nblocks;
-       blk += nw) {
+  for (int64_t blk = w0; blk < nblocks; blk += nw) {
     const int n = b.bstat[blk].x;
     for (int k = lane; k < n; k += 32) {
       const int id = (int)(blk * kBlkIds + k);
-      if (b.bpar[id] != id) continue;   // roots never change after the unions
-      const uint32_t t = 0xffffffffu - (uint32_t)b.rkey[id];
+      if (__ldcg(&b.bpar[id]) != id) continue;   // roots never change after the unions
+      const uint32_t t = 0xffffffffu - (uint32_t)__ldcg(&b.rkey[id]);
       const int ty = (int)(t / (uint32_t)Tx), tx = (int)(t - (uint32_t)ty * (uint32_t)Tx);
       atomicOr(&b.pbits[((size_t)b.bgrp[id] * Ty + ty) * b.words + (tx >> 5)], 1u << (tx & 31));
     }
   }
+}
+
+__device__ __forceinline__ int64_t grid_warp() {
+  return ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+}
+__device__ __forceinline__ int64_t grid_warps() { return ((int64_t)gridDim.x * blockDim.x) >> 5; }
+
+__global__ void k_blk_merge(int64_t stride, int Tx, int64_t nblocks, BlockScratch b,
+                            unsigned* status) {
+  pdl_begin();
+  blk_merge(stride, Tx, nblocks, b, status, grid_warp(), grid_warps());
+}
+
+__global__ void k_blk_resolve(int64_t nblocks, BlockScratch b) {
+  pdl_begin();
+  blk_resolve(nblocks, b, grid_warp(), grid_warps());
+}
+
+__global__ void k_blk_mark(int Tx, int Ty, int64_t nblocks, BlockScratch b) {
+  pdl_begin();
+  blk_mark(Tx, Ty, nblocks, b, grid_warp(), grid_warps());
 }
 
 // Ordered compaction of the peak bitmap, one warp per tile row and
@@ -985,11 +997,10 @@ __global__ void __launch_bounds__(kPbThreads) k_pbits_write(int64_t nrows, int T
   }
 }
 
-// The selected count (the blocks' sum) against the selection capacity.
-__global__ void __launch_bounds__(1024) k_blk_check(int64_t nblocks, BlockScratch b, int64_t cap,
-                                                    unsigned* status, unsigned* want) {
-  pdl_begin();
-  __shared__ long long part[32];
+// The selected count (the blocks' sum) against the selection capacity, by one
+// CTA of 1024 threads.
+__device__ __forceinline__ void blk_check(int64_t nblocks, const BlockScratch& b, int64_t cap,
+                                          unsigned* status, unsigned* want, long long* part) {
   long long n = 0;
   for (int64_t i = threadIdx.x; i < nblocks; i += 1024) n += b.bstat[i].z;
   for (int o = 16; o; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
@@ -1003,6 +1014,75 @@ __global__ void __launch_bounds__(1024) k_blk_check(int64_t nblocks, BlockScratc
       if (want) atomicMax(want, (unsigned)(tot < 0xffffffffll ? tot : 0xffffffffll));
     }
   }
+}
+
+// One CTA scans the row counts of the CTAs of k_pbits_count, another checks
+// the capacity.
+__global__ void __launch_bounds__(1024) k_blk_scan(int nblk, int64_t nblocks, BlockScratch b,
+                                                   int64_t cap, unsigned* status, unsigned* want) {
+  pdl_begin();
+  __shared__ long long sh[1024];
+  if (blockIdx.x == 0)
+    scan_counts(nblk, b.blkcnt, b.blkoff, &b.counters[2], cap, status, (unsigned*)nullptr, sh);
+  else
+    blk_check(nblocks, b, cap, status, want, sh);
+}
+
+// Small maps: everything after the labelling in one CTA, whose barriers cost
+// a fraction of the launches they replace (the full labelling of blocks of
+// many runs, unions, peaks, row counts, their scan and the check: seven).
+// Bounded by kTailBlocks blocks and kTailRows rows, what 32 warps walk in about
+// the time of the launches.
+constexpr int kTailThreads = 1024;
+constexpr int64_t kTailBlocks = 256;
+constexpr int64_t kTailRows = 4096;
+
+__global__ void __launch_bounds__(kTailThreads) k_blk_tail(const float* __restrict__ vals,
+                                                           int64_t stride, int Tx, int Ty,
+                                                           int64_t nblocks, int64_t nrows,
+                                                           BlockScratch b, int64_t cap,
+                                                           unsigned* status, unsigned* want) {
+  pdl_begin();
+  __shared__ union {
+    BlkShared<kTailThreads, kBlkMaxRuns> label;
+    long long scan[1024];
+  } sh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (__syncthreads_or(tid < nblocks && b.bstat[tid].w)) {
+    const int nbx = (Tx + kBlkX - 1) / kBlkX, nby = (Ty + kBlkY - 1) / kBlkY;
+    for (int k = 0; k < nblocks; ++k) {
+      if (!b.bstat[k].w) continue;   // the same word for every thread
+      __syncthreads();
+      blk_label(sh.label, vals, stride, Tx, Ty, b, k, k / (nbx * nby), k % nbx, k / nbx % nby, status);
+      __syncthreads();
+    }
+  }
+  blk_merge(stride, Tx, nblocks, b, status, warp, kTailThreads / 32);
+  __syncthreads();
+  blk_resolve(nblocks, b, warp, kTailThreads / 32);
+  __syncthreads();
+  blk_mark(Tx, Ty, nblocks, b, warp, kTailThreads / 32);
+  __syncthreads();
+  // a thread per tile row (the bits set above are past the L1 cache)
+  for (int64_t r = tid; r < nrows; r += kTailThreads) {
+    const uint32_t* row = b.pbits + (size_t)r * b.words;
+    int c = 0;
+    for (int w = 0; w < b.words; ++w) c += __popc(__ldcg(row + w));
+    b.rowcnt[r] = c;
+  }
+  __syncthreads();
+  const int ncta = (int)((nrows + kRowsPerCta - 1) / kRowsPerCta);
+  for (int i = tid; i < ncta; i += kTailThreads) {
+    int c = 0;
+    for (int64_t r = (int64_t)i * kRowsPerCta; r < nrows && r < (int64_t)(i + 1) * kRowsPerCta; ++r)
+      c += b.rowcnt[r];
+    b.blkcnt[i] = c;
+  }
+  __syncthreads();
+  scan_counts(ncta, b.blkcnt, b.blkoff, &b.counters[2], cap, status, (unsigned*)nullptr, sh.scan);
+  __syncthreads();
+  blk_check(nblocks, b, cap, status, want, sh.scan);
+  (void)lane;
 }
 
 static int block_words(int Tx) { return (Tx + 31) / 32; }
@@ -1066,8 +1146,9 @@ void block_scratch_carve(void* base, int groups, int Tx, int Ty, int64_t stride,
 }
 
 cudaError_t launch_block_select(const float* vals, int groups, int64_t stride, int Tx, int Ty,
-                                const float* thr, const BlockScratch& b, SelItem* peaks,
-                                int64_t cap, unsigned* status, unsigned* want, cudaStream_t st) {
+                                const double* cs, double tau, double* inv, const BlockScratch& b,
+                                SelItem* peaks, int64_t cap, unsigned* status, unsigned* want,
+                                cudaStream_t st) {
   // peaks == nullptr: the caller emits straight from the rows (launch_emit_rows)
   const int64_t nblocks = block_count(groups, Tx, Ty);
   if (groups < 1 || groups > 65535 || (Ty + kBlkY - 1) / kBlkY > 65535 ||
@@ -1077,36 +1158,43 @@ cudaError_t launch_block_select(const float* vals, int groups, int64_t stride, i
   // (counters[2], the peak count, is written by the scan below; nothing else
   // is read, so no clearing launch sits between the noise and this chain)
   const int64_t nrows = (int64_t)groups * Ty;
+  const int64_t ncta = (nrows + kRowsPerCta - 1) / kRowsPerCta;
+  if (ncta > b.nblk) return cudaErrorInvalidValue;   // sized by block_scratch_carve
+  int launches = 2;
   cudaError_t e = launch_pdl(k_blk_mask, dim3((unsigned)((nrows * 32 + kMaskThreads - 1) / kMaskThreads)),
-                             dim3(kMaskThreads), 0, st, vals, stride, Tx, Ty, nrows, thr, b);
+                             dim3(kMaskThreads), 0, st, vals, stride, Tx, Ty, nrows, cs, tau, inv, b);
   const dim3 grid((Tx + kBlkX - 1) / kBlkX, (Ty + kBlkY - 1) / kBlkY, groups);
   if (e == cudaSuccess)
     e = launch_pdl(k_blk_cc, grid, dim3(kBlkFewThreads), 0, st, vals, stride, Tx, Ty, b, status);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_blk_cc_full,
-                   dim3((unsigned)std::min<int64_t>((nblocks + kBlkThreads - 1) / kBlkThreads, 152 * 4)),
-                   dim3(kBlkThreads), 0, st, vals, stride, Tx, Ty, nblocks, b, status);
-  const unsigned wgrid = (unsigned)std::min<int64_t>((nblocks + 7) / 8, 152 * 64);   // a warp per block
-  if (e == cudaSuccess)
-    e = launch_pdl(k_blk_merge, dim3(wgrid), dim3(256), 0, st, stride, Tx, nblocks, b, status);
-  if (e == cudaSuccess) e = launch_pdl(k_blk_resolve, dim3(wgrid), dim3(256), 0, st, nblocks, b);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_blk_mark, dim3(wgrid), dim3(256), 0, st, Tx, Ty, nblocks, b);
+  if (nblocks <= kTailBlocks && nrows <= kTailRows) {
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_tail, dim3(1), dim3(kTailThreads), 0, st, vals, stride, Tx, Ty, nblocks,
+                     nrows, b, cap, status, want);
+    launches += 1;
+  } else {
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_cc_full,
+                     dim3((unsigned)std::min<int64_t>((nblocks + kBlkThreads - 1) / kBlkThreads, 152 * 4)),
+                     dim3(kBlkThreads), 0, st, vals, stride, Tx, Ty, nblocks, b, status);
+    const unsigned wgrid = (unsigned)std::min<int64_t>((nblocks + 7) / 8, 152 * 64);   // a warp per block
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_merge, dim3(wgrid), dim3(256), 0, st, stride, Tx, nblocks, b, status);
+    if (e == cudaSuccess) e = launch_pdl(k_blk_resolve, dim3(wgrid), dim3(256), 0, st, nblocks, b);
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_mark, dim3(wgrid), dim3(256), 0, st, Tx, Ty, nblocks, b);
+    if (e == cudaSuccess)
+      e = launch_pdl(k_pbits_count, dim3((unsigned)ncta), dim3(kPbThreads), 0, st, nrows, b);
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_scan, dim3(2), dim3(1024), 0, st, (int)ncta, nblocks, b, cap, status, want);
+    launches += 6;
+  }
+  if (e == cudaSuccess && peaks) {
+    e = launch_pdl(k_pbits_write, dim3((unsigned)ncta), dim3(kPbThreads), 0, st, nrows, Tx, Ty, vals,
+                   stride, b, peaks, cap);
+    launches += 1;
+  }
   if (e != cudaSuccess) return e;
-  const int64_t ncta = (nrows + kRowsPerCta - 1) / kRowsPerCta;
-  if (ncta > b.nblk) return cudaErrorInvalidValue;   // sized by block_scratch_carve
-  const unsigned rgrid = (unsigned)ncta;   // a warp per row
-  e = launch_pdl(k_pbits_count, dim3(rgrid), dim3(kPbThreads), 0, st, nrows, b);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_scan_blocks, dim3(1), dim3(1024), 0, st, (int)ncta, (const int*)b.blkcnt,
-                   b.blkoff, &b.counters[2], cap, status, (unsigned*)nullptr);
-  if (e == cudaSuccess && peaks)
-    e = launch_pdl(k_pbits_write, dim3(rgrid), dim3(kPbThreads), 0, st, nrows, Tx, Ty, vals, stride,
-                   b, peaks, cap);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_blk_check, dim3(1), dim3(1024), 0, st, nblocks, b, cap, status, want);
-  if (e != cudaSuccess) return e;
-  count_launches(peaks ? 10 : 9);
+  count_launches(launches);
   return cudaGetLastError();
 }
 
@@ -1241,12 +1329,23 @@ __device__ __forceinline__ float significance(const CandArgs& a, const SelItem& 
   return (float)(((double)it.v - a.cs[2 * it.group]) * a.inv[it.group]);
 }
 
+// Candidates so far: those before this branch's and its peaks, at most the
+// buffer's (by one thread of the emitting kernel; no other one reads it).
+__device__ __forceinline__ void set_count(const CandArgs& a, int64_t total, unsigned* status) {
+  if (total > a.cap) {
+    total = a.cap;
+    atomicOr(status, kErrCapacity);
+  }
+  *a.nout = (int)total;
+}
+
 // Frequency branch: one thread per peak; tile-centre order is (y, x) order,
 // so the peaks' list order is already the output order.
 __global__ void k_emit_freq(CandArgs a, const SelItem* __restrict__ items, const int* np_,
-                            const int* __restrict__ plist) {
+                            const int* __restrict__ plist, unsigned* status) {
   pdl_begin();
   const int np = *np_;
+  if (status && blockIdx.x == 0 && threadIdx.x == 0) set_count(a, np, status);
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
     const SelItem it = peak_item(items, plist, p);
     const int ty = it.t / a.Tx, tx = it.t - (it.t / a.Tx) * a.Tx;
@@ -1368,7 +1467,8 @@ __global__ void __launch_bounds__(kGroupWarps * 32) k_group_sort(CandArgs a, con
                                                                  const fitrig_candidate* tmp,
                                                                  const SelItem* __restrict__ items,
                                                                  const int* __restrict__ plist,
-                                                                 const int* base_) {
+                                                                 const int* base_,
+                                                                 unsigned* status) {
   pdl_begin();
   __shared__ int counts[kGroupWarps][kMaxW];
   // one peak: its group (snapshot, tile row) and, for the count and the
@@ -1413,6 +1513,7 @@ __global__ void __launch_bounds__(kGroupWarps * 32) k_group_sort(CandArgs a, con
   };
   const int np = *np_;
   const int base = base_ ? *base_ : 0;
+  if (status && blockIdx.x == 0 && threadIdx.x == 0) set_count(a, (int64_t)base + np, status);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int* cnt = counts[warp];
   const int wid = blockIdx.x * kGroupWarps + warp;
@@ -1530,8 +1631,11 @@ constexpr int kRowsBatch = 4;
 template <bool WIDE, int MAXW>
 __global__ void __launch_bounds__(kPbThreads, MAXW == 1 ? 6 : 4) k_emit_rows(CandArgs a, const float* __restrict__ vals,
                                                           int64_t nrows, BlockScratch b,
-                                                          int64_t cap, const int* base_) {
+                                                          int64_t cap, const int* base_,
+                                                          unsigned* status) {
   pdl_begin();
+  const int64_t base = base_ ? *base_ : 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) set_count(a, base + b.counters[2], status);
   const int lane = threadIdx.x & 31;
   const int64_t r = ((int64_t)blockIdx.x * kPbThreads + threadIdx.x) >> 5;
   if (r >= nrows || (WIDE && b.rowcnt[r] == 0)) return;
@@ -1542,7 +1646,6 @@ __global__ void __launch_bounds__(kPbThreads, MAXW == 1 ? 6 : 4) k_emit_rows(Can
   const uint8_t* ag = a.arg ? a.arg + (size_t)g * a.stride + t0 : nullptr;
   const float* vg = vals + (size_t)g * a.stride + t0;
   const int64_t roff = row_offset(b, r);
-  const int64_t base = *base_;
   auto arg_of = [&](int t) -> int { return MAXW == 1 ? 0 : ag[t]; };
   // place of the next peak of each in-tile row over the words so far
   int next[MAXW];
@@ -1646,7 +1749,6 @@ __global__ void __launch_bounds__(kPbThreads, MAXW == 1 ? 6 : 4) k_emit_rows(Can
 }
 
 __global__ void k_add_count(int* total, const int* part) {
-  pdl_begin();
   *total += *part;
 }
 
@@ -1667,31 +1769,30 @@ cudaError_t launch_export_candidates(const fitrig_candidate* src, const int* n,
 }
 
 cudaError_t launch_emit_peaks(const CandArgs& a, const SelItem* peaks, const int* npeak,
-                              int* base, fitrig_candidate* tmp, cudaStream_t st) {
+                              const int* base, fitrig_candidate* tmp, unsigned* status,
+                              cudaStream_t st) {
   cudaError_t e;
+  int launches = 1;
   if (a.branch == FITRIG_BRANCH_FREQ) {
     e = launch_pdl(k_emit_freq, dim3(152 * 4), dim3(256), 0, st, a, peaks, npeak,
-                   (const int*)nullptr);
-    count_launches(1);
+                   (const int*)nullptr, status);
   } else if (a.arg) {
     e = launch_pdl(k_group_sort<true>, dim3(152 * 4), dim3(kGroupWarps * 32), 0, st, a, npeak,
-                   (const fitrig_candidate*)tmp, peaks, (const int*)nullptr, (const int*)base);
-    count_launches(1);
+                   (const fitrig_candidate*)tmp, peaks, (const int*)nullptr, base, status);
   } else {
     e = launch_pdl(k_emit_image, dim3(152 * 4), dim3(256), 0, st, a, peaks, npeak,
                    (const int*)nullptr, tmp);
     if (e == cudaSuccess)
       e = launch_pdl(k_group_sort<false>, dim3(152 * 4), dim3(kGroupWarps * 32), 0, st, a, npeak,
-                     (const fitrig_candidate*)tmp, peaks, (const int*)nullptr, (const int*)base);
-    count_launches(2);
+                     (const fitrig_candidate*)tmp, peaks, (const int*)nullptr, base, status);
+    launches = 2;
   }
-  if (e == cudaSuccess) e = launch_pdl(k_add_count, dim3(1), dim3(1), 0, st, a.nout, npeak);
-  count_launches(1);
+  count_launches(launches);
   return e;
 }
 
 cudaError_t launch_emit_rows(const CandArgs& a, const float* vals, int groups, const BlockScratch& b,
-                             int64_t cap, int* base, cudaStream_t st) {
+                             int64_t cap, const int* base, unsigned* status, cudaStream_t st) {
   if ((!a.arg && a.w != 1) || a.w < 1 || a.w > kRowsMaxW ||
       ((int64_t)groups * a.Ty + kRowsPerCta - 1) / kRowsPerCta > b.nblk)
     return cudaErrorInvalidValue;
@@ -1699,17 +1800,15 @@ cudaError_t launch_emit_rows(const CandArgs& a, const float* vals, int groups, c
   const dim3 grid((unsigned)((nrows * 32 + kPbThreads - 1) / kPbThreads));
   cudaError_t e;
   if (a.w == 1)
-    e = launch_pdl(k_emit_rows<true, 1>, grid, dim3(kPbThreads), 0, st, a, vals, nrows, b, cap,
-                   (const int*)base);
+    e = launch_pdl(k_emit_rows<true, 1>, grid, dim3(kPbThreads), 0, st, a, vals, nrows, b, cap, base,
+                   status);
   else if (b.words > 32)
     e = launch_pdl(k_emit_rows<true, kRowsMaxW>, grid, dim3(kPbThreads), 0, st, a, vals, nrows, b,
-                   cap, (const int*)base);
+                   cap, base, status);
   else
     e = launch_pdl(k_emit_rows<false, kRowsMaxW>, grid, dim3(kPbThreads), 0, st, a, vals, nrows, b,
-                   cap, (const int*)base);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_add_count, dim3(1), dim3(1), 0, st, a.nout, (const int*)&b.counters[2]);
-  count_launches(2);
+                   cap, base, status);
+  count_launches(1);
   return e;
 }
 
@@ -1722,17 +1821,17 @@ cudaError_t launch_emit_candidates(const CandArgs& a, const SelectScratch& s, in
   k_peak_write<<<s.nblk, kSelThreads, 0, st>>>(s.nsel, s.parent, s.peak, s.nblk, s.blkoff,
                                                s.plist);
   if (a.branch == FITRIG_BRANCH_FREQ) {
-    k_emit_freq<<<152 * 4, 256, 0, st>>>(a, s.items, s.npeak, s.plist);
+    k_emit_freq<<<152 * 4, 256, 0, st>>>(a, s.items, s.npeak, s.plist, nullptr);
     count_launches(4);
   } else {
     if (a.arg) {
       k_group_sort<true><<<152 * 4, kGroupWarps * 32, 0, st>>>(a, s.npeak, tmp, s.items, s.plist,
-                                                               base);
+                                                               base, nullptr);
       count_launches(4);
     } else {
       k_emit_image<<<152 * 4, 256, 0, st>>>(a, s.items, s.npeak, s.plist, tmp);
       k_group_sort<false><<<152 * 4, kGroupWarps * 32, 0, st>>>(a, s.npeak, tmp, s.items,
-                                                                s.plist, base);
+                                                                s.plist, base, nullptr);
       count_launches(5);
     }
   }

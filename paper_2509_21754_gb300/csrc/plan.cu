@@ -191,10 +191,10 @@ struct fitrig_plan_s {
   float* d_vp = nullptr;
   uint8_t* d_arg = nullptr;      // fused in-tile arg-max (thread-per-tile path)
   double* d_inv = nullptr;       // units + 1 reciprocal scales
-  unsigned* d_small = nullptr;   // [0] gmax key, [1] status flags, [2] ncand
-  unsigned long long* d_invalid = nullptr;
+  // [0] gmax key, [1] status flags, [2] ncand, [3] wanted capacity, [4..5] d_invalid
+  unsigned* d_small = nullptr;
+  unsigned long long* d_invalid = nullptr;   // inside d_small
   double* d_cs = nullptr;        // (units + 1) x (centre, scale)
-  float* d_thr = nullptr;        // units + 1
   void* d_noise = nullptr;
   void* d_split = nullptr;       // split median/MAD scratch (NoiseScratch::split)
   void* d_blk = nullptr;         // block-tiled components (BlockScratch) of the image branch
@@ -272,8 +272,8 @@ static void drop_graph(fitrig_plan_t p);
 
 static void free_all(fitrig_plan_t p) {
   drop_graph(p);
-  void* ptrs[] = {p->d_stack, p->d_vp,  p->d_small, p->d_invalid,  p->d_cs, p->d_arg, p->d_inv,
-                  p->d_thr,   p->d_noise, p->d_split, p->d_blk, p->d_noise_f, p->d_split_f,
+  void* ptrs[] = {p->d_stack, p->d_vp,  p->d_small, p->d_cs, p->d_arg, p->d_inv,
+                  p->d_noise, p->d_split, p->d_blk, p->d_noise_f, p->d_split_f,
                   p->d_blk_f, p->d_fpeaks, p->d_sel, p->d_cand, p->d_cand_tmp,
                   p->d_bin,   p->d_tw,  p->d_staging, p->d_report, p->d_accum,
                   p->d_hist,  p->d_hwts, p->d_htw,
@@ -535,9 +535,8 @@ static int allocate(fitrig_plan_t p) {
     CK(dmalloc(p, &p->d_arg, (size_t)U * p->vstride));
   CK(dmalloc(p, &p->d_inv, sizeof(double) * (U + 1)));
   CK(dmalloc(p, &p->d_small, 64));
-  CK(dmalloc(p, &p->d_invalid, sizeof(unsigned long long)));
+  p->d_invalid = reinterpret_cast<unsigned long long*>(p->d_small + 4);
   CK(dmalloc(p, &p->d_cs, sizeof(double) * 2 * (U + 1)));
-  CK(dmalloc(p, &p->d_thr, sizeof(float) * (U + 1)));
   const int nblk_img = std::max(1, std::min(1024, (152 * 4 + U - 1) / U));
   const int nblk_freq = 152 * 4;
   // the image branch's estimates (U maps) and eta's (one map) run on two
@@ -1003,9 +1002,8 @@ static void rec(fitrig_plan_t p, int k, int end, cudaStream_t st) {
 // events (not used inside graphs).
 static cudaError_t enqueue_clear(fitrig_plan_t p, cudaStream_t st) {
   // a serving ring keeps word 0, the running maximum M over every snapshot seen
-  cudaError_t e = p->ring ? cudaMemsetAsync(p->d_small + 1, 0, 12, st)
-                          : cudaMemsetAsync(p->d_small, 0, 16, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->d_invalid, 0, sizeof(unsigned long long), st);
+  cudaError_t e = p->ring ? cudaMemsetAsync(p->d_small + 1, 0, 20, st)
+                          : cudaMemsetAsync(p->d_small, 0, 24, st);
   if (e == cudaSuccess && p->d_smax)
     e = cudaMemsetAsync(p->d_smax, 0, sizeof(unsigned) * 2 * p->L, st);
   return e;
@@ -1129,10 +1127,9 @@ static cudaError_t enqueue_post(fitrig_plan_t p, cudaStream_t st, bool timed) {
   if (image) {
     if (timed) rec(p, FITRIG_KERNEL_NOISE, 0, is);
     CKE(launch_noise(p->d_vp, U, p->vstride, p->T, p->noise, ns_img, p->d_cs, is));
-    CKE(launch_thresholds(p->d_cs, U, p->tau, p->d_thr, p->d_inv, is));
     if (timed) rec(p, FITRIG_KERNEL_NOISE, 1, is);
     if (timed) rec(p, FITRIG_KERNEL_SELECT, 0, is);
-    CKE(launch_block_select(p->d_vp, U, p->vstride, p->Tx, p->Ty, p->d_thr, p->blk,
+    CKE(launch_block_select(p->d_vp, U, p->vstride, p->Tx, p->Ty, p->d_cs, p->tau, p->d_inv, p->blk,
                             rows_emit ? nullptr : p->sel.items, p->sel.capacity, status,
                             p->sel.want, is));
     if (is != st) CKE(cudaEventRecord(p->join_ev, is));
@@ -1157,29 +1154,27 @@ static cudaError_t enqueue_post(fitrig_plan_t p, cudaStream_t st, bool timed) {
     mark(FITRIG_KERNEL_SPECTRUM, 1);
     double* cs = p->d_cs + 2 * U;
     CKE(launch_noise(p->d_eta, 1, p->vstride, p->T, p->noise, ns_freq, cs, st));
-    CKE(launch_thresholds(cs, 1, p->tau, p->d_thr + U, p->d_inv + U, st));
-    CKE(launch_block_select(p->d_eta, 1, p->vstride, p->Tx, p->Ty, p->d_thr + U, p->blk_f,
-                            p->d_fpeaks, p->T, status, p->sel.want, st));
+    CKE(launch_block_select(p->d_eta, 1, p->vstride, p->Tx, p->Ty, cs, p->tau, p->d_inv + U,
+                            p->blk_f, p->d_fpeaks, p->T, status, p->sel.want, st));
     ca.branch = FITRIG_BRANCH_FREQ;
     ca.cs = cs;              // eta's estimate (group 0 of its selection)
     ca.inv = p->d_inv + U;
-    CKE(launch_emit_peaks(ca, p->d_fpeaks, &p->blk_f.counters[2], nout, p->d_cand_tmp, st));
+    CKE(launch_emit_peaks(ca, p->d_fpeaks, &p->blk_f.counters[2], nullptr, p->d_cand_tmp, status, st));
   }
   if (image) {
     if (is != st) CKE(cudaStreamWaitEvent(st, p->join_ev, 0));
+    const int* before = freq ? &p->blk_f.counters[2] : nullptr;   // the frequency candidates lead
     ca.branch = FITRIG_BRANCH_IMAGE;
     ca.arg = p->d_arg;
     ca.cs = p->d_cs;
     ca.inv = p->d_inv;
     if (rows_emit)
-      CKE(launch_emit_rows(ca, p->d_vp, U, p->blk, p->sel.capacity, nout, st));
+      CKE(launch_emit_rows(ca, p->d_vp, U, p->blk, p->sel.capacity, before, status, st));
     else
-      CKE(launch_emit_peaks(ca, p->sel.items, &p->blk.counters[2], nout, p->d_cand_tmp, st));
+      CKE(launch_emit_peaks(ca, p->sel.items, &p->blk.counters[2], before, p->d_cand_tmp, status, st));
     mark(FITRIG_KERNEL_SELECT, 1);
   }
-  CKE(launch_clamp_count(nout, (int)p->cand_cap, status, st));
-  CKE(cudaMemcpyAsync(p->h_pinned, p->d_small, 16, cudaMemcpyDeviceToHost, st));
-  CKE(cudaMemcpyAsync(p->h_pinned + 4, p->d_invalid, 8, cudaMemcpyDeviceToHost, st));
+  CKE(cudaMemcpyAsync(p->h_pinned, p->d_small, 24, cudaMemcpyDeviceToHost, st));
   return cudaSuccess;
 }
 
@@ -1226,8 +1221,7 @@ static int grow_select(fitrig_plan_t p) {
 // Post-processing again after grow_select (status words and invalid counts
 // are cleared; M and the tile statistics are kept).
 static int repost(fitrig_plan_t p, cudaStream_t st, int32_t* ncand) {
-  CK(cudaMemsetAsync(p->d_small + 1, 0, 12, st));
-  CK(cudaMemsetAsync(p->d_invalid, 0, sizeof(unsigned long long), st));
+  CK(cudaMemsetAsync(p->d_small + 1, 0, 20, st));
   CK(enqueue_post(p, st, true));
   CK(cudaStreamSynchronize(st));
   return finish_detect(p, ncand);
