@@ -1921,6 +1921,126 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __r
   }
 }
 
+// ---------------------------------------------------------------- MEDMAD, resident form
+// Maps of up to kSmallMax values: one CTA per map holds the keys in shared
+// memory and selects the median and then the MAD (on the keys of |v - median|)
+// by rounds of 2048-bin histograms over the current key range until it is one
+// key.  Integer counting over all finite values, so the result is the element
+// a sort gives, for any input (ties, a constant map): there is no bracket to
+// miss and no fallback launch.  The split form's six launches take 50 to 60 us
+// however small the map is; here the time is the rounds' (two to four each),
+// their barriers and shared atomics: 1 to 64 maps of 1000 / 7000 / 16,384 /
+// 32,768 values 10 / 12 / 16 / 24 us, against 36 / 51 / 55 / 58 us for one map and
+// 60 to 94 us for 62 in the cluster form of callers without scratch.
+constexpr int kSmallMax = 48 * 1024;   // 192 KB of keys
+static_assert(kSmallMax % 4 == 0, "whole float4s");
+
+__global__ void __launch_bounds__(kSplitThreads) k_medmad_small(const float* __restrict__ vals,
+                                                                int64_t stride, int64_t n,
+                                                                double* cs,
+                                                                unsigned long long* invalid) {
+  pdl_begin();
+  extern __shared__ uint32_t skeys[];   // [stride]: the map's keys, kNoKey where not finite
+  __shared__ unsigned hist[kSplitBins];
+  __shared__ unsigned long long wsum[kSplitThreads / 32], found[2];
+  __shared__ uint32_t kmin, kmax;
+  __shared__ unsigned nfin;
+  const int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, m = (int)stride;
+  const float* v = vals + (size_t)g * stride;
+  float med = 0.f;
+  for (int mad = 0; mad < 2; ++mad) {
+    if (tid == 0) {
+      kmin = 0xffffffffu;
+      kmax = 0u;
+      nfin = 0;
+    }
+    __syncthreads();
+    uint32_t lmin = 0xffffffffu, lmax = 0u;
+    unsigned nf = 0;
+    for (int i = tid; i < m; i += kSplitThreads) {
+      uint32_t key = kNoKey;
+      if (mad) {
+        const uint32_t k0 = skeys[i];
+        if (k0 != kNoKey) key = f32_key(fabsf(f32_from_key(k0) - med));
+      } else {
+        const float x = v[i];
+        if (finite_bits(x)) key = f32_key(x);
+      }
+      skeys[i] = key;
+      if (key != kNoKey) {
+        lmin = min(lmin, key);
+        lmax = max(lmax, key);
+        ++nf;
+      }
+    }
+    lmin = __reduce_min_sync(0xffffffffu, lmin);
+    lmax = __reduce_max_sync(0xffffffffu, lmax);
+    nf = __reduce_add_sync(0xffffffffu, nf);
+    if (lane == 0) {
+      atomicMin(&kmin, lmin);
+      atomicMax(&kmax, lmax);
+      atomicAdd(&nfin, nf);
+    }
+    __syncthreads();
+    const unsigned total = nfin;
+    if (total == 0) {
+      if (tid == 0) {
+        cs[2 * g] = NAN;
+        cs[2 * g + 1] = 0.0;
+        if (invalid && n > 0) atomicAdd(invalid, (unsigned long long)n);
+      }
+      return;
+    }
+    uint32_t lo = kmin, hi = kmax;
+    unsigned long long rank = (total - 1) / 2;
+    while (lo < hi) {   // (at most eleven bits of the range are left after each round)
+      const unsigned sh = split_shift(lo, hi);
+      for (int b = tid; b < kSplitBins; b += kSplitThreads) hist[b] = 0;
+      __syncthreads();
+      for (int i = tid; i < m; i += kSplitThreads) {
+        const uint32_t k = skeys[i];
+        if (k >= lo && k <= hi) atomicAdd(&hist[(k - lo) >> sh], 1u);
+      }
+      __syncthreads();
+      unsigned bin;
+      unsigned long long below;
+      if (!split_find(hist, rank, &bin, &below, wsum, found)) break;   // (the rank is always inside)
+      rank -= below;
+      const uint32_t nlo = lo + (bin << sh);
+      const unsigned long long top = (unsigned long long)nlo + (1ull << sh) - 1;
+      hi = top < hi ? (uint32_t)top : hi;
+      lo = nlo;
+    }
+    const float val = f32_from_key(lo);
+    if (mad) {
+      if (tid == 0) {
+        cs[2 * g] = (double)med;
+        cs[2 * g + 1] = kMadToSigma * (double)val;
+        if (invalid && (int64_t)total < n)
+          atomicAdd(invalid, (unsigned long long)(n - (int64_t)total));
+      }
+      return;
+    }
+    med = val;
+    __syncthreads();   // every thread has read the totals before they are reset
+  }
+}
+
+static cudaError_t launch_medmad_small(const float* vals, int groups, int64_t stride, int64_t n,
+                                       double* cs, unsigned long long* invalid, cudaStream_t st) {
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_medmad_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallMax * (int)sizeof(uint32_t));
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  const cudaError_t e = launch_pdl(k_medmad_small, dim3(groups), dim3(kSplitThreads),
+                                   (size_t)stride * sizeof(uint32_t), st, vals, stride, n, cs, invalid);
+  count_launches(1);
+  return e;
+}
+
 template <bool VEC>
 static cudaError_t launch_split_t(const float* vals, int groups, int64_t stride, int64_t n,
                                   const NoiseScratch& ns, double* cs, cudaStream_t st) {
@@ -2003,6 +2123,9 @@ cudaError_t launch_noise(const float* vals, int groups, int64_t stride, int64_t 
     return cudaGetLastError();
   }
   if (mode != FITRIG_NOISE_MEDMAD) return cudaErrorInvalidValue;
+  // small maps: resident in one CTA's shared memory, as many values as fit
+  if (s.allow_cluster && stride <= kSmallMax)
+    return launch_medmad_small(vals, groups, stride, n, cs, s.invalid, st);
   // The split form reads a map twice whatever its size, the grid-wide passes
   // six times with shared atomics per value: 30 maps of 16.8 M values take
   // 0.93 ms against 6.05 ms, 6 maps of 24.2 M with eta's 0.54 against 2.27 ms
