@@ -10,16 +10,17 @@
 // TMA load into a ring of shared-memory stages; each thread carries x^(s+1)
 // and D^(s) of its pixels in registers.  Per unit, Delta and r of the extended
 // block go to shared memory, a horizontal pass forms the w-wide row sums and
-// maxima, and a vertical pass finishes the windows and writes v (windows above
-// 9; smaller ones take the shuffle kernel below, which keeps Delta and r in
-// registers).  Halo pixels
+// maxima, and a vertical pass finishes the windows and writes v (windows of 1
+// and above 9; the others take the shuffle kernels below, which keep Delta and r
+// in registers).  Halo pixels
 // outside the image read as zero, which adds nothing to the sums or the
 // maximum (Delta >= 0), so only n_p needs the clipping.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
-#include "internal.cuh"
+#include "march.cuh"
 
 namespace fitrig {
 
@@ -162,8 +163,8 @@ __global__ void __launch_bounds__(kSlideMaxThreads) k_slide(const __grid_constan
 }
 
 // ---------------------------------------------------------------- small windows
-// Odd windows up to 9 (h <= 4): one thread per column of the extended block,
-// 16 output rows per CTA.  Each thread carries x^(s+1) and D^(s) of its
+// Windows 7 and 9 (h = 3, 4): one thread per column of the extended block,
+// eight output rows per CTA.  Each thread carries x^(s+1) and D^(s) of its
 // column's 16 + 2h rows in registers; per unit, each row's Delta and r go
 // straight into the horizontal window by warp shuffles (a warp of 32 columns
 // yields the 32 - 2h windows that lie inside it; neighbouring warps overlap by
@@ -280,7 +281,9 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_shf(const __grid_co
           const float d = fabsf(dn - dp[i]);   // Delta
           const float ref = SIGNED ? xp[i] : fabsf(xp[i]);
           const float xh = (xp[i] == 0.f) ? kGuardC : ref;   // Eq. 5
-          const float r = fminf(__fdividef(d, xh), 1.f);     // Eq. 4
+          // Eq. 4 (in the ABS reading the saturation is the clamp, and the
+          // approximate reciprocal needs none of the division's range checks)
+          const float r = SIGNED ? fminf(__fdividef(d, xh), 1.f) : __saturatef(d * rcp_approx(xh));
           lane_window<W>(d, r, rs[i % W], rm[i % W], rq[i % W]);
           if (i >= W - 1) {
             const int oy = i - (W - 1);        // output row, window rows oy .. i
@@ -333,10 +336,254 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_shf(const __grid_co
   if (lane == 0 && mx > -INFINITY) atomicMax(a.gmax, f32_key(mx));
 }
 
+// ---------------------------------------------------------------- smallest windows
+// Windows 3 and 5: one thread per pair of columns of the extended
+// block.  Each thread carries x^(s+1) and D^(s) of its columns' rows in
+// registers; per unit, each row's Delta and r go straight into the horizontal
+// window: the W - 1 columns to the right come by warp shuffles (a warp of 64
+// columns yields the windows that begin in its first 64 - 2h; neighbouring
+// warps overlap by 2h columns), and the vertical window is summed over the last
+// w rows of horizontal results, held in registers as the rows stream past.  No
+// Delta or r image is written to shared memory, and the only barrier per
+// snapshot is the ring's.
+// Two columns a thread share the shuffled values (w = 5: 4 shuffles a pixel
+// instead of 9 with a column a thread and windows by doubling), and the zero
+// guard of the ratio is one test per thread and unit.  The sums keep the
+// doubling's order: (x0 + x1) + (x2 + x3), then the rest.  Bound by the latency
+// of its chains at 16 warps per SM, and by its code's size: 12 or 16 output rows
+// repeat fewer halo rows but spill or lose a CTA (32 x 4096^2, w = 5: 8 rows 1.51
+// ms, 12 rows 1.63, 16 rows 2.12; a column a thread 1.73), and at w = 7 and 9 the
+// pairs' registers cost more than the shuffles saved (586 -> 627, 735 -> 1004 us
+// for 32 x 2048^2).
+
+template <int W>
+struct PairShape {
+  static constexpr int kH = W / 2;
+  static constexpr int kRows = 8;                               // output rows per CTA
+  static constexpr int kEH = kRows + 2 * kH;
+  static constexpr int kOWW = W == 3 ? 60 : 64 - 2 * kH;        // output columns per warp
+  static constexpr int kOW = kShfWarps * kOWW;                  // a multiple of 8: x0 - h is 8 - h past
+  static constexpr int kOff = 8 - kH;                           // a TMA-aligned column
+  static constexpr int kBoxW = (kOff + (kShfWarps - 1) * kOWW + 64 + 7) / 8 * 8;
+  static_assert((W == 3 || W == 5) && kOW % 8 == 0 && kBoxW <= 256, "shuffle march shape");
+};
+
+// The sum over e[i .. i + W) in the order of lane doubling.
+template <int W>
+__device__ __forceinline__ float window_sum(const float* e, const float* p, int i) {
+  if (W == 3) return p[i] + e[i + 2];
+  return (p[i] + p[i + 2]) + e[i + 4];
+}
+
+template <typename T, int W, bool SIGNED>
+__global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_pair(
+    const __grid_constant__ CUtensorMap tmap, const SlideArgs a) {
+  using S = PairShape<W>;
+  constexpr int H = S::kH, EH = S::kEH;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const SlideGeom& g = a.g;
+  const int NS = g.stages;
+  const uint32_t stage0 = smem_u32(smem);
+  const uint32_t bar0 = smem_u32(smem + (size_t)NS * g.stage_bytes);
+  constexpr uint32_t box_bytes = (uint32_t)(S::kBoxW * EH * (int)sizeof(T));
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int x0 = blockIdx.x * S::kOW, y0 = blockIdx.y * S::kRows;
+  const int xload = x0 - 8;                     // (negative for the first block: zero fill)
+  const int s0 = blockIdx.z * a.seg_units;                // first unit of the segment
+  const int L = min(a.seg_units, a.nsnap - 2 - s0) + 2;   // its snapshots
+  const int z0 = a.zrot + s0;
+  float* const vp = a.vp + (size_t)s0 * (size_t)a.vstride;
+  unsigned* const smax = a.smax ? a.smax + s0 : nullptr;
+  if (tid == 0) {
+    prefetch_tmap(&tmap);
+    for (int i = 0; i < NS; ++i) mbar_init(bar0 + 8 * i, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int j = 0; j < NS && j < L; ++j) {
+      mbar_expect_tx(bar0 + 8 * j, box_bytes);
+      tma_load_3d(stage0 + j * (uint32_t)g.stage_bytes, &tmap, xload, y0 - H, (z0 + j) % a.nsnap,
+                  bar0 + 8 * j);
+    }
+  }
+  // this lane's two output columns and their clipped widths
+  const int ox = x0 + warp * S::kOWW + 2 * lane;
+  const bool out0 = 2 * lane < S::kOWW && ox < a.nx, out1 = 2 * lane < S::kOWW && ox + 1 < a.nx;
+  const bool pair = out1 && (a.nx & 1) == 0;    // 8-byte aligned (ox and vstride are even)
+  const int nxw0 = min(ox + H, a.nx - 1) - max(ox - H, 0) + 1;
+  const int nxw1 = min(ox + 1 + H, a.nx - 1) - max(ox + 1 - H, 0) + 1;
+  float x[EH][2], d[EH][2];
+#pragma unroll
+  for (int i = 0; i < EH; ++i) x[i][0] = x[i][1] = d[i][0] = d[i][1] = 0.f;
+  float mx = -INFINITY;
+  const uint64_t deadline = globaltimer_ns() + a.timeout_ns;
+
+  // one unit's rows; FAST: no x^(s+1) of this warp's pixels is zero
+  auto unit = [&](auto fast_tag, const T* st, int j, float& sm) {
+    constexpr bool FAST = decltype(fast_tag)::value;
+    float rs[W][2], rm[W][2], rq[W][2];   // horizontal windows of the last W rows (a ring)
+    float* const out = vp + (size_t)(j - 2) * (size_t)a.vstride + ox;
+#pragma unroll
+    for (int i = 0; i < EH; ++i) {
+      float e[W + 1], q[W + 1];   // Delta and r of this lane's columns and the W - 1 after them
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const float xn = to_f32(st[i * S::kBoxW + c]);
+        sm = fmaxf(sm, xn);
+        const float dn = fabsf(xn - x[i][c]);   // D^(s+1)
+        e[c] = fabsf(dn - d[i][c]);             // Delta
+        if (FAST) {
+          q[c] = __saturatef(e[c] * fabsf(rcp_approx(x[i][c])));
+        } else {
+          const float ref = SIGNED ? x[i][c] : fabsf(x[i][c]);
+          const float xh = (x[i][c] == 0.f) ? kGuardC : ref;   // Eq. 5
+          q[c] = fminf(__fdividef(e[c], xh), 1.f);             // Eq. 4
+        }
+        d[i][c] = dn;
+        x[i][c] = xn;
+      }
+#pragma unroll
+      for (int k = 2; k <= W; ++k) {
+        e[k] = __shfl_down_sync(0xffffffffu, e[k & 1], k >> 1);
+        q[k] = __shfl_down_sync(0xffffffffu, q[k & 1], k >> 1);
+      }
+      float pe[W], pq[W], m = 0.f;   // neighbouring pairs; the maximum of the shared columns
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        pe[k] = e[k] + e[k + 1];
+        pq[k] = q[k] + q[k + 1];
+      }
+#pragma unroll
+      for (int k = 1; k < W; ++k) m = fmaxf(m, e[k]);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        rs[i % W][c] = window_sum<W>(e, pe, c);
+        rq[i % W][c] = window_sum<W>(q, pq, c);
+        rm[i % W][c] = fmaxf(m, e[c ? W : 0]);
+      }
+      if (i >= W - 1) {
+        const int oy = i - (W - 1);        // output row, window rows oy .. i
+        const int y = y0 + oy;
+        float v[2];
+        const int nyw = min(y + H, a.ny - 1) - max(y - H, 0) + 1;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float S1 = 0.f, S2 = 0.f, S3 = 0.f;
+#pragma unroll
+          for (int k = 0; k < W; ++k) {
+            S1 += rs[(oy + k) % W][c];
+            S2 = fmaxf(S2, rm[(oy + k) % W][c]);
+            S3 += rq[(oy + k) % W][c];
+          }
+          // 1 / n_p^2: a constant inside the image, one division at its
+          // border (the tile march's form of the product)
+          constexpr float kInvFull = 1.f / (float)(W * W * W * W);
+          const int nxw = c ? nxw1 : nxw0;
+          float inv = kInvFull;
+          if (nyw != W || nxw != W) {
+            const float np = (float)(nyw * nxw);
+            inv = 1.f / (np * np);
+          }
+          v[c] = S1 * S2 * S3 * inv;
+          if (!isfinite(S1) || !isfinite(v[c])) v[c] = NAN;
+        }
+        if (y < a.ny) {
+          float* o = out + (size_t)y * a.nx;
+          if (pair) {
+            *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
+          } else {
+            if (out0) o[0] = v[0];
+            if (out1) o[1] = v[1];
+          }
+        }
+      }
+    }
+  };
+
+  for (int j = 0; j < L; ++j) {
+    const int stg = j % NS;
+    // one decision per warp, so that every lane takes part in the shuffles
+    const bool ok = __all_sync(0xffffffffu,
+                               mbar_wait_bounded(bar0 + 8 * stg, (uint32_t)((j / NS) & 1), deadline));
+    const T* st = reinterpret_cast<const T*>(smem + (size_t)stg * g.stage_bytes) + S::kOff +
+                  warp * S::kOWW + 2 * lane;
+    float sm = -INFINITY;
+    if (ok && j >= 2) {
+      float mn = INFINITY;
+      if (!SIGNED) {
+#pragma unroll
+        for (int i = 0; i < EH; ++i) mn = fminf(mn, fminf(fabsf(x[i][0]), fabsf(x[i][1])));
+      }
+      if (!SIGNED && __all_sync(0xffffffffu, mn != 0.f))
+        unit(std::true_type{}, st, j, sm);
+      else
+        unit(std::false_type{}, st, j, sm);
+    } else if (ok) {
+#pragma unroll
+      for (int i = 0; i < EH; ++i) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const float xn = to_f32(st[i * S::kBoxW + c]);
+          sm = fmaxf(sm, xn);
+          d[i][c] = fabsf(xn - x[i][c]);   // D^(0) once j == 1
+          x[i][c] = xn;
+        }
+      }
+    }
+    if (__syncthreads_or(!ok)) {
+      // a stage never completed: flag it, let copies in flight land (bounded)
+      if (tid == 0) {
+        atomicOr(a.status, kErrTimeout);
+        const uint64_t d2 = globaltimer_ns() + 1000000ull;
+        for (int jj = j; jj < L && jj < j + NS; ++jj)
+          mbar_wait_bounded(bar0 + 8 * (jj % NS), (uint32_t)((jj / NS) & 1), d2);
+      }
+      return;
+    }
+    mx = fmaxf(mx, sm);
+    if (smax) warp_max_to(sm, smax + j);
+    if (tid == 0 && j + NS < L) {
+      fence_proxy_async_smem();
+      mbar_expect_tx(bar0 + 8 * stg, box_bytes);
+      tma_load_3d(stage0 + stg * (uint32_t)g.stage_bytes, &tmap, xload, y0 - H,
+                  (z0 + j + NS) % a.nsnap, bar0 + 8 * stg);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0 && mx > -INFINITY) atomicMax(a.gmax, f32_key(mx));
+}
+
+template <int W>
+static void pair_geometry(int elem_bytes, SlideGeom* g) {
+  using S = PairShape<W>;
+  g->w = W;
+  g->h = S::kH;
+  g->OW = S::kOW;
+  g->OH = S::kRows;
+  g->EW = S::kOW + 2 * S::kH;
+  g->EH = S::kEH;
+  g->nseg = 0;
+  g->boxW = S::kBoxW;
+  g->threads = kShfWarps * 32;
+  g->stages = 3;
+  g->stage_bytes = ((size_t)S::kBoxW * S::kEH * elem_bytes + 127) / 128 * 128;
+  g->smem_bytes = g->stages * g->stage_bytes + 8 * g->stages;
+}
+
 bool slide_geometry(int w, int elem_bytes, SlideGeom* g) {
   if (w < 1 || (w & 1) == 0 || w > 31) return false;
   const int h = w / 2;
-  if (w >= 3 && w <= 9) {   // the shuffle kernel (nseg = 0 marks it)
+  if (w == 3) {
+    pair_geometry<3>(elem_bytes, g);
+    return true;
+  }
+  if (w == 5) {
+    pair_geometry<5>(elem_bytes, g);
+    return true;
+  }
+  if (w == 7 || w == 9) {   // the shuffle kernel (nseg = 0 marks both)
     const int OW = kShfWarps * (32 - 2 * h);
     const int EW = OW + 2 * h, EH = kShfRows + 2 * h;
     const int boxW = (EW + 7 + 7) / 8 * 8;
@@ -408,7 +655,7 @@ static cudaError_t launch_segments(K kern, const CUtensorMap* tmap, SlideArgs a,
 
 template <typename T, int W, bool SIGNED>
 static cudaError_t launch_shf_t(const CUtensorMap* tmap, const SlideArgs& a, cudaStream_t st) {
-  auto kern = k_slide_shf<T, W, SIGNED>;
+  auto kern = W <= 5 ? k_slide_pair<T, W <= 5 ? W : 5, SIGNED> : k_slide_shf<T, W <= 5 ? 7 : W, SIGNED>;
   static size_t configured = 0;
   if (a.g.smem_bytes > configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
