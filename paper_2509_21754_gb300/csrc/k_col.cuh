@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(ColShape<W>::kThreads) k_stack_col(const __gri
   using S = ColShape<W>;
   constexpr int BW = S::kBW, NT = S::kTBX * S::kTBY, RV = W * S::kV;
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ unsigned hold[S::kThreads / 32][kSnapChunk];
   const int NS = a.g.stages;
   float4* part = reinterpret_cast<float4*>(smem + (size_t)NS * a.g.stage_bytes);
   const uint32_t bar0 = smem_u32(part + 2 * NT * S::kStride);
@@ -154,7 +155,7 @@ __global__ void __launch_bounds__(ColShape<W>::kThreads) k_stack_col(const __gri
       return;
     }
     mx = fmaxf(mx, sm);
-    if (a.smax) warp_max_to(sm, a.smax + s0 + j);
+    if (a.smax) snap_max(hold, a.smax + s0, sm, j, L);
     if (tid == 0 && j + NS < L) {
       fence_proxy_async_smem();
       mbar_expect_tx(bar0 + 8 * stg, box_bytes);
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(ColShape<W>::kThreads) k_stack_col(const __gri
       }
     }
   }
-  warp_max_to(mx, a.gmax);   // (whole warps: kThreads is a multiple of 32)
+  warp_raise_max(mx, a.gmax);   // (whole warps: kThreads is a multiple of 32)
 }
 
 template <typename T, int W, bool SIGNED>

@@ -1031,10 +1031,10 @@ __global__ void __launch_bounds__(1024) k_blk_scan(int nblk, int64_t nblocks, Bl
 // Small maps: everything after the labelling in one CTA, whose barriers cost
 // a fraction of the launches they replace (the full labelling of blocks of
 // many runs, unions, peaks, row counts, their scan and the check: seven).
-// Bounded by kTailBlocks blocks and kTailRows rows, what 32 warps walk in about
-// the time of the launches.
+// Bounded by kTailBlocks blocks, four per warp (256 took 39 us against about 28
+// in launches of their own), and by the rows whose counts fit in shared memory.
 constexpr int kTailThreads = 1024;
-constexpr int64_t kTailBlocks = 256;
+constexpr int64_t kTailBlocks = 128;
 constexpr int64_t kTailRows = 4096;
 
 __global__ void __launch_bounds__(kTailThreads) k_blk_tail(const float* __restrict__ vals,
@@ -1046,8 +1046,9 @@ __global__ void __launch_bounds__(kTailThreads) k_blk_tail(const float* __restri
   __shared__ union {
     BlkShared<kTailThreads, kBlkMaxRuns> label;
     long long scan[1024];
+    int rows[kTailRows];
   } sh;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5;
   if (__syncthreads_or(tid < nblocks && b.bstat[tid].w)) {
     const int nbx = (Tx + kBlkX - 1) / kBlkX, nby = (Ty + kBlkY - 1) / kBlkY;
     for (int k = 0; k < nblocks; ++k) {
@@ -1063,26 +1064,35 @@ __global__ void __launch_bounds__(kTailThreads) k_blk_tail(const float* __restri
   __syncthreads();
   blk_mark(Tx, Ty, nblocks, b, warp, kTailThreads / 32);
   __syncthreads();
-  // a thread per tile row (the bits set above are past the L1 cache)
-  for (int64_t r = tid; r < nrows; r += kTailThreads) {
-    const uint32_t* row = b.pbits + (size_t)r * b.words;
-    int c = 0;
-    for (int w = 0; w < b.words; ++w) c += __popc(__ldcg(row + w));
-    b.rowcnt[r] = c;
+  // the peaks of every tile row: a thread per bitmap word (the bits set above
+  // are past the L1 cache)
+  for (int r = tid; r < nrows; r += kTailThreads) sh.rows[r] = 0;
+  __syncthreads();
+  const int nwords = (int)nrows * b.words;
+  for (int i0 = tid; i0 < nwords; i0 += 8 * kTailThreads) {
+    uint32_t w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int i = i0 + k * kTailThreads;
+      w[k] = i < nwords ? __ldcg(b.pbits + i) : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (w[k]) atomicAdd(&sh.rows[(i0 + k * kTailThreads) / b.words], __popc(w[k]));
   }
   __syncthreads();
+  for (int r = tid; r < nrows; r += kTailThreads) b.rowcnt[r] = sh.rows[r];
   const int ncta = (int)((nrows + kRowsPerCta - 1) / kRowsPerCta);
   for (int i = tid; i < ncta; i += kTailThreads) {
     int c = 0;
     for (int64_t r = (int64_t)i * kRowsPerCta; r < nrows && r < (int64_t)(i + 1) * kRowsPerCta; ++r)
-      c += b.rowcnt[r];
+      c += sh.rows[r];
     b.blkcnt[i] = c;
   }
   __syncthreads();
   scan_counts(ncta, b.blkcnt, b.blkoff, &b.counters[2], cap, status, (unsigned*)nullptr, sh.scan);
   __syncthreads();
   blk_check(nblocks, b, cap, status, want, sh.scan);
-  (void)lane;
 }
 
 static int block_words(int Tx) { return (Tx + 31) / 32; }

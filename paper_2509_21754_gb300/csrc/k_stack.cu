@@ -44,6 +44,7 @@ template <typename T, int R, bool SIGNED>
 __global__ void __launch_bounds__(kStackMaxThreads) k_stack_tile(const __grid_constant__ CUtensorMap tmap,
                                                      const StackArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ unsigned hold[kStackMaxThreads / 32][kSnapChunk];
   const StackGeom& g = a.g;
   const int NS = g.stages;
   float4* part = reinterpret_cast<float4*>(smem + (size_t)NS * g.stage_bytes);
@@ -155,7 +156,10 @@ __global__ void __launch_bounds__(kStackMaxThreads) k_stack_tile(const __grid_co
     }
     mx = fmaxf(mx, sm);
     const bool full_warp = (tid >> 5) < (g.threads >> 5);
-    if (smax) max_to(sm, smax + j, full_warp);
+    if (smax) {
+      if (full_warp) snap_max(hold, smax, sm, j, L);
+      else max_to(sm, smax + j, false);
+    }
     if (tid == 0 && j + NS < L) {
       fence_proxy_async_smem();
       mbar_expect_tx(bar0 + 8 * stg, box_bytes);
@@ -256,6 +260,7 @@ struct FieldView {
   float* vp;
   uint8_t* arg;
   unsigned* smax;
+  unsigned (*hold)[kSnapChunk];   // snap_max's notes (shared memory)
   unsigned* status;
 };
 
@@ -533,7 +538,7 @@ __device__ __forceinline__ bool march_small(const CUtensorMap* tmap, const Field
     float sm = -INFINITY;
     key_load<W, W>(f.key, f.kpitch, x0 + tbx * W, y0 + tb * W, f.nx, f.ny, xa, sm);
     mx = fmaxf(mx, sm);
-    if (f.smax) warp_max_to(sm, f.smax);
+    if (f.smax) snap_max(f.hold, f.smax, sm, 0, L);
   }
 #pragma unroll
   for (int j = j0; j < 2; ++j) {
@@ -546,7 +551,7 @@ __device__ __forceinline__ bool march_small(const CUtensorMap* tmap, const Field
     }
     if (!ring_release(rg, ok, tmap, f.status, j, L, x0, y0, f.zrot, f.ring)) return false;
     mx = fmaxf(mx, sm);
-    if (f.smax) warp_max_to(sm, f.smax + j);
+    if (f.smax) snap_max(f.hold, f.smax, sm, j, L);
   }
   // After the prologue x^(1) and D^(0) are in (xb, db) when L > 1.
   auto unit = [&](int j, const float (&xp)[N], const float (&dp)[N], float (&xn)[N],
@@ -558,7 +563,7 @@ __device__ __forceinline__ bool march_small(const CUtensorMap* tmap, const Field
     if (ok) tile_unit<T, W, 32 * W, SIGNED, DELTA, true>(stage(), xp, dp, xn, dn, sm, s1, s2, s3, am);
     if (!ring_release(rg, ok, tmap, f.status, j, L, x0, y0, f.zrot, f.ring)) return false;
     mx = fmaxf(mx, sm);
-    if (f.smax) warp_max_to(sm, f.smax + j);
+    if (f.smax) snap_max(f.hold, f.smax, sm, j, L);
     if (live) {
       float v = s1 * s2 * s3 * inv_n2;
       if (!isfinite(s1) || !isfinite(v)) v = NAN;
@@ -574,20 +579,16 @@ __device__ __forceinline__ bool march_small(const CUtensorMap* tmap, const Field
   return true;
 }
 
-__device__ __forceinline__ void block_max_to(float mx, unsigned* gmax) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0 && mx > -INFINITY) atomicMax(gmax, f32_key(mx));
-}
-
 template <typename T, int W, bool SIGNED, bool DELTA>
 __global__ void __launch_bounds__(kSmallMaxThreads) k_stack_small(const __grid_constant__ CUtensorMap tmap,
                                                                const StackArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ unsigned hold[kSmallMaxThreads / 32][kSnapChunk];
   if (threadIdx.x == 0) prefetch_tmap(&tmap);
   Ring rg;
   ring_init(rg, smem, a.g, (int)sizeof(T));
   FieldView f;
+  f.hold = hold;
   const int s0 = blockIdx.z * a.seg_units;   // first unit of the segment
   const size_t v0 = (size_t)s0 * (size_t)a.vstride;
   f.nx = a.nx;
@@ -609,7 +610,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_stack_small(const __grid_c
   if (!march_small<T, W, SIGNED, DELTA>(&tmap, f, blockIdx.x, blockIdx.y, a.g.TBY, rg, smem,
                                         deadline, mx))
     return;
-  block_max_to(mx, a.gmax);
+  warp_raise_max(mx, a.gmax);
 }
 
 // Windows that are multiples of 4 up to 64 (8, 16, 32, 64): the thread-per-tile
@@ -632,7 +633,8 @@ __device__ __forceinline__ size_t sub_part_offset(const StackGeom& g) {
 
 template <typename T, bool SIGNED, bool DELTA>
 __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackArgs& a, Ring& rg,
-                                          unsigned char* smem, uint64_t deadline, float& mx) {
+                                          unsigned char* smem, unsigned (*hold)[kSnapChunk],
+                                          uint64_t deadline, float& mx) {
   constexpr int N = 16;
   const StackGeom& g = a.g;
   const int w = g.w, gl = w / 4;             // lanes (and warps) per tile side
@@ -674,7 +676,7 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
     float sm = -INFINITY;
     key_load<4, 4>(a.key, a.kpitch, x0 + lane * 4, y0 + warp * 4, a.nx, a.ny, xa, sm);
     mx = fmaxf(mx, sm);
-    if (smax) warp_max_to(sm, smax);
+    if (smax) snap_max(hold, smax, sm, 0, L);
   }
 #pragma unroll
   for (int j = j0; j < 2; ++j) {
@@ -687,7 +689,7 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
     }
     if (!ring_release(rg, ok, tmap, a.status, j, L, x0, y0, z0, a.nsnap)) return false;
     mx = fmaxf(mx, sm);
-    if (smax) warp_max_to(sm, smax + j);
+    if (smax) snap_max(hold, smax, sm, j, L);
   }
   auto unit = [&](int j, const float (&xp)[N], const float (&dp)[N], float (&xn)[N],
                   float (&dn)[N]) -> bool {
@@ -705,7 +707,7 @@ __device__ __forceinline__ bool march_sub(const CUtensorMap* tmap, const StackAr
     if (lane % gl == 0) pp[warp * g.TBX + lane / gl] = make_float4(s1, s2, s3, 0.f);
     if (!ring_release(rg, ok, tmap, a.status, j, L, x0, y0, z0, a.nsnap)) return false;
     mx = fmaxf(mx, sm);
-    if (smax) warp_max_to(sm, smax + j);
+    if (smax) snap_max(hold, smax, sm, j, L);
     if (rlive) {
       float S1 = 0.f, S2 = 0.f, S3 = 0.f;
       for (int k = 0; k < gl; ++k) {
@@ -734,13 +736,14 @@ template <typename T, bool SIGNED, int MAXT, bool DELTA>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) k_stack_sub(const __grid_constant__ CUtensorMap tmap,
                                                                 const StackArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ unsigned hold[MAXT / 32][kSnapChunk];
   if (threadIdx.x == 0) prefetch_tmap(&tmap);
   Ring rg;
   ring_init(rg, smem, a.g, (int)sizeof(T));
   float mx = -INFINITY;
   const uint64_t deadline = globaltimer_ns() + a.timeout_ns;
-  if (!march_sub<T, SIGNED, DELTA>(&tmap, a, rg, smem, deadline, mx)) return;
-  block_max_to(mx, a.gmax);
+  if (!march_sub<T, SIGNED, DELTA>(&tmap, a, rg, smem, hold, deadline, mx)) return;
+  warp_raise_max(mx, a.gmax);
 }
 
 // Persistent form over many fields (one launch for a whole batch): each CTA
@@ -748,7 +751,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 2 : 1) k_stack_sub(const _
 // fields are ordered largest first.  Every field has its own TMA descriptor in
 // global memory; the ring carries over between items.
 template <typename T, int W, bool SIGNED>
-__global__ void __launch_bounds__(kSmallMaxThreads) k_stack_multi(const FieldDesc* __restrict__ fields,
+__global__ void __launch_bounds__(kSmallMaxThreads, W == 5 ? 2 : 1) k_stack_multi(const FieldDesc* __restrict__ fields,
                                                                int nfields, int64_t nitems,
                                                                unsigned long long* counter,
                                                                const StackGeom g,
@@ -756,6 +759,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_stack_multi(const FieldDes
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ long long s_item;
   __shared__ int s_field;
+  __shared__ unsigned hold[kSmallMaxThreads / 32][kSnapChunk];
   Ring rg;
   ring_init(rg, smem, g, (int)sizeof(T));
   const uint64_t deadline = globaltimer_ns() + timeout_ns;
@@ -778,6 +782,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_stack_multi(const FieldDes
     const FieldDesc& d = fields[fi];
     const long long b = it - d.item0;
     FieldView f;
+    f.hold = hold;
     f.nx = d.nx;
     f.ny = d.ny;
     f.L = f.ring = d.L;
@@ -793,7 +798,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_stack_multi(const FieldDes
     if (!march_small<T, W, SIGNED>(&d.tmap, f, (int)(b % d.gridX), (int)(b / d.gridX), g.TBY, rg,
                                    smem, deadline, mx))
       return;
-    block_max_to(mx, d.gmax);
+    warp_raise_max(mx, d.gmax);
   }
 }
 

@@ -15,15 +15,50 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
-// Maximum of v over the calling threads into *key.  Full warps reduce with
-// shuffles first; the threads of a trailing partial warp (a block size that is
-// not a multiple of 32) go straight to the atomic.
+// Maxima of a march.  Every warp of every CTA has one for the stack and, with
+// the running M, one per snapshot, and all CTAs are at about the same
+// snapshot, so that an atomic each would queue up at one address (64 x 4096^2,
+// w = 5, running M: 1.4 M of them, march 2.12 ms).  The words only grow during a
+// launch, so a warp looks first (past the L1 cache) and leaves a maximum that is
+// no larger than what is there: 0.71 ms, the march without running M 0.69.  (The
+// sliding march spends far longer between snapshots and keeps its atomics.)
+__device__ __forceinline__ void raise_max(unsigned* word, unsigned key) {
+  if (key > __ldcg(word)) atomicMax(word, key);
+}
+
+// This warp's maximum of v into *key (every lane calls it; -inf is skipped).
+__device__ __forceinline__ void warp_raise_max(float v, unsigned* key) {
+  const unsigned k = __reduce_max_sync(0xffffffffu, v > -INFINITY ? f32_key(v) : 0u);
+  if ((threadIdx.x & 31) == 0 && k) raise_max(key, k);
+}
+
+// The snapshots' maxima: lane 0 notes each in shared memory, and the warp looks
+// at sixteen words together.  put() is called by every lane of a full warp for
+// j = 0 .. L - 1 in order.
+constexpr int kSnapChunk = 16;
+__device__ __forceinline__ void snap_max(unsigned (*hold)[kSnapChunk], unsigned* smax, float v, int j,
+                                         int L) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned k = __reduce_max_sync(0xffffffffu, v > -INFINITY ? f32_key(v) : 0u);
+  if (lane == 0) hold[warp][j % kSnapChunk] = k;
+  if (j % kSnapChunk != kSnapChunk - 1 && j != L - 1) return;
+  __syncwarp();
+  if (lane <= j % kSnapChunk) {
+    const unsigned h = hold[warp][lane];
+    if (h) raise_max(smax + (j - j % kSnapChunk) + lane, h);
+  }
+  __syncwarp();
+}
+
+// Maximum of v over the calling threads into *key.  Full warps reduce first;
+// the threads of a trailing partial warp (a block size that is not a multiple
+// of 32) look for themselves.
 __device__ __forceinline__ void max_to(float v, unsigned* key, bool full_warp) {
   if (full_warp) {
-    warp_max_to(v, key);
+    warp_raise_max(v, key);
     return;
   }
-  if (v > -INFINITY) atomicMax(key, f32_key(v));
+  if (v > -INFINITY) raise_max(key, f32_key(v));
 }
 
 // The sums and maximum of one tile's PER column partials, added in the order
