@@ -125,72 +125,74 @@ __global__ void __launch_bounds__(kDftThreads) k_dft_short(const float* __restri
     tws[i] = tw[(size_t)k * H + q];
   }
   __syncthreads();
-  const int64_t t = (int64_t)blockIdx.x * kDftThreads + threadIdx.x;
-  if (t >= T) return;
-  float s = 0.f, comp = 0.f;
-  bool ok = true;
-  float* my = ys + threadIdx.x;
-  for (int q = 0; q < n; ++q) {
-    const float v = wts ? vp[(size_t)q * vs + t] * wts[q] : vp[(size_t)q * vs + t];
-    ok = ok && isfinite(v);
-    my[q * kDftThreads] = v;
-    const float y = v - comp;
-    const float u = s + y;
-    comp = (u - s) - y;
-    s = u;
-  }
-  if (!ok) {
-    eta[t] = NAN;
-    bin[t] = -1;
-    return;
-  }
-  const float mean = s / (float)n;
-  const bool even = (n & 1) == 0;
-  const float y0 = my[0] - mean;
-  const float ymid = even ? my[(n / 2) * kDftThreads] - mean : 0.f;
-  float re[KMAX], im[KMAX];
-#pragma unroll
-  for (int k = 0; k < KMAX; ++k) {
-    re[k] = y0 + ((even && ((k + 1) & 1)) ? -ymid : ymid);
-    im[k] = 0.f;
-  }
-  for (int q = 1; q <= H; ++q) {
-    const float a = my[q * kDftThreads] - mean;
-    const float b = my[(n - q) * kDftThreads] - mean;
-    const float e = a + b, o = a - b;
-    const float2* row = tws + (q - 1) * K;
-#pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-      if (k < K) {
-        const float2 cs = row[k];
-        re[k] = fmaf(e, cs.x, re[k]);
-        im[k] = fmaf(o, cs.y, im[k]);
-      }
+  // (a CTA takes many groups of tiles: its twiddle table costs more than a group)
+  for (int64_t t = (int64_t)blockIdx.x * kDftThreads + threadIdx.x; t < T;
+       t += (int64_t)gridDim.x * kDftThreads) {
+    float s = 0.f, comp = 0.f;
+    bool ok = true;
+    float* my = ys + threadIdx.x;
+    for (int q = 0; q < n; ++q) {
+      const float v = wts ? vp[(size_t)q * vs + t] * wts[q] : vp[(size_t)q * vs + t];
+      ok = ok && isfinite(v);
+      my[q * kDftThreads] = v;
+      const float y = v - comp;
+      const float u = s + y;
+      comp = (u - s) - y;
+      s = u;
     }
-  }
-  float best = -1.f;
-  int bk = 1;
-  if constexpr (HARM) {
-    // the series is spent: its column holds the magnitudes for the harmonic sum
-#pragma unroll
-    for (int k = 0; k < KMAX; ++k)
-      if (k < K) my[k * kDftThreads] = sqrtf(re[k] * re[k] + im[k] * im[k]);
-    harmonic_best(my, kDftThreads, K, hmax, best, bk);
-    eta[t] = best;
-    bin[t] = bk;
-  } else {
+    if (!ok) {
+      eta[t] = NAN;
+      bin[t] = -1;
+      continue;
+    }
+    const float mean = s / (float)n;
+    const bool even = (n & 1) == 0;
+    const float y0 = my[0] - mean;
+    const float ymid = even ? my[(n / 2) * kDftThreads] - mean : 0.f;
+    float re[KMAX], im[KMAX];
 #pragma unroll
     for (int k = 0; k < KMAX; ++k) {
-      if (k < K) {
-        const float m2 = re[k] * re[k] + im[k] * im[k];
-        if (m2 > best) {
-          best = m2;
-          bk = k + 1;
+      re[k] = y0 + ((even && ((k + 1) & 1)) ? -ymid : ymid);
+      im[k] = 0.f;
+    }
+    for (int q = 1; q <= H; ++q) {
+      const float a = my[q * kDftThreads] - mean;
+      const float b = my[(n - q) * kDftThreads] - mean;
+      const float e = a + b, o = a - b;
+      const float2* row = tws + (q - 1) * K;
+#pragma unroll
+      for (int k = 0; k < KMAX; ++k) {
+        if (k < K) {
+          const float2 cs = row[k];
+          re[k] = fmaf(e, cs.x, re[k]);
+          im[k] = fmaf(o, cs.y, im[k]);
         }
       }
     }
-    eta[t] = sqrtf(best);
-    bin[t] = bk;
+    float best = -1.f;
+    int bk = 1;
+    if constexpr (HARM) {
+      // the series is spent: its column holds the magnitudes for the harmonic sum
+#pragma unroll
+      for (int k = 0; k < KMAX; ++k)
+        if (k < K) my[k * kDftThreads] = sqrtf(re[k] * re[k] + im[k] * im[k]);
+      harmonic_best(my, kDftThreads, K, hmax, best, bk);
+      eta[t] = best;
+      bin[t] = bk;
+    } else {
+#pragma unroll
+      for (int k = 0; k < KMAX; ++k) {
+        if (k < K) {
+          const float m2 = re[k] * re[k] + im[k] * im[k];
+          if (m2 > best) {
+            best = m2;
+            bk = k + 1;
+          }
+        }
+      }
+      eta[t] = sqrtf(best);
+      bin[t] = bk;
+    }
   }
 }
 
@@ -228,107 +230,110 @@ __global__ void __launch_bounds__(kDftThreads) k_dft_even(const float* __restric
   }
   for (int k = threadIdx.x; k < m; k += blockDim.x) tk[k] = ang(k);
   __syncthreads();
-  const int64_t t = (int64_t)blockIdx.x * kDftThreads + threadIdx.x;
-  if (t >= T) return;
   float* my = ys + threadIdx.x;
-  // the series arrives by asynchronous global -> shared copies, all n of a
-  // thread in flight at once (coalesced over the CTA's tiles)
-  for (int q = 0; q < n; ++q) {
-    const uint32_t dst = smem_u32(my + q * kDftThreads);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst),
-                 "l"(vp + (size_t)q * vs + t)
-                 : "memory");
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  float sum = 0.f;
-  bool ok = true;
-  for (int q = 0; q < n; ++q) {
-    float v = my[q * kDftThreads];
-    if (wts) {
-      v *= wts[q];
-      my[q * kDftThreads] = v;
+  // (a CTA takes many groups of tiles: its twiddle tables cost more than a group
+  // of short series; a thread's column of ys is its own, so no barrier is needed)
+  for (int64_t t = (int64_t)blockIdx.x * kDftThreads + threadIdx.x; t < T;
+       t += (int64_t)gridDim.x * kDftThreads) {
+    // the series arrives by asynchronous global -> shared copies, all n of a
+    // thread in flight at once (coalesced over the CTA's tiles)
+    for (int q = 0; q < n; ++q) {
+      const uint32_t dst = smem_u32(my + q * kDftThreads);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst),
+                   "l"(vp + (size_t)q * vs + t)
+                   : "memory");
     }
-    ok = ok && isfinite(v);
-    sum += v;
-  }
-  if (!ok) {
-    eta[t] = NAN;
-    bin[t] = -1;
-    return;
-  }
-  const float mean = sum / (float)n;
-  auto ye = [&](int j) { return my[(2 * j) * kDftThreads] - mean; };       // y_(2j)
-  auto yo = [&](int j) { return my[(2 * j + 1) * kDftThreads] - mean; };   // y_(2j+1)
-  const float ye0 = ye(0), yo0 = yo(0);
-  const bool meven = (m & 1) == 0;
-  const float yem = meven ? ye(m / 2) : 0.f, yom = meven ? yo(m / 2) : 0.f;
-  float E0 = ye0 + yem, O0 = yo0 + yom;   // bin 0 of each half
-  float er[KH], es[KH], orr[KH], os[KH];  // bins 1..K: real parts, and the sums of
-                                          // the odd folds times sin (imag = -that)
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    float sum = 0.f;
+    bool ok = true;
+    for (int q = 0; q < n; ++q) {
+      float v = my[q * kDftThreads];
+      if (wts) {
+        v *= wts[q];
+        my[q * kDftThreads] = v;
+      }
+      ok = ok && isfinite(v);
+      sum += v;
+    }
+    if (!ok) {
+      eta[t] = NAN;
+      bin[t] = -1;
+      continue;
+    }
+    const float mean = sum / (float)n;
+    auto ye = [&](int j) { return my[(2 * j) * kDftThreads] - mean; };       // y_(2j)
+    auto yo = [&](int j) { return my[(2 * j + 1) * kDftThreads] - mean; };   // y_(2j+1)
+    const float ye0 = ye(0), yo0 = yo(0);
+    const bool meven = (m & 1) == 0;
+    const float yem = meven ? ye(m / 2) : 0.f, yom = meven ? yo(m / 2) : 0.f;
+    float E0 = ye0 + yem, O0 = yo0 + yom;   // bin 0 of each half
+    float er[KH], es[KH], orr[KH], os[KH];  // bins 1..K: real parts, and the sums of
+                                            // the odd folds times sin (imag = -that)
 #pragma unroll
-  for (int k = 0; k < KH; ++k) {
-    const float sg = ((k + 1) & 1) ? -1.f : 1.f;   // (-1)^(k+1)
-    er[k] = ye0 + sg * yem;
-    orr[k] = yo0 + sg * yom;
-    es[k] = 0.f;
-    os[k] = 0.f;
-  }
-  for (int j = 1; j <= Hm; ++j) {
-    const float a = ye(j), b = ye(m - j), c = yo(j), d = yo(m - j);
-    const float ee = a + b, eo = a - b, oe = c + d, oo = c - d;
-    E0 += ee;
-    O0 += oe;
-    const float2* row = th + (j - 1) * K;
+    for (int k = 0; k < KH; ++k) {
+      const float sg = ((k + 1) & 1) ? -1.f : 1.f;   // (-1)^(k+1)
+      er[k] = ye0 + sg * yem;
+      orr[k] = yo0 + sg * yom;
+      es[k] = 0.f;
+      os[k] = 0.f;
+    }
+    for (int j = 1; j <= Hm; ++j) {
+      const float a = ye(j), b = ye(m - j), c = yo(j), d = yo(m - j);
+      const float ee = a + b, eo = a - b, oe = c + d, oo = c - d;
+      E0 += ee;
+      O0 += oe;
+      const float2* row = th + (j - 1) * K;
+#pragma unroll
+      for (int k = 0; k < KH; ++k) {
+        if (k < K) {
+          const float2 w = row[k];
+          er[k] = fmaf(ee, w.x, er[k]);
+          es[k] = fmaf(eo, w.y, es[k]);
+          orr[k] = fmaf(oe, w.x, orr[k]);
+          os[k] = fmaf(oo, w.y, os[k]);
+        }
+      }
+    }
+    // X_k = E_k + W^k O_k, W^k = (c, -s):  Re = Er + c Or + s Oi,  Im = Ei + c Oi - s Or
+    float best = -1.f;
+    int bk = 1;
+    // with harmonic summing the spent series column collects |X_k| at row k - 1
+    constexpr bool harm = HARM;
+    auto take = [&](int k, float Er, float Ei, float Or, float Oi) {
+      const float2 w = tk[k];
+      const float re = Er + w.x * Or + w.y * Oi;
+      const float im = Ei + w.x * Oi - w.y * Or;
+      const float m2 = re * re + im * im;
+      if constexpr (harm) my[(k - 1) * kDftThreads] = sqrtf(m2);
+      if (m2 > best || (m2 == best && k < bk)) {
+        best = m2;
+        bk = k;
+      }
+    };
 #pragma unroll
     for (int k = 0; k < KH; ++k) {
       if (k < K) {
-        const float2 w = row[k];
-        er[k] = fmaf(ee, w.x, er[k]);
-        es[k] = fmaf(eo, w.y, es[k]);
-        orr[k] = fmaf(oe, w.x, orr[k]);
-        os[k] = fmaf(oo, w.y, os[k]);
+        take(k + 1, er[k], -es[k], orr[k], -os[k]);                    // bin k+1
+        if (m - (k + 1) > K) take(m - (k + 1), er[k], es[k], orr[k], os[k]);   // its mirror
       }
     }
-  }
-  // X_k = E_k + W^k O_k, W^k = (c, -s):  Re = Er + c Or + s Oi,  Im = Ei + c Oi - s Or
-  float best = -1.f;
-  int bk = 1;
-  // with harmonic summing the spent series column collects |X_k| at row k - 1
-  constexpr bool harm = HARM;
-  auto take = [&](int k, float Er, float Ei, float Or, float Oi) {
-    const float2 w = tk[k];
-    const float re = Er + w.x * Or + w.y * Oi;
-    const float im = Ei + w.x * Oi - w.y * Or;
-    const float m2 = re * re + im * im;
-    if constexpr (harm) my[(k - 1) * kDftThreads] = sqrtf(m2);
-    if (m2 > best || (m2 == best && k < bk)) {
-      best = m2;
-      bk = k;
+    {
+      const float x = E0 - O0;   // bin m
+      const float m2 = x * x;
+      if constexpr (HARM) my[(m - 1) * kDftThreads] = fabsf(x);
+      if (m2 > best || (m2 == best && m < bk)) {
+        best = m2;
+        bk = m;
+      }
     }
-  };
-#pragma unroll
-  for (int k = 0; k < KH; ++k) {
-    if (k < K) {
-      take(k + 1, er[k], -es[k], orr[k], -os[k]);                    // bin k+1
-      if (m - (k + 1) > K) take(m - (k + 1), er[k], es[k], orr[k], os[k]);   // its mirror
+    if constexpr (HARM) {
+      harmonic_best(my, kDftThreads, m, hmax, best, bk);
+      eta[t] = best;
+      bin[t] = bk;
+    } else {
+      eta[t] = sqrtf(best);
+      bin[t] = bk;
     }
-  }
-  {
-    const float x = E0 - O0;   // bin m
-    const float m2 = x * x;
-    if constexpr (HARM) my[(m - 1) * kDftThreads] = fabsf(x);
-    if (m2 > best || (m2 == best && m < bk)) {
-      best = m2;
-      bk = m;
-    }
-  }
-  if constexpr (HARM) {
-    harmonic_best(my, kDftThreads, m, hmax, best, bk);
-    eta[t] = best;
-    bin[t] = bk;
-  } else {
-    eta[t] = sqrtf(best);
-    bin[t] = bk;
   }
 }
 
@@ -982,6 +987,18 @@ cudaError_t launch_spectrum(const float* vp, int n, int64_t T, int64_t vs,
   return launch_spectrum_method(vp, n, T, vs, twiddle, wts, hmax, eta, bin, kSpectrumAuto, st);
 }
 
+// CTAs of the short kernels.  Up to 32 points: what shared memory (sm bytes
+// each) lets be resident, at most 16 per SM, so that each walks several groups of
+// tiles and builds its tables once (24.2 M series of 6 points 655 -> 529 us, and
+// 250 with the bins' registers cut to the four there are); longer series
+// hide the tables behind their own sums, and a CTA per group balances better
+// (672,400 of 62 points: 77 us, 85 as a loop).
+static unsigned short_grid(int n, int64_t blocks, size_t sm) {
+  if (n > 32) return (unsigned)blocks;
+  const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(16, (int64_t)(227 * 1024 / (sm + 1024))));
+  return (unsigned)std::min<int64_t>(blocks, 152 * per_sm);
+}
+
 // Every length that is not the radix kernel's; `direct`: without the splitting.
 static cudaError_t launch_odd_length(const float* vp, int n, int64_t T, int64_t vs,
                                      const float2* twiddle, const float* wts, int hmax, float* eta,
@@ -993,8 +1010,9 @@ static cudaError_t launch_odd_length(const float* vp, int n, int64_t T, int64_t 
     const int m = n / 2, Hm = (m - 1) / 2, Kh = m / 2;
     const size_t sm = (size_t)(Hm > 0 ? Hm * Kh : 0) * sizeof(float2) + (size_t)m * sizeof(float2) +
                       (size_t)n * kDftThreads * sizeof(float);
-    auto kern = harm ? k_dft_even<16, true> : k_dft_even<16, false>;
-    kern<<<(unsigned)blocks, kDftThreads, sm, st>>>(vp, n, T, vs, twiddle, wts, hmax, eta, bin);
+    auto kern = Kh <= 4 ? (harm ? k_dft_even<4, true> : k_dft_even<4, false>)
+                        : (harm ? k_dft_even<16, true> : k_dft_even<16, false>);
+    kern<<<short_grid(n, blocks, sm), kDftThreads, sm, st>>>(vp, n, T, vs, twiddle, wts, hmax, eta, bin);
     count_launches(1);
     return cudaGetLastError();
   }
@@ -1002,7 +1020,7 @@ static cudaError_t launch_odd_length(const float* vp, int n, int64_t T, int64_t 
     const size_t sm = (size_t)H * K * sizeof(float2) + (size_t)n * kDftThreads * sizeof(float);
     auto kern = K <= 16 ? (harm ? k_dft_short<16, true> : k_dft_short<16, false>)
                         : (harm ? k_dft_short<32, true> : k_dft_short<32, false>);
-    kern<<<(unsigned)blocks, kDftThreads, sm, st>>>(vp, n, T, vs, twiddle, wts, hmax, eta, bin);
+    kern<<<short_grid(n, blocks, sm), kDftThreads, sm, st>>>(vp, n, T, vs, twiddle, wts, hmax, eta, bin);
     count_launches(1);
     return cudaGetLastError();
   }
