@@ -250,7 +250,8 @@ FITRIG_API int fitrig_push_snapshot(fitrig_plan_t plan, const void* data, int dt
  * holds ny rows of `row_pitch_elems` elements (0 means nx).  A host buffer is
  * borrowed until the call returns (one synchronisation at the end, not one per
  * snapshot).  When the snapshots follow each other without a gap in the storage
- * type, the block goes as one transfer of count * ny rows.  With FITRIG_OPT_ACCUMULATE = K they are raw snapshots (K per slot).
+ * type, the block goes as one transfer of count * ny rows.  With
+ * FITRIG_OPT_ACCUMULATE = K they are raw snapshots (K per slot).
  * EINVAL for count < 0 or a stride shorter than one snapshot; ESTATE (nothing
  * pushed) when they do not fit into the remaining slots.
  */
