@@ -656,10 +656,11 @@ __global__ void __launch_bounds__(kClusterThreads, 4) k_medmad_cluster(const flo
 // One thread-block cluster of 8 CTAs per group, for maps of moderate size.
 // The exact lower median and MAD are found with two passes over the map
 // instead of one pass per radix digit:
-//   * every CTA bins the same fixed, evenly spread sample of the group (up to
-//     288 runs of 32 consecutive values) twice -- over the sample's key range,
-//     then over the bins holding the targets -- and so finds the same sample
-//     quantiles A <= B at ranks 1/2 -+ delta of the sample;
+//   * a fixed, evenly spread sample of the group (up to 576 runs of 32
+//     consecutive values, an eighth of the runs per CTA, kept in shared memory
+//     for both brackets) is binned twice -- over the sample's key range, then
+//     over the bins holding the targets, the histograms summed over the cluster
+//     -- which gives the sample quantiles A <= B at ranks 1/2 -+ delta;
 //   * one pass, each CTA over its share, counts the finite values and the
 //     keys below A, and copies the keys in [A, B] into its shared memory;
 //   * if the median's rank lies among the copies of the cluster, rounds of
@@ -673,11 +674,19 @@ __global__ void __launch_bounds__(kClusterThreads, 4) k_medmad_cluster(const flo
 // sample only decides how much is copied.  When a bracket misses its rank or
 // the copies do not fit, the group is marked (scale -1) and the multi-pass
 // cluster kernel above, launched next, computes it instead.
+// What bounds it: with four CTAs per SM in one wave, the phases' latencies.  When
+// every CTA gathered and binned the whole sample (288 runs) for itself, twice,
+// the sample took 13 to 20 us and its quantiles 11 to 24 us per bracket, of 200
+// for 62 maps of 672,400 values (the passes 45 and 33, the selects 10 and 8);
+// shared out over the cluster the whole takes 209 -> 171 us, with twice the
+// sample and so 30% fewer copies.
 constexpr int kFastThreads = 256;
 constexpr int kFastWarps = kFastThreads / 32;
 constexpr int kFastBins = 2048;                    // 64 coarse bins of 32
-constexpr int kFastPool = 9 * 1024;                // keys copied per CTA
-constexpr int kFastRuns = kFastPool / 32;          // sample runs of 32 values
+constexpr int kFastPool = 6912;                    // keys copied per CTA
+constexpr int kFastRuns = 576;                     // sample runs of 32 values
+constexpr int kFastSlots = kFastRuns / kClusterCtas * 32;   // a CTA's sample values
+static_assert(kFastSlots % kFastThreads == 0, "whole rounds of sample values");
 constexpr int64_t kFastMaxPerGroup = 2 << 20;
 constexpr uint32_t kFinLo = 0x00800000u;   // key of -FLT_MAX
 constexpr uint32_t kFinHi = 0xff7fffffu;   // key of +FLT_MAX
@@ -691,7 +700,7 @@ __device__ __forceinline__ bool finite_bits(float x) {
 
 struct FastFind {
   unsigned long long below;   // keys before the bin
-  unsigned bin, size;
+  unsigned bin;
 };
 
 __device__ __forceinline__ unsigned fast_shift(unsigned long long lo, unsigned long long hi) {
@@ -699,76 +708,6 @@ __device__ __forceinline__ unsigned fast_shift(unsigned long long lo, unsigned l
   unsigned s = 0;
   while ((width - 1) >> s >= (unsigned long long)kFastBins) ++s;
   return s;
-}
-
-// Exclusive scan of one CTA's 2048 bins (eight per thread); returns, for
-// each of up to three ranks, the bin holding it.  Every thread must call it.
-__device__ void fast_find(const unsigned* h, const unsigned long long* rank, int nr, FastFind* out,
-                          unsigned long long* wsum) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned c[8];
-  unsigned mine = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    c[i] = h[8 * tid + i];
-    mine += c[i];
-  }
-  unsigned long long incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) wsum[warp] = incl;
-  __syncthreads();
-  unsigned long long before = incl - mine;
-  for (int w = 0; w < warp; ++w) before += wsum[w];
-  for (int r = 0; r < nr; ++r) {
-    const unsigned long long k = rank[r];
-    if (k >= before && k < before + mine) {
-      unsigned long long cum = before;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (k >= cum && k < cum + c[i]) out[r] = FastFind{cum, (unsigned)(8 * tid + i), c[i]};
-        cum += c[i];
-      }
-    }
-  }
-  __syncthreads();
-}
-
-// Sample quantiles of the n keys in pool (range [kmin, kmax]) at ranks
-// t[0] <= t[nt-1]: a histogram over the whole range, then one over the bins
-// holding the first and last target.  Returns the lower edge of the first
-// target's final bin and the upper edge of the last one's.  CTA-local.
-__device__ void fast_quantiles(const uint32_t* pool, unsigned n, unsigned kmin, unsigned kmax,
-                               const unsigned long long* t, int nt, unsigned* hist,
-                               unsigned long long* wsum, FastFind* res, uint32_t* qlo,
-                               uint32_t* qhi) {
-  unsigned long long lo = kmin, hi = kmax;
-  unsigned long long rk[2] = {t[0], t[nt - 1]};
-  for (int round = 0; round < 2; ++round) {
-    const unsigned sh = fast_shift(lo, hi);
-    for (int b = threadIdx.x; b < kFastBins; b += kFastThreads) hist[b] = 0;
-    if (threadIdx.x < 2) res[threadIdx.x] = FastFind{0ull, 0u, 0u};
-    __syncthreads();
-    for (unsigned i = threadIdx.x; i < n; i += kFastThreads) {
-      const uint32_t k = pool[i];
-      if (k >= lo && k <= hi) atomicAdd(&hist[(unsigned)((k - lo) >> sh)], 1u);
-    }
-    __syncthreads();
-    fast_find(hist, rk, 2, res, wsum);
-    const FastFind f0 = res[0], f1 = res[1];
-    const unsigned long long nlo = lo + ((unsigned long long)f0.bin << sh);
-    const unsigned long long nhi = min(hi, lo + ((unsigned long long)f1.bin << sh) + ((1ull << sh) - 1));
-    rk[0] -= f0.below;
-    rk[1] -= f0.below;
-    lo = nlo;
-    hi = nhi;
-    __syncthreads();   // res and hist are rewritten next round
-  }
-  *qlo = (uint32_t)lo;
-  *qhi = (uint32_t)hi;
 }
 
 // Sample ranks 1/2 -+ delta of n sample keys (delta = 4.5 standard errors of
@@ -806,12 +745,13 @@ __global__ void __launch_bounds__(kFastThreads, 4) k_medmad_fast(const float* __
                                                                  double* cs,
                                                                  unsigned long long* invalid) {
   __shared__ uint32_t pool[kFastPool];
+  __shared__ float samp[kFastSlots];       // this CTA's sample; NaN: no value
   __shared__ unsigned hist[2][kFastBins];
   __shared__ unsigned coarse[2][64];
   __shared__ unsigned sum64[64];
-  __shared__ unsigned long long wsum[kFastWarps];
   __shared__ FastFind res[2];
-  __shared__ unsigned cnt, kmin, kmax;
+  __shared__ unsigned cnt;
+  __shared__ unsigned srange[2][3];        // each bracket's sample: least and greatest key, count
   __shared__ unsigned long long mine[3];   // this CTA's pass counts: finite, low, copies
   __shared__ unsigned long long sel[3];    // cluster selection state: lo, hi, rank
   cg::cluster_group cl = cg::this_cluster();
@@ -820,68 +760,135 @@ __global__ void __launch_bounds__(kFastThreads, 4) k_medmad_fast(const float* __
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* v = vals + (size_t)g * stride;
   const int64_t nv = VEC ? stride / 4 : stride;
-  // sample slots: one run of 32 values per 32 slots
-  const unsigned slots = 32u * (unsigned)min((stride + 31) / 32, (int64_t)kFastRuns);
+  // cluster rounds alternate between the two histograms: one is cleared again
+  // only after the next round's cluster barrier, when no CTA still reads it
   int buf = 0;
 
   auto reset = [&]() {
     if (tid == 0) {
       cnt = 0;
-      kmin = 0xffffffffu;
-      kmax = 0;
       mine[0] = mine[1] = mine[2] = 0;
     }
     __syncthreads();
   };
-  // the sample (the same runs in every CTA) as keys of v or of |v - med|:
-  // run c fills slots 32c .. 32c+31; a value that is not finite leaves key 0,
-  // below every finite key, which the ranges of the quantile rounds exclude
-  auto sample = [&](bool mad, float med) -> unsigned {
-    const int64_t runs = (stride + 31) / 32;
-    const int64_t use = runs < kFastRuns ? runs : kFastRuns;
-    unsigned lmin = 0xffffffffu, lmax = 0u, nfin = 0;
-    for (int64_t c = warp; c < use; c += kFastWarps) {   // every run into L2 first
-      const int64_t i = (c * runs / use) * 32 + lane;
-      if (i < stride) asm volatile("prefetch.global.L2 [%0];" ::"l"((const void*)(v + i)));
-    }
-    constexpr int B = 12;
-    for (int64_t c0 = warp; c0 < use; c0 += B * kFastWarps) {
-      float x[B];
-      bool in[B];
+  // This CTA's part of the sample: run c of the group's goes to CTA c mod 8.
+  auto gather = [&]() {
+    const unsigned runs = (unsigned)((stride + 31) / 32);   // at most kFastMaxPerGroup / 32
+    const unsigned use = min(runs, (unsigned)kFastRuns);
+    constexpr int B = kFastSlots / kFastThreads;
+    float x[B];
 #pragma unroll
-      for (int b = 0; b < B; ++b) {
-        const int64_t c = c0 + b * kFastWarps;
-        const int64_t i = (c * runs / use) * 32 + lane;
-        in[b] = c < use && i < stride;
-        x[b] = in[b] ? v[i] : 0.f;
-      }
-#pragma unroll
-      for (int b = 0; b < B; ++b) {
-        const int64_t c = c0 + b * kFastWarps;
-        const float y = mad ? fabsf(x[b] - med) : x[b];
-        const bool ok = in[b] && finite_bits(x[b]) && finite_bits(y);
-        const uint32_t key = ok ? f32_key(y) : 0u;
-        if (c < use) pool[c * 32 + lane] = key;
-        if (ok) {
-          lmin = min(lmin, key);
-          lmax = max(lmax, key);
-          ++nfin;
-        }
-      }
+    for (int b = 0; b < B; ++b) {
+      const unsigned c = (unsigned)(b * kFastWarps + warp) * kClusterCtas + crank;
+      const int64_t i = (int64_t)(c * runs / use) * 32 + lane;
+      x[b] = c < use && i < stride ? v[i] : __uint_as_float(0x7fffffffu);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lmin = min(lmin, __shfl_xor_sync(0xffffffffu, lmin, o));
-      lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-      nfin += __shfl_xor_sync(0xffffffffu, nfin, o);
-    }
-    if (lane == 0) {
-      atomicMin(&kmin, lmin);
-      atomicMax(&kmax, lmax);
-      atomicAdd(&cnt, nfin);
+    for (int b = 0; b < B; ++b) samp[b * kFastThreads + tid] = x[b];
+    if (tid < 2) {
+      srange[tid][0] = 0xffffffffu;
+      srange[tid][1] = 0u;
+      srange[tid][2] = 0u;
     }
     __syncthreads();
-    return cnt;
+  };
+  // key of a sample value, or of its |v - med|; 0, below every finite key,
+  // where that is not finite
+  auto samp_key = [&](int l, bool mad, float med) -> uint32_t {
+    const float x = samp[l];
+    const float y = mad ? fabsf(x - med) : x;
+    return finite_bits(x) && finite_bits(y) ? f32_key(y) : 0u;
+  };
+  // This round's histogram summed over the cluster by coarse bins, into sum64.
+  auto coarse_sums = [&]() {
+    const unsigned* h = hist[buf];
+    const int c = tid >> 2, part = tid & 3;   // 64 coarse bins of 32
+    unsigned sum = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum += h[c * 32 + part * 8 + i];
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    if (part == 0) coarse[buf][c] = sum;
+    cl.sync();   // every CTA's histogram and coarse counts are complete
+    if (tid < 64) {
+      unsigned t = 0;
+      for (int r = 0; r < kClusterCtas; ++r) t += cl.map_shared_rank(coarse[buf], r)[tid];
+      sum64[tid] = t;
+    }
+    __syncthreads();
+  };
+  // One warp: the bin of the cluster's histogram that holds the rank.
+  auto find_bin = [&](unsigned long long rank) -> FastFind {
+    int cbin, fbin;
+    unsigned long long cbelow, fbelow;
+    unsigned size;
+    warp_find64(sum64, rank, &cbin, &cbelow, &size);
+    unsigned f = 0;
+    for (int r = 0; r < kClusterCtas; ++r) f += cl.map_shared_rank(hist[buf], r)[cbin * 32 + lane];
+    warp_find32(f, rank - cbelow, &fbin, &fbelow, &size);
+    return FastFind{cbelow + fbelow, (unsigned)(cbin * 32 + fbin)};
+  };
+  // The bracket of the median (or of the MAD): the lower edge of the bin of the
+  // first target rank and the upper edge of the last one's, after a histogram
+  // over the sample's range and one over the bins between.  Returns the number
+  // of finite values in the cluster's sample; with none, no bracket.
+  auto bracket = [&](bool mad, float med, uint32_t* qlo, uint32_t* qhi) -> unsigned {
+    unsigned lmin = 0xffffffffu, lmax = 0u, nfin = 0;
+    for (int l = tid; l < kFastSlots; l += kFastThreads) {
+      const uint32_t key = samp_key(l, mad, med);
+      if (key) {
+        lmin = min(lmin, key);
+        lmax = max(lmax, key);
+        ++nfin;
+      }
+    }
+    lmin = __reduce_min_sync(0xffffffffu, lmin);
+    lmax = __reduce_max_sync(0xffffffffu, lmax);
+    nfin = __reduce_add_sync(0xffffffffu, nfin);
+    unsigned* own = srange[mad];
+    if (lane == 0) {
+      atomicMin(&own[0], lmin);
+      atomicMax(&own[1], lmax);
+      atomicAdd(&own[2], nfin);
+    }
+    cl.sync();   // (also: no CTA still reads the counts of the pass before)
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+    unsigned ns = 0;
+    for (int r = 0; r < kClusterCtas; ++r) {
+      const unsigned* o = cl.map_shared_rank(own, r);
+      kmin = min(kmin, o[0]);
+      kmax = max(kmax, o[1]);
+      ns += o[2];
+    }
+    if (ns == 0) return 0;
+    unsigned long long lo = kmin, hi = kmax, t[2];
+    fast_targets(ns, t);
+    for (int round = 0; round < 2; ++round) {
+      const unsigned sh = fast_shift(lo, hi);
+      for (int b = tid; b < kFastBins; b += kFastThreads) hist[buf][b] = 0;
+      __syncthreads();
+      for (int l = tid; l < kFastSlots; l += kFastThreads) {
+        const uint32_t k = samp_key(l, mad, med);
+        if (k >= lo && k <= hi) atomicAdd(&hist[buf][(unsigned)((k - lo) >> sh)], 1u);
+      }
+      __syncthreads();
+      coarse_sums();
+      if (warp < 2) {
+        const FastFind f = find_bin(t[warp]);
+        if (lane == 0) res[warp] = f;
+      }
+      __syncthreads();
+      const FastFind f0 = res[0], f1 = res[1];
+      hi = min(hi, lo + ((unsigned long long)f1.bin << sh) + ((1ull << sh) - 1));
+      lo += (unsigned long long)f0.bin << sh;
+      t[0] -= f0.below;
+      t[1] -= f0.below;
+      __syncthreads();   // res is rewritten next round
+      buf ^= 1;
+    }
+    *qlo = (uint32_t)lo;
+    *qhi = (uint32_t)hi;
+    return ns;
   };
   // One pass over this CTA's share.  keyof(x) maps a value to the key that is
   // ranked (the key of v, or of |v - median|); over keys, the finite values
@@ -989,7 +996,6 @@ __global__ void __launch_bounds__(kFastThreads, 4) k_medmad_fast(const float* __
     for (int round = 0; round < 8 && lo < hi; ++round) {
       const unsigned sh = fast_shift(lo, hi);
       unsigned* h = hist[buf];
-      unsigned* co = coarse[buf];
       for (int b = tid; b < kFastBins; b += kFastThreads) h[b] = 0;
       __syncthreads();
       for (unsigned i = tid; i < n; i += kFastThreads) {
@@ -997,38 +1003,14 @@ __global__ void __launch_bounds__(kFastThreads, 4) k_medmad_fast(const float* __
         if (k >= lo && k <= hi) atomicAdd(&h[(unsigned)((k - lo) >> sh)], 1u);
       }
       __syncthreads();
-      {
-        const int c = tid >> 2, part = tid & 3;   // 64 coarse bins of 32
-        unsigned sum = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) sum += h[c * 32 + part * 8 + i];
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        if (part == 0) co[c] = sum;
-      }
-      cl.sync();   // every CTA's histogram and coarse counts are complete
-      if (tid < 64) {
-        unsigned t = 0;
-        for (int r = 0; r < kClusterCtas; ++r) t += cl.map_shared_rank(co, r)[tid];
-        sum64[tid] = t;
-      }
-      __syncthreads();
+      coarse_sums();
       if (warp == 0) {
-        int cbin;
-        unsigned long long cbelow;
-        unsigned csize;
-        warp_find64(sum64, rank, &cbin, &cbelow, &csize);
-        unsigned f = 0;
-        for (int r = 0; r < kClusterCtas; ++r) f += cl.map_shared_rank(h, r)[cbin * 32 + lane];
-        int fbin;
-        unsigned long long fbelow;
-        unsigned fsize;
-        warp_find32(f, rank - cbelow, &fbin, &fbelow, &fsize);
+        const FastFind f = find_bin(rank);
         if (lane == 0) {
-          const unsigned long long nlo = lo + ((unsigned long long)(cbin * 32 + fbin) << sh);
+          const unsigned long long nlo = lo + ((unsigned long long)f.bin << sh);
           sel[0] = nlo;
           sel[1] = min(hi, nlo + ((1ull << sh) - 1));
-          sel[2] = rank - cbelow - fbelow;
+          sel[2] = rank - f.below;
         }
       }
       __syncthreads();
@@ -1045,15 +1027,10 @@ __global__ void __launch_bounds__(kFastThreads, 4) k_medmad_fast(const float* __
     cl.sync();   // nobody leaves while others may still read its shared memory
   };
 
-  // ---- median bracket from the sample (the same in every CTA)
-  reset();
-  unsigned ns = sample(false, 0.f);
+  // ---- median bracket from the sample
+  gather();
   uint32_t kA = 0, kB = 0;
-  if (ns > 0) {
-    unsigned long long t[2];
-    fast_targets(ns, t);
-    fast_quantiles(pool, slots, kmin, kmax, t, 2, hist[1], wsum, res, &kA, &kB);
-  }
+  const unsigned ns = bracket(false, 0.f, &kA, &kB);
   // ---- pass 1: finite count, keys below A, copies of [A, B]
   reset();
   unsigned long long tot[3];
@@ -1075,25 +1052,17 @@ __global__ void __launch_bounds__(kFastThreads, 4) k_medmad_fast(const float* __
   }
   const float med = f32_from_key(select(kA, kB, R - tot[1]));
   // ---- MAD bracket from the sample of |v - median|
-  cl.sync();   // every CTA is done with its copies before they are replaced
-  reset();
-  ns = sample(true, med);
   uint32_t mlo = 0, mhi = 0xffffffffu;
-  if (ns > 0) {
-    unsigned long long t[2];
-    fast_targets(ns, t);
-    fast_quantiles(pool, slots, kmin, kmax, t, 2, hist[buf], wsum, res, &mlo, &mhi);
-  }
+  const unsigned nm = bracket(true, med, &mlo, &mhi);
   // ---- pass 2: |v - median| <= m_lo counted, (m_lo, m_hi) copied
-  cl.sync();   // no CTA still reads the previous counts
-  if (ns == 0 || mhi <= mlo + 1u) {   // no key strictly inside: the bracket cannot hold the MAD
+  if (nm == 0 || mhi <= mlo + 1u) {   // no key strictly inside: the bracket cannot hold the MAD
     leave(true);
     return;
   }
   reset();
   pass([&](float x) { return finite_bits(x) ? f32_key(fabsf(x - med)) : kNoKey; }, mlo + 1,
        mlo + 1, mhi - 1, tot);
-  if (ns == 0 || tot[2] == ~0ull || R < tot[1] || R >= tot[1] + tot[2]) {
+  if (tot[2] == ~0ull || R < tot[1] || R >= tot[1] + tot[2]) {
     leave(true);
     return;
   }

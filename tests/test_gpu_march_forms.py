@@ -56,7 +56,7 @@ def test_segments_of_a_long_series(w, running):
     check(99, 41, 83, w, running=running, branch=F.BRANCH_BOTH)
 
 
-@pytest.mark.parametrize("n", [1, 2, 2049, 48 * 1024 - 1, 48 * 1024, 48 * 1024 + 1])
+@pytest.mark.parametrize("n", [1, 2, 2049, 48 * 1024 - 1, 48 * 1024, 48 * 1024 + 1, 300_000, 1 << 21])
 @pytest.mark.parametrize("kind", ["skewed", "constant", "nan"])
 def test_noise_at_the_resident_limit(n, kind):
     groups = 3
