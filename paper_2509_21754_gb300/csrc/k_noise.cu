@@ -679,7 +679,8 @@ __global__ void __launch_bounds__(kClusterThreads, 4) k_medmad_cluster(const flo
 // the sample took 13 to 20 us and its quantiles 11 to 24 us per bracket, of 200
 // for 62 maps of 672,400 values (the passes 45 and 33, the selects 10 and 8);
 // shared out over the cluster the whole takes 209 -> 171 us, with twice the
-// sample and so 30% fewer copies.
+// sample and so 30% fewer copies; 156 us with the target ranks in FP32 and the
+// coarse sums free of bank conflicts.
 constexpr int kFastThreads = 256;
 constexpr int kFastWarps = kFastThreads / 32;
 constexpr int kFastBins = 2048;                    // 64 coarse bins of 32
@@ -703,20 +704,21 @@ struct FastFind {
   unsigned bin;
 };
 
+static_assert(kFastBins == 2048, "fast_shift assumes 11-bit bins");
+// the least s with (hi - lo) >> s < 2048; keys are 32 bits wide
 __device__ __forceinline__ unsigned fast_shift(unsigned long long lo, unsigned long long hi) {
-  const unsigned long long width = hi - lo + 1;   // <= 2^32
-  unsigned s = 0;
-  while ((width - 1) >> s >= (unsigned long long)kFastBins) ++s;
-  return s;
+  return 32 - __clz((int)((uint32_t)(hi - lo) >> 11));
 }
 
 // Sample ranks 1/2 -+ delta of n sample keys (delta = 4.5 standard errors of
-// a sample median, counting each run of 32 values as half as informative).
+// a sample median, counting each run of 32 values as half as informative).  In
+// FP32: the ranks only decide how much the passes copy, and every thread
+// evaluates this (FP64 is slow on this part).
 __device__ __forceinline__ void fast_targets(unsigned ns, unsigned long long* t) {
-  const double d = 4.5 * 0.5 / sqrt(0.5 * (double)ns) + 1.0 / (double)ns;
-  const double m = (double)(ns - 1);
-  const double a = floor((0.5 - d) * m), b = ceil((0.5 + d) * m);
-  t[0] = a < 0.0 ? 0ull : (unsigned long long)a;
+  const float d = 4.5f * 0.5f * rsqrtf(0.5f * (float)ns) + 1.0f / (float)ns;
+  const float m = (float)(ns - 1);
+  const float a = floorf((0.5f - d) * m), b = ceilf((0.5f + d) * m);
+  t[0] = a < 0.0f ? 0ull : (unsigned long long)a;
   t[1] = b > m ? (unsigned long long)m : (unsigned long long)b;
 }
 
@@ -805,7 +807,7 @@ __global__ void __launch_bounds__(kFastThreads, 4) k_medmad_fast(const float* __
     const int c = tid >> 2, part = tid & 3;   // 64 coarse bins of 32
     unsigned sum = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) sum += h[c * 32 + part * 8 + i];
+    for (int i = 0; i < 8; ++i) sum += h[c * 32 + part * 8 + ((i + c) & 7)];   // 32 banks
     sum += __shfl_xor_sync(0xffffffffu, sum, 1);
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
     if (part == 0) coarse[buf][c] = sum;
@@ -1383,18 +1385,6 @@ __device__ unsigned split_sample(const float* v, int64_t stride, bool mad, float
   return *nfin_sh;
 }
 
-// Sample ranks 1/2 -+ delta of ns sample values (delta = 4.5 standard errors of
-// a sample median, a run of 32 values counting as half as informative).
-// The ranks only decide how much the passes copy, so FP32 is enough (FP64 is
-// slow on this part, and every thread evaluates this).
-__device__ __forceinline__ void split_targets(unsigned ns, unsigned long long* t) {
-  const float d = 4.5f * 0.5f * rsqrtf(0.5f * (float)ns) + 1.0f / (float)ns;
-  const float m = (float)(ns - 1);
-  const float a = floorf((0.5f - d) * m), b = ceilf((0.5f + d) * m);
-  t[0] = a < 0.f ? 0ull : (unsigned long long)a;
-  t[1] = b > m ? (unsigned long long)(ns - 1) : (unsigned long long)b;
-}
-
 // Sample quantiles at ranks t[0] <= t[1] among the finite sample keys (range
 // [kmin, kmax]): one histogram over the range, one over the bins holding the
 // two targets; returns the lower edge of t[0]'s final bin and the upper edge
@@ -1450,7 +1440,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_bracket(const float* __
   uint32_t A = 1, B = 0;   // empty range when the sample has no finite value
   if (ns > 0) {
     unsigned long long t[2];
-    split_targets(ns, t);
+    fast_targets(ns, t);
     split_quantiles(spool, slots, kmm[0], kmm[1], t, hist, wsum, found, &A, &B);
   }
   if (threadIdx.x == 0) {
@@ -1869,7 +1859,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __r
   uint32_t mlo = 0, mhi = 0;
   if (ns > 0) {
     unsigned long long t[2];
-    split_targets(ns, t);
+    fast_targets(ns, t);
     split_quantiles(spool, slots, kmm[0], kmm[1], t, hist, wsum, found, &mlo, &mhi);
   }
   if (ns == 0 || mhi <= mlo + 1u) {   // no key strictly inside the bracket
