@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kSlideMaxThreads) k_slide(const __grid_constan
 // ---------------------------------------------------------------- small windows
 // Windows 7 and 9 (h = 3, 4): one thread per column of the extended block,
 // eight output rows per CTA.  Each thread carries x^(s+1) and D^(s) of its
-// column's 16 + 2h rows in registers; per unit, each row's Delta and r go
+// column's 8 + 2h rows in registers; per unit, each row's Delta and r go
 // straight into the horizontal window by warp shuffles (a warp of 32 columns
 // yields the 32 - 2h windows that lie inside it; neighbouring warps overlap by
 // 2h columns), and the vertical window is summed over the last w rows of
@@ -281,9 +281,11 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_shf(const __grid_co
           const float d = fabsf(dn - dp[i]);   // Delta
           const float ref = SIGNED ? xp[i] : fabsf(xp[i]);
           const float xh = (xp[i] == 0.f) ? kGuardC : ref;   // Eq. 5
-          // Eq. 4 (in the ABS reading the saturation is the clamp, and the
-          // approximate reciprocal needs none of the division's range checks)
-          const float r = SIGNED ? fminf(__fdividef(d, xh), 1.f) : __saturatef(d * rcp_approx(xh));
+          // Eq. 4.  A division: the approximate reciprocal of a subnormal x is
+          // infinite.  (Two forms of the unit's code as in the pairs' march, one
+          // without the guard, cost more than they saved: 669 us for 32 x 2048^2
+          // at w = 7 and 798 at w = 9, 596 and 728 so.)
+          const float r = fminf(__fdividef(d, xh), 1.f);
           lane_window<W>(d, r, rs[i % W], rm[i % W], rq[i % W]);
           if (i >= W - 1) {
             const int oy = i - (W - 1);        // output row, window rows oy .. i
@@ -419,7 +421,9 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_pair(
   float mx = -INFINITY;
   const uint64_t deadline = globaltimer_ns() + a.timeout_ns;
 
-  // one unit's rows; FAST: no x^(s+1) of this warp's pixels is zero
+  // one unit's rows; FAST: every x^(s+1) of this warp's pixels is a normal number
+  // (not zero, whose guard is Eq. 5's, nor subnormal, whose approximate reciprocal
+  // is infinite)
   auto unit = [&](auto fast_tag, const T* st, int j, float& sm) {
     constexpr bool FAST = decltype(fast_tag)::value;
     float rs[W][2], rm[W][2], rq[W][2];   // horizontal windows of the last W rows (a ring)
@@ -515,7 +519,7 @@ __global__ void __launch_bounds__(kShfWarps * 32, 4) k_slide_pair(
 #pragma unroll
         for (int i = 0; i < EH; ++i) mn = fminf(mn, fminf(fabsf(x[i][0]), fabsf(x[i][1])));
       }
-      if (!SIGNED && __all_sync(0xffffffffu, mn != 0.f))
+      if (!SIGNED && __all_sync(0xffffffffu, mn >= FLT_MIN))
         unit(std::true_type{}, st, j, sm);
       else
         unit(std::false_type{}, st, j, sm);
