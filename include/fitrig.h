@@ -226,7 +226,10 @@ FITRIG_API int fitrig_plan_set(fitrig_plan_t plan, int option, int64_t value);
  * fitrig_push_snapshot -- copy the next snapshot (slot = number pushed so far)
  * into the plan's device stack.  `data` holds ny rows of `row_pitch_elems`
  * elements (0 means nx) of type `dtype`; it is a device pointer when
- * `on_device` is non-zero, else host memory.  A dtype different from the
+ * `on_device` is non-zero, else host memory.  Device memory is the plan's
+ * device's; another GPU's is taken (by the runtime's copy) where the snapshot is
+ * stored as it is, of the storage type and neither coded nor accumulated.  A
+ * dtype different from the
  * storage type is converted on the device (round to nearest even); with
  * FITRIG_CODING_DELTA it is coded on the device instead (see
  * FITRIG_OPT_CODING).  The

@@ -832,6 +832,27 @@ static cudaError_t copy_rows_h2d(fitrig_plan_t p, void* dst, size_t dpitch, cons
   return e;
 }
 
+// Whether a kernel of the plan's device may read the elements at src: device
+// memory of that GPU, at a multiple of the half types' two bytes.  Another GPU's
+// memory, host memory that was passed as device memory and odd addresses are
+// the runtime's copy's, which reaches them or refuses the call.
+static bool kernel_readable(fitrig_plan_t p, const void* src) {
+  if (reinterpret_cast<uintptr_t>(src) % 2) return false;
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, src) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == p->device;
+}
+
+// Device-to-device copy of ny rows of `width` bytes on `st`.
+static cudaError_t copy_rows_d2d(fitrig_plan_t p, void* dst, size_t dpitch, const void* src,
+                                 size_t spitch, size_t width, int64_t ny, cudaStream_t st) {
+  if (kernel_readable(p, src)) return launch_repitch(src, spitch, dst, dpitch, width, ny, st);
+  return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, ny, cudaMemcpyDeviceToDevice, st);
+}
+
 // One snapshot into the next slot; arguments already validated.  With `sync`
 // a host push returns only after its copy finished (the caller may then reuse
 // the buffer); without it the caller synchronises the plan's stream.
@@ -888,7 +909,8 @@ static int push_one(fitrig_plan_t p, const void* data, int dtype, int on_device,
   }
   if (dtype == p->storage) {
     if (on_device)
-      CK(launch_repitch(data, rp * ib, dst, p->pitch * eb, (size_t)p->nx * ib, p->ny, st));
+      CK(copy_rows_d2d(p, dst, (size_t)p->pitch * eb, data, (size_t)rp * ib, (size_t)p->nx * ib,
+                       p->ny, st));
     else
       CK(copy_rows_h2d(p, dst, (size_t)p->pitch * eb, data, (size_t)rp * ib, (size_t)p->nx * ib,
                        p->ny, st));
@@ -963,7 +985,7 @@ FITRIG_API int fitrig_push_snapshots(fitrig_plan_t p, const void* data, int32_t 
     else if (dp == row && sp == row)
       CK(cudaMemcpyAsync(dst, data, row * (size_t)rows, cudaMemcpyDeviceToDevice, st));
     else
-      CK(launch_repitch(data, sp, dst, dp, row, rows, st));
+      CK(copy_rows_d2d(p, dst, dp, data, sp, row, rows, st));
     p->pushed += count;
     p->detected = false;
     if (p->coding == FITRIG_CODING_DELTA) p->dstate_stale = true;
