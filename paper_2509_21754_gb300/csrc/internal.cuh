@@ -161,6 +161,16 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
   return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// Raises a kernel's limit of dynamic shared memory on the current device to
+// `bytes` (never lowers it).  The limit belongs to a device, so one flag a
+// process would leave a second GPU without it, and it is one word that all
+// threads share: a launch that needs less must not lower it under another's.
+cudaError_t allow_smem_limit(const void* kern, size_t bytes);
+template <typename K>
+cudaError_t allow_smem(K* kern, size_t bytes) {
+  return allow_smem_limit(reinterpret_cast<const void*>(kern), bytes);
+}
+
 // Stack-march geometry chosen on the host (see k_stack.cu).
 struct StackGeom {
   int w;              // tile size

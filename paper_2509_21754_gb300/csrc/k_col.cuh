@@ -187,13 +187,8 @@ __global__ void __launch_bounds__(ColShape<W>::kThreads) k_stack_col(const __gri
 template <typename T, int W, bool SIGNED>
 static cudaError_t launch_col_w(const CUtensorMap* tmap, const StackArgs& a, cudaStream_t st) {
   auto kern = k_stack_col<T, W, SIGNED>;
-  static size_t configured = 0;
-  if (a.g.smem_bytes > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)a.g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    configured = a.g.smem_bytes;
-  }
+  const cudaError_t lim = allow_smem(kern, a.g.smem_bytes);
+  if (lim != cudaSuccess) return lim;
   return launch_segments(kern, tmap, a, st);
 }
 

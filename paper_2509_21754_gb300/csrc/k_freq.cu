@@ -907,13 +907,8 @@ static cudaError_t launch_long(const float* vp, int n, int64_t T, int64_t vs,
                                int* bin, cudaStream_t st) {
   const int K = n / 2;
   const size_t sm = (size_t)kLongWarps * (long_ldy(n) + K + 1) * sizeof(float);
-  static size_t long_configured = 0;
-  if (sm > 48 * 1024 && sm > long_configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_dft_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    if (e != cudaSuccess) return e;
-    long_configured = sm;
-  }
+  const cudaError_t lim = allow_smem(k_dft_long, sm);
+  if (lim != cudaSuccess) return lim;
   const int64_t lblocks = (T + kLongWarps - 1) / kLongWarps;
   k_dft_long<<<(unsigned)lblocks, kLongWarps * 32, sm, st>>>(vp, n, T, vs, tw_row, wts, hmax,
                                                              eta, bin);
@@ -927,13 +922,8 @@ static cudaError_t launch_mixed_t(const float* vp, int n, int P, int64_t T, int6
                                   int* bin, cudaStream_t st) {
   const size_t sm = sizeof(float2) * ((size_t)n + (size_t)WARPS * mixed_lds(n, P)) +
                     sizeof(float) * (size_t)WARPS * long_ldy(n);
-  static size_t configured = 0;
-  if (sm > 48 * 1024 && sm > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_dft_mixed<WARPS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    configured = sm;
-  }
+  const cudaError_t lim = allow_smem(k_dft_mixed<WARPS>, sm);
+  if (lim != cudaSuccess) return lim;
   const int64_t blocks = (T + WARPS - 1) / WARPS;
   k_dft_mixed<WARPS><<<(unsigned)blocks, WARPS * 32, sm, st>>>(vp, n, P, T, vs, tw, wts, hmax, eta,
                                                               bin);
@@ -946,13 +936,8 @@ static cudaError_t launch_fft_t(const float* vp, int n, int64_t T, int64_t vs, c
                                 const float* wts, int hmax, float* eta, int* bin,
                                 cudaStream_t st) {
   const size_t sm = (size_t)TILES * fft_tile(n / 2, TILES) * sizeof(float2);
-  static size_t configured = 0;
-  if (sm > 48 * 1024 && sm > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_fft_pow2<TILES>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    configured = sm;
-  }
+  const cudaError_t lim = allow_smem(k_fft_pow2<TILES>, sm);
+  if (lim != cudaSuccess) return lim;
   int logN = 0;
   while ((2 << logN) < n) ++logN;   // N = n / 2 = 2^logN
   const int64_t blocks = (T + TILES - 1) / TILES;
@@ -1034,13 +1019,8 @@ static cudaError_t launch_odd_length(const float* vp, int n, int64_t T, int64_t 
     return launch_long(vp, n, T, vs, twiddle, wts, hmax, eta, bin, st);
   }
   const size_t smem = (size_t)n * kDftThreads * sizeof(float);
-  static size_t configured = 0;
-  if (smem > 48 * 1024 && smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_dft, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = smem;
-  }
+  const cudaError_t lim = allow_smem(k_dft, smem);
+  if (lim != cudaSuccess) return lim;
   k_dft<<<(unsigned)blocks, kDftThreads, smem, st>>>(vp, n, T, vs, twiddle, wts, eta, bin);
   count_launches(1);
   return cudaGetLastError();

@@ -1987,13 +1987,11 @@ __global__ void __launch_bounds__(kSplitThreads) k_medmad_small(const float* __r
 
 static cudaError_t launch_medmad_small(const float* vals, int groups, int64_t stride, int64_t n,
                                        double* cs, unsigned long long* invalid, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_medmad_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallMax * (int)sizeof(uint32_t));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  // on every call: fitrig_noise_static serves every device, and a device's next
+  // context after a reset (the limit belongs to a context)
+  const cudaError_t lim = cudaFuncSetAttribute(
+      k_medmad_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallMax * (int)sizeof(uint32_t));
+  if (lim != cudaSuccess) return lim;
   const cudaError_t e = launch_pdl(k_medmad_small, dim3(groups), dim3(kSplitThreads),
                                    (size_t)stride * sizeof(uint32_t), st, vals, stride, n, cs, invalid);
   count_launches(1);
@@ -2006,19 +2004,10 @@ static cudaError_t launch_split_t(const float* vals, int groups, int64_t stride,
   const SplitPtrs sp = split_ptrs(ns.split, groups, stride);
   if ((int64_t)sp.nchunk * kSplitSlot != ns.split_cap) return cudaErrorInvalidValue;   // carved for another stride
   const size_t dyn = (size_t)kSplitPool * sizeof(uint32_t);
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_split_bracket,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_split_select<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)dyn);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_split_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)dyn);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  cudaError_t lim = allow_smem(k_split_bracket, dyn);
+  if (lim == cudaSuccess) lim = allow_smem(k_split_select<false>, dyn);
+  if (lim == cudaSuccess) lim = allow_smem(k_split_select<true>, dyn);
+  if (lim != cudaSuccess) return lim;
   const dim3 pgrid((unsigned)sp.nchunk, (unsigned)groups);
   // CTAs that share a large map's copies: two waves of the chip over all maps,
   // at least one chunk per warp

@@ -660,13 +660,8 @@ static cudaError_t launch_segments(K kern, const CUtensorMap* tmap, SlideArgs a,
 template <typename T, int W, bool SIGNED>
 static cudaError_t launch_shf_t(const CUtensorMap* tmap, const SlideArgs& a, cudaStream_t st) {
   auto kern = W <= 5 ? k_slide_pair<T, W <= 5 ? W : 5, SIGNED> : k_slide_shf<T, W <= 5 ? 7 : W, SIGNED>;
-  static size_t configured = 0;
-  if (a.g.smem_bytes > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)a.g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    configured = a.g.smem_bytes;
-  }
+  const cudaError_t lim = allow_smem(kern, a.g.smem_bytes);
+  if (lim != cudaSuccess) return lim;
   return launch_segments(kern, tmap, a, st);
 }
 
@@ -682,13 +677,8 @@ static cudaError_t launch_slide_t(const CUtensorMap* tmap, const SlideArgs& a, c
     }
   }
   auto kern = k_slide<T, SIGNED>;
-  static size_t configured = 0;
-  if (a.g.smem_bytes > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)a.g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    configured = a.g.smem_bytes;
-  }
+  const cudaError_t lim = allow_smem(kern, a.g.smem_bytes);
+  if (lim != cudaSuccess) return lim;
   return launch_segments(kern, tmap, a, st);
 }
 

@@ -878,20 +878,14 @@ cudaError_t launch_delta_finite_max(const float* key, int64_t kpitch, const void
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(152 * 4, (total + 255) / 256));
   if (storage == FITRIG_BF16) {
     auto kern = k_delta_finite_max<bf16_t>;
-    if (sm > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)sm);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t lim = allow_smem(kern, sm);
+    if (lim != cudaSuccess) return lim;
     kern<<<blocks, 256, sm, st>>>(key, kpitch, static_cast<const bf16_t*>(stack), slice, L, ny, nx,
                                   pitch, gmax, smax);
   } else if (storage == FITRIG_F16) {
     auto kern = k_delta_finite_max<f16_t>;
-    if (sm > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)sm);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t lim = allow_smem(kern, sm);
+    if (lim != cudaSuccess) return lim;
     kern<<<blocks, 256, sm, st>>>(key, kpitch, static_cast<const f16_t*>(stack), slice, L, ny, nx,
                                   pitch, gmax, smax);
   } else {
@@ -1059,26 +1053,16 @@ int march_seg_units(int64_t boxes, int per_sm, int units) {
 template <typename T, int R, bool SIGNED>
 static cudaError_t launch_one(const CUtensorMap* tmap, const StackArgs& a, cudaStream_t st) {
   auto kern = k_stack_tile<T, R, SIGNED>;
-  static size_t configured = 0;
-  if (a.g.smem_bytes > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)a.g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    configured = a.g.smem_bytes;
-  }
+  const cudaError_t lim = allow_smem(kern, a.g.smem_bytes);
+  if (lim != cudaSuccess) return lim;
   return launch_segments(kern, tmap, a, st);
 }
 
 template <typename T, int W, bool SIGNED, bool DELTA>
 static cudaError_t launch_small(const CUtensorMap* tmap, const StackArgs& a, cudaStream_t st) {
   auto kern = k_stack_small<T, W, SIGNED, DELTA>;
-  static size_t configured = 0;
-  if (a.g.smem_bytes > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)a.g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    configured = a.g.smem_bytes;
-  }
+  const cudaError_t lim = allow_smem(kern, a.g.smem_bytes);
+  if (lim != cudaSuccess) return lim;
   return launch_segments(kern, tmap, a, st);
 }
 
@@ -1086,13 +1070,8 @@ template <typename T, bool SIGNED, bool DELTA>
 static cudaError_t launch_sub(const CUtensorMap* tmap, const StackArgs& a, cudaStream_t st) {
   const bool big = a.g.threads > 256;
   auto kern = big ? k_stack_sub<T, SIGNED, 512, DELTA> : k_stack_sub<T, SIGNED, 256, DELTA>;
-  static size_t configured[2] = {0, 0};
-  if (a.g.smem_bytes > configured[big]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)a.g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    configured[big] = a.g.smem_bytes;
-  }
+  const cudaError_t lim = allow_smem(kern, a.g.smem_bytes);
+  if (lim != cudaSuccess) return lim;
   return launch_segments(kern, tmap, a, st);
 }
 
@@ -1161,13 +1140,8 @@ static cudaError_t launch_multi_t(const FieldDesc* fields, int nfields, int64_t 
                                   unsigned long long* counter, const StackGeom& g, int grid,
                                   uint64_t timeout_ns, cudaStream_t st) {
   auto kern = k_stack_multi<T, W, SIGNED>;
-  static size_t configured = 0;
-  if (g.smem_bytes > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    configured = g.smem_bytes;
-  }
+  const cudaError_t lim = allow_smem(kern, g.smem_bytes);
+  if (lim != cudaSuccess) return lim;
   kern<<<grid, g.threads, g.smem_bytes, st>>>(fields, nfields, nitems, counter, g, timeout_ns);
   count_launches(1);
   return cudaGetLastError();
@@ -1202,7 +1176,7 @@ int multi_blocks_per_sm(const StackGeom& g, int storage, int rmode) {
   else { FITRIG_PICK(f16_t) }
 #undef FITRIG_PICK
   if (!fn) return 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem_bytes) != cudaSuccess ||
+  if (allow_smem(fn, g.smem_bytes) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, g.threads, g.smem_bytes) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;

@@ -133,6 +133,21 @@ struct Ingest {
 
 void fitrig::count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+cudaError_t fitrig::allow_smem_limit(const void* kern, size_t bytes) {
+  if (bytes <= (size_t)32 * 1024) return cudaSuccess;   // (48 KB with the kernel's static memory)
+  static std::mutex mtx;
+  static std::map<std::pair<const void*, int>, size_t> limits;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mtx);
+  size_t& limit = limits[{kern, dev}];
+  if (bytes <= limit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) limit = bytes;
+  return e;
+}
+
 struct fitrig_plan_s {
   // configuration
   int nx = 0, ny = 0, L = 0, w = 0, branch = 0;
