@@ -1899,8 +1899,6 @@ struct fitrig_server_s {
   std::vector<ServerField*> fields;   // index = field id
   std::deque<int> waiting;            // FIFO of queued field ids
   int active = 0;
-  Ingest ingest;                      // all fields' rows that do not fill the pitch (under mtx;
-                                      // 32 MB beside the budget, allocated at the first such push)
   std::mutex rmtx;                    // results only (never held across CUDA calls)
   std::deque<ServerResult> results;
 };
@@ -1917,6 +1915,53 @@ struct UnitTicket {
 };
 
 constexpr int32_t kServeCandCap = 1 << 16;
+
+// Host rows of a field that do not fill the pitch go linearly (see Ingest) to
+// the field's two candidate buffers, which are idle from the end of one trigger
+// (the candidates are exported by then) to the next, in as many pieces as it
+// takes, and a kernel sets them at their pitch.  All of it is on the field's own
+// stream: it needs no memory beside the field's reservation, and no field waits
+// for another's trigger.  Pieces below kLeastPiece (windows of 16 and more) gain
+// nothing over pitched copies.  Eight fields of 1331 to 4576 pixels a side (4 to
+// 42 MB of BF16): a round 1.35 ms, 1.65 with pitched copies.
+constexpr size_t kLeastPiece = (size_t)2 << 20;
+
+bool lends_rows(fitrig_plan_t p, size_t dpitch, size_t width) {
+  const size_t area = sizeof(fitrig_candidate) * (size_t)p->cand_cap;
+  return Ingest::suits(dpitch, width, width, width * (size_t)p->ny) &&
+         area >= std::max(width, kLeastPiece);
+}
+
+bool host_memory(const void* data) {
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, data) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeUnregistered;
+}
+
+cudaError_t push_linear(fitrig_plan_t p, char* dst, size_t dpitch, const char* src, size_t width,
+                        cudaStream_t st) {
+  void* const buf[2] = {p->d_cand, p->d_cand_tmp};
+  const int64_t ny = p->ny;
+  const int64_t most = (int64_t)(sizeof(fitrig_candidate) * (size_t)p->cand_cap / width);
+  const int64_t pieces = (ny + most - 1) / most, per = (ny + pieces - 1) / pieces;
+  cudaError_t e = cudaSuccess;
+  for (int64_t r0 = 0; r0 < ny; r0 += 2 * per) {   // two copies, then their re-pitching
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+      const int64_t r = r0 + k * per, n = std::min(per, ny - r);
+      if (n > 0)
+        e = cudaMemcpyAsync(buf[k], src + (size_t)r * width, width * (size_t)n,
+                            cudaMemcpyHostToDevice, st);
+    }
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+      const int64_t r = r0 + k * per, n = std::min(per, ny - r);
+      if (n > 0) e = launch_repitch(buf[k], width, dst + (size_t)r * dpitch, dpitch, width, n, st);
+    }
+  }
+  return e;
+}
 
 // Host callback, in stream order after a unit's trigger and export.
 void CUDART_CB unit_done(void* arg) {
@@ -2132,13 +2177,8 @@ FITRIG_API int fitrig_server_push(fitrig_server_t s, int32_t field, const void* 
     if (unit) CK(launch_stamp(f->d_stamps + 0, st));
     if (dtype == p->storage) {
       const size_t row = (size_t)p->nx * ib, dp = (size_t)p->pitch * eb;
-      cudaPointerAttributes at{};
-      const bool staged = Ingest::suits(dp, row, row, row * (size_t)p->ny) &&
-                          cudaPointerGetAttributes(&at, data) == cudaSuccess &&
-                          (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeUnregistered) &&
-                          s->ingest.ready();
-      if (staged)
-        CK(s->ingest.rows(dst, dp, static_cast<const char*>(data), row, p->ny, st));
+      if (lends_rows(p, dp, row) && host_memory(data))
+        CK(push_linear(p, dst, dp, static_cast<const char*>(data), row, st));
       else
         CK(cudaMemcpy2DAsync(dst, dp, data, row, row, p->ny, cudaMemcpyDefault, st));
     } else {
@@ -2383,7 +2423,6 @@ FITRIG_API int fitrig_server_destroy(fitrig_server_t s) {
       delete f;
     }
     s->fields.clear();
-    s->ingest.release();
   }
   delete s;
   return FITRIG_OK;
