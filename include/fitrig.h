@@ -240,8 +240,9 @@ FITRIG_API int fitrig_plan_set(fitrig_plan_t plan, int option, int64_t value);
  * already on the plan's stream; the plan's stream waits for them), so that
  * several copy engines share the transfer; pinned host memory is fastest.
  * Contiguous host rows that do not fill the device pitch (a row is not a
- * multiple of 128 bytes) go through a 32 MB device buffer of the plan, from
- * 4 MB on, allocated at the first such push (without it if there is no room).
+ * multiple of 128 bytes) go through staging slots on the device, from 4 MB on:
+ * the candidates' second buffer, or, where that is too small, memory of the size
+ * of the push and at most 32 MB, allocated at the first such push.
  */
 FITRIG_API int fitrig_push_snapshot(fitrig_plan_t plan, const void* data, int dtype,
                                     int on_device, int64_t row_pitch_elems);

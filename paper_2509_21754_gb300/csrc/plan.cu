@@ -52,78 +52,82 @@ std::atomic<long long> g_launches{0};
 // Host-to-device copies of rows that do not fill the device pitch.  The copy
 // engines move such rows at half the link's rate (6200-byte rows: 102 GB/s
 // however many streams share them, against 210 GB/s for one linear copy), so
-// contiguous host rows go to a ring of staging slots as linear copies on two
-// streams of their own, and a kernel on the caller's stream sets them at their
-// pitch while the next slot is filled: 20 snapshots of 2600 x 3100 BF16 from
-// pinned memory with the detect 3.65 -> 2.27 ms.
+// contiguous host rows go to staging slots as linear copies on two streams of
+// their own, and a kernel on the caller's stream sets them at their pitch while
+// the next slot is filled: 20 snapshots of 2600 x 3100 BF16 from pinned memory
+// with the detect 3.65 -> 2.27 ms.
 struct Ingest {
   static constexpr int kSlots = 4;
   static constexpr size_t kSlot = (size_t)8 << 20;   // 40 us of copying each
   static constexpr size_t kLeast = (size_t)4 << 20;  // below, the launches cost what is gained
-  char* buf = nullptr;
   cudaStream_t cs[2] = {};   // alternate, so that one's copy covers the other's wait and launch
   cudaEvent_t start = nullptr, full[kSlots] = {}, freed[kSlots] = {};
-  int next = 0;
-  bool failed = false;   // no memory for it: such copies stay pitched ones
+  bool ok = false;
 
-  bool ready() {
-    if (buf) return true;
-    if (failed) return false;
-    bool ok = cudaMalloc(&buf, kSlots * kSlot) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&cs[0], cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&cs[1], cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&start, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; ok && i < kSlots; ++i)
-      ok = cudaEventCreateWithFlags(&full[i], cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&freed[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) {
-      (void)cudaGetLastError();
-      release();
-      failed = true;
+  cudaError_t create() {
+    if (ok) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    for (cudaStream_t& c : cs)
+      if (e == cudaSuccess && !c) e = cudaStreamCreateWithFlags(&c, cudaStreamNonBlocking);
+    auto event = [&](cudaEvent_t& v) {
+      if (e == cudaSuccess && !v) e = cudaEventCreateWithFlags(&v, cudaEventDisableTiming);
+    };
+    event(start);
+    for (int i = 0; i < kSlots; ++i) {
+      event(full[i]);
+      event(freed[i]);
     }
-    return ok;
+    ok = e == cudaSuccess;
+    return e;
   }
 
   void release() {
-    for (cudaStream_t c : cs)
+    for (cudaStream_t& c : cs) {
       if (c) cudaStreamSynchronize(c);
-    if (buf) cudaFree(buf);
-    for (cudaStream_t c : cs)
       if (c) cudaStreamDestroy(c);
-    if (start) cudaEventDestroy(start);
-    for (int i = 0; i < kSlots; ++i) {
-      if (full[i]) cudaEventDestroy(full[i]);
-      if (freed[i]) cudaEventDestroy(freed[i]);
-      full[i] = freed[i] = nullptr;
+      c = nullptr;
     }
-    buf = nullptr;
-    cs[0] = cs[1] = nullptr;
-    start = nullptr;
+    auto event = [](cudaEvent_t& v) {
+      if (v) cudaEventDestroy(v);
+      v = nullptr;
+    };
+    event(start);
+    for (int i = 0; i < kSlots; ++i) {
+      event(full[i]);
+      event(freed[i]);
+    }
+    ok = false;
   }
 
   static bool suits(size_t dpitch, size_t spitch, size_t width, size_t bytes) {
     return spitch == width && dpitch != width && width <= kSlot && bytes >= kLeast;
   }
 
-  // `rows` contiguous host rows to dst (pitch dpitch), ordered on st: the
-  // copies start after the work already on st, and st waits for them.
-  cudaError_t rows(char* dst, size_t dpitch, const char* src, size_t width, int64_t rows,
-                   cudaStream_t st) {
-    cudaError_t e = cudaEventRecord(start, st);
+  // `rows` contiguous host rows to dst (pitch dpitch) through the `area` bytes at
+  // buf, ordered on st: the copies start after the work already on st, and st
+  // waits for them.  (area >= width)
+  cudaError_t rows(char* buf, size_t area, char* dst, size_t dpitch, const char* src, size_t width,
+                   int64_t rows, cudaStream_t st) {
+    int slots = (int)std::min<size_t>(kSlots, (area + kSlot - 1) / kSlot);
+    if (area / slots < width + 256) slots = 1;
+    const size_t slot = std::min(kSlot, slots == 1 ? area : area / slots / 256 * 256);
+    cudaError_t e = create();
+    if (e == cudaSuccess) e = cudaEventRecord(start, st);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(cs[i], start, 0);
-    const int64_t per = (int64_t)(kSlot / width);
-    for (int64_t r = 0; r < rows && e == cudaSuccess; r += per) {
+    const int64_t per = (int64_t)(slot / width);
+    int k = 0;
+    for (int64_t r = 0; r < rows && e == cudaSuccess; r += per, ++k) {
       const int64_t n = std::min(per, rows - r);
-      char* slot = buf + (size_t)next * kSlot;
-      const cudaStream_t c = cs[next & 1];
-      e = cudaStreamWaitEvent(c, freed[next], 0);   // (a slot never used yet: no wait)
+      const int i = k % slots;
+      const cudaStream_t c = cs[k & 1];
+      char* from = buf + (size_t)i * slot;
+      if (k >= slots) e = cudaStreamWaitEvent(c, freed[i], 0);
       if (e == cudaSuccess)
-        e = cudaMemcpyAsync(slot, src + (size_t)r * width, width * (size_t)n, cudaMemcpyHostToDevice, c);
-      if (e == cudaSuccess) e = cudaEventRecord(full[next], c);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(st, full[next], 0);
-      if (e == cudaSuccess) e = launch_repitch(slot, width, dst + (size_t)r * dpitch, dpitch, width, n, st);
-      if (e == cudaSuccess) e = cudaEventRecord(freed[next], st);
-      next = (next + 1) % kSlots;
+        e = cudaMemcpyAsync(from, src + (size_t)r * width, width * (size_t)n, cudaMemcpyHostToDevice, c);
+      if (e == cudaSuccess) e = cudaEventRecord(full[i], c);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(st, full[i], 0);
+      if (e == cudaSuccess) e = launch_repitch(from, width, dst + (size_t)r * dpitch, dpitch, width, n, st);
+      if (e == cudaSuccess) e = cudaEventRecord(freed[i], st);
     }
     return e;
   }
@@ -244,7 +248,9 @@ struct fitrig_plan_s {
   // host-to-device pushes are split over these streams (several copy engines)
   cudaStream_t copy_st[4] = {};
   cudaEvent_t copy_ev[5] = {};
-  Ingest ingest;   // rows that do not fill the pitch (allocated at their first push)
+  Ingest ingest;                 // rows that do not fill the pitch
+  void* d_push = nullptr;        // their staging slots where no idle buffer is large enough
+  size_t push_bytes = 0;
   // a detect repeated on the same state replays a captured graph of its
   // stream work (see fitrig_detect); the state is (pushed, zrot, generation
   // of the selection lists)
@@ -290,7 +296,7 @@ static void free_all(fitrig_plan_t p) {
   void* ptrs[] = {p->d_stack, p->d_vp,  p->d_small, p->d_cs, p->d_arg, p->d_inv,
                   p->d_noise, p->d_split, p->d_blk, p->d_noise_f, p->d_split_f,
                   p->d_blk_f, p->d_fpeaks, p->d_sel, p->d_cand, p->d_cand_tmp,
-                  p->d_bin,   p->d_tw,  p->d_staging, p->d_report, p->d_accum,
+                  p->d_bin,   p->d_tw,  p->d_staging, p->d_push, p->d_report, p->d_accum,
                   p->d_hist,  p->d_hwts, p->d_htw,
                   p->d_smax,  p->d_mrun, p->d_wts, p->d_key, p->d_dstate};   // d_eta lives inside d_vp
   for (void* q : ptrs)
@@ -801,6 +807,30 @@ FITRIG_API int fitrig_plan_set(fitrig_plan_t p, int option, int64_t value) {
   }
 }
 
+// Staging memory for a push of `bytes` from the host: the candidates' second
+// buffer, which nothing uses between detects (32 bytes per entry of the
+// selection limit: a pushed stack's automatic limit nearly always has room for
+// two slots), else memory that is kept for later pushes and counted as the
+// plan's: no more than the push, nor four slots.  Null where there is no room.
+static char* push_area(fitrig_plan_t p, size_t bytes, size_t* area) {
+  const size_t lent = sizeof(fitrig_candidate) * (size_t)p->cand_cap;
+  const size_t most = std::min(bytes, Ingest::kSlots * Ingest::kSlot);
+  if (lent >= std::min(most, 2 * Ingest::kSlot)) {
+    *area = std::min(lent, Ingest::kSlots * Ingest::kSlot);
+    return reinterpret_cast<char*>(p->d_cand_tmp);
+  }
+  if (!p->d_push) {
+    if (dmalloc(p, &p->d_push, most) != cudaSuccess) {
+      (void)cudaGetLastError();
+      p->d_push = nullptr;
+      return nullptr;
+    }
+    p->push_bytes = most;
+  }
+  *area = p->push_bytes;
+  return static_cast<char*>(p->d_push);
+}
+
 // Host-to-device copy of ny rows of `width` bytes, ordered on `st`.  Large
 // snapshots are split into row bands copied on up to four side streams, so
 // that several copy engines move them at once; the bands start after the work
@@ -810,8 +840,13 @@ static cudaError_t copy_rows_h2d(fitrig_plan_t p, void* dst, size_t dpitch, cons
                                  size_t spitch, size_t width, int64_t ny, cudaStream_t st) {
   const size_t bytes = width * (size_t)ny;
   const bool linear = dpitch == width && spitch == width;
-  if (Ingest::suits(dpitch, spitch, width, bytes) && p->ingest.ready())
-    return p->ingest.rows(static_cast<char*>(dst), dpitch, static_cast<const char*>(src), width, ny, st);
+  if (Ingest::suits(dpitch, spitch, width, bytes)) {
+    size_t area = 0;
+    char* buf = push_area(p, bytes, &area);
+    if (buf && area >= width)
+      return p->ingest.rows(buf, area, static_cast<char*>(dst), dpitch,
+                            static_cast<const char*>(src), width, ny, st);
+  }
   int nb = bytes >= ((size_t)32 << 20) ? 4 : 1;
   if (nb > 1 && !p->copy_st[0]) {
     for (int i = 0; i < 4; ++i) {
