@@ -378,9 +378,12 @@ struct BlockScratch {
   uint32_t* sbits;            // [groups][Ty][words] selected-tile bitmap (v > thr)
   unsigned long long* pairs;  // [blocks][pairs per block] selected neighbours across block edges
   int64_t pcap;
-  int4* bstat;                // [blocks] boundary components, pairs, selected tiles of each block,
-                              // 1 while the block is left to k_blk_cc_full
-  int* counters;              // [2] peaks
+  int4* bstat;                // [blocks] boundary components, pairs, selected tiles of each block
+  int* full;                  // [blocks] the blocks left to k_blk_cc_full
+  int* counters;              // [1] blocks taken by k_blk_cc_full's CTAs beside their first, [2]
+                              // peaks, [3] blocks in `full`
+  unsigned* runs;             // runs of the sampled rows; zero before launch_block_select (the
+                              // caller's: not carved)
   int64_t cap;                // boundary-component slots (blocks x slots per block)
   int words;                  // bitmap words per tile row
   int nblk;                   // CTAs of the ordered compaction (kRowsPerCta tile rows each)

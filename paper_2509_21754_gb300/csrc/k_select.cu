@@ -508,7 +508,9 @@ constexpr int kBlkMaxRuns = kBlkT / 2;   // runs of a block (alternating bits at
 // Selected-tile bitmap: bit (tx & 31) of word tx / 32 of row (g, ty) is
 // v > the group's threshold (never for NaN: an invalid tile); bits past the row's end are 0.
 // One warp per row: all of the row's loads (coalesced, up to 32 per lane) are
-// issued before its ballots.
+// issued before its ballots.  The first row of each CTA adds its runs (those of
+// neighbouring words counted apart) to *b.runs, from which k_blk_cc sees how dense
+// the selection is.
 constexpr int kMaskThreads = 256;
 __global__ void __launch_bounds__(kMaskThreads) k_blk_mask(const float* __restrict__ vals,
                                                            int64_t stride, int Tx, int Ty,
@@ -517,6 +519,7 @@ __global__ void __launch_bounds__(kMaskThreads) k_blk_mask(const float* __restri
                                                            double tau, double* inv,
                                                            BlockScratch b) {
   pdl_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) b.counters[1] = b.counters[3] = 0;
   const int lane = threadIdx.x & 31;
   const int64_t r = ((int64_t)blockIdx.x * kMaskThreads + threadIdx.x) >> 5;
   if (r >= nrows) return;
@@ -527,6 +530,7 @@ __global__ void __launch_bounds__(kMaskThreads) k_blk_mask(const float* __restri
   th = __shfl_sync(0xffffffffu, th, 0);
   const float* row = vals + (size_t)g * stride + (int64_t)ty * Tx;
   uint32_t* out = b.sbits + (size_t)r * b.words;
+  unsigned runs = 0;
   for (int w0 = 0; w0 < b.words; w0 += 32) {
     float x[32];
 #pragma unroll
@@ -541,12 +545,18 @@ __global__ void __launch_bounds__(kMaskThreads) k_blk_mask(const float* __restri
       if (lane == u) mine = bal;
     }
     if (w0 + lane < b.words) out[w0 + lane] = mine;
+    runs += __popc(mine & ~(mine << 1));
+  }
+  if (threadIdx.x < 32) {
+    runs = __reduce_add_sync(0xffffffffu, runs);
+    if (lane == 0 && runs) atomicAdd(b.runs, runs);
   }
 }
 
 // The labelling of one block by NT threads, for blocks of at most MAXR runs.
 // Returns false, with nothing written, when the block has more (then every
-// thread sees it).
+// thread sees it) or with `skip` (the caller's word from memory, looked at once
+// the block's own loads are on their way).
 template <int NT, int MAXR>
 struct BlkShared {
   unsigned long long mrow[kBlkY];   // the block's rows
@@ -566,7 +576,8 @@ struct BlkShared {
 template <int NT, int MAXR>
 __device__ __forceinline__ bool blk_label(BlkShared<NT, MAXR>& sh, const float* __restrict__ vals,
                                           int64_t stride, int Tx, int Ty, const BlockScratch& b,
-                                          int64_t bidx, int g, int bx, int by, unsigned* status) {
+                                          int64_t bidx, int g, int bx, int by, bool skip,
+                                          unsigned* status) {
   static_assert(NT >= 64 && MAXR <= kBlkMaxRuns, "a thread per row");
   constexpr int kIter = (MAXR + NT - 1) / NT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -611,6 +622,7 @@ __device__ __forceinline__ bool blk_label(BlkShared<NT, MAXR>& sh, const float* 
       if (right) atomicOr(&sh.hright, 1ull << r);
     }
   }
+  if (skip) return false;
   // 2. the run list: counts per row, their scan (one thread per row, the
   // first kBlkY / 32 warps), then each row's runs
   if (tid < kBlkY) {
@@ -792,44 +804,54 @@ __device__ __forceinline__ bool blk_label(BlkShared<NT, MAXR>& sh, const float* 
 // selected, and its labelling is a chain of short dependent steps: what counts
 // is how many blocks an SM has in hand.  Two warps and shared memory for
 // kBlkFewRuns runs let 20 blocks share an SM, where 256 threads and room for
-// the most runs a block can have (2048) let six.  A block with more runs is
-// marked (bstat.w) and left to k_blk_cc_full, launched next.  Bound by issue and
-// the divergence of its loops over runs.  30 sliding maps of 16.8 M pixels 1378
-// -> 688 us, 6 maps of 24.2 M tiles 528 -> 420 us, 62 maps of 672 k 114 -> 108.
+// the most runs a block can have (2048) let six: k_blk_cc, 30 sliding maps of 16.8
+// M pixels 1378 -> 688 us, 6 maps of 24.2 M tiles 528 -> 420, 62 maps of 672 k 114
+// -> 108.  Bound by issue and the divergence of the loops over runs.
+// k_blk_cc_full takes what is left, one block to a CTA at a time over the whole
+// chip: the blocks of more runs, which k_blk_cc lists; all blocks where the
+// selection is dense (kDenseRuns a block on average by the sample of k_blk_mask,
+// 12% of the tiles, 4 sigma on sky: k_blk_cc then returns at once); and all blocks
+// of maps that fill no more than one wave of its own CTAs.  Selection of 62 maps
+// of 672 k tiles at 2 / 3 / 4 / 6 sigma 452 / 373 / 337 / 262 us; every block in
+// full 436 / 370 / 335 / 282; listed without the dense rule 516 / 415 / 337 / 259;
+// with the blocks found and labelled in turn by a CTA for each 256 of them 4326 / 460
+// / 338 / 262.  14 maps of 42 k tiles (224 blocks) at 2 / 6 sigma 51 / 36 us, listed
+// 94 / 47.
 constexpr int kBlkFewThreads = 64;
 constexpr int kBlkFewRuns = 512;
+constexpr int kDenseRuns = 360;
+constexpr int kBlkFullPerSm = 6;
+enum { kFullListed = 0, kFullAll = 1 };   // k_blk_cc_full's blocks
 
 __global__ void __launch_bounds__(kBlkFewThreads, 20) k_blk_cc(const float* __restrict__ vals,
                                                                int64_t stride, int Tx, int Ty,
-                                                               BlockScratch b, unsigned* status) {
+                                                               unsigned dense, BlockScratch b,
+                                                               unsigned* status) {
   pdl_begin();
   __shared__ BlkShared<kBlkFewThreads, kBlkFewRuns> sh;
+  const bool skip = *b.runs >= dense;
   const int64_t bidx = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
   if (!blk_label(sh, vals, stride, Tx, Ty, b, bidx, (int)blockIdx.z, (int)blockIdx.x,
-                 (int)blockIdx.y, status) &&
-      threadIdx.x == 0)
-    b.bstat[bidx] = make_int4(0, 0, 0, 1);
+                 (int)blockIdx.y, skip, status) &&
+      !skip && threadIdx.x == 0)
+    b.full[atomicAdd(&b.counters[3], 1)] = (int)bidx;
 }
 
-__global__ void __launch_bounds__(kBlkThreads) k_blk_cc_full(const float* __restrict__ vals,
-                                                             int64_t stride, int Tx, int Ty,
-                                                             int64_t nblocks, BlockScratch b,
-                                                             unsigned* status) {
+__global__ void __launch_bounds__(kBlkThreads, kBlkFullPerSm) k_blk_cc_full(
+    const float* __restrict__ vals, int64_t stride, int Tx, int Ty, int nblocks, int blocks,
+    unsigned dense, BlockScratch b, unsigned* status) {
   pdl_begin();
   __shared__ BlkShared<kBlkThreads, kBlkMaxRuns> sh;
   const int nbx = (Tx + kBlkX - 1) / kBlkX, nby = (Ty + kBlkY - 1) / kBlkY;
-  for (int64_t b0 = (int64_t)blockIdx.x * kBlkThreads; b0 < nblocks;
-       b0 += (int64_t)gridDim.x * kBlkThreads) {
-    const int64_t i = b0 + threadIdx.x;
-    if (!__syncthreads_or(i < nblocks && b.bstat[i].w)) continue;
-    for (int k = 0; k < kBlkThreads && b0 + k < nblocks; ++k) {
-      const int64_t bidx = b0 + k;
-      if (!b.bstat[bidx].w) continue;   // the same word for every thread
-      __syncthreads();                  // nobody reads it any more, nor the last block's memory
-      blk_label(sh, vals, stride, Tx, Ty, b, bidx, (int)(bidx / ((int64_t)nbx * nby)),
-                (int)(bidx % nbx), (int)(bidx / nbx % nby), status);
-      __syncthreads();
-    }
+  const bool all = blocks == kFullAll || *b.runs >= dense;
+  const int n = all ? nblocks : b.counters[3];
+  __shared__ int next[2];
+  for (int i = blockIdx.x, k = 0; i < n; i = next[k], k ^= 1) {
+    const int bidx = all ? i : b.full[i];
+    if (threadIdx.x == 0) next[k] = (int)gridDim.x + atomicAdd(&b.counters[1], 1);
+    blk_label(sh, vals, stride, Tx, Ty, b, bidx, bidx / (nbx * nby), bidx % nbx, bidx / nbx % nby,
+              false, status);
+    __syncthreads();   // the next block's memory
   }
 }
 
@@ -1029,35 +1051,24 @@ __global__ void __launch_bounds__(1024) k_blk_scan(int nblk, int64_t nblocks, Bl
 }
 
 // Small maps: everything after the labelling in one CTA, whose barriers cost
-// a fraction of the launches they replace (the full labelling of blocks of
-// many runs, unions, peaks, row counts, their scan and the check: seven).
-// Bounded by kTailBlocks blocks, four per warp (256 took 39 us against about 28
-// in launches of their own), and by the rows whose counts fit in shared memory.
+// a fraction of the launches they replace (unions, peaks, row counts, their scan
+// and the check: six).  Bounded by kTailBlocks blocks, four per warp (256 took 39
+// us against about 28 in launches of their own), and by the rows whose counts fit
+// in shared memory.
 constexpr int kTailThreads = 1024;
 constexpr int64_t kTailBlocks = 128;
 constexpr int64_t kTailRows = 4096;
 
-__global__ void __launch_bounds__(kTailThreads) k_blk_tail(const float* __restrict__ vals,
-                                                           int64_t stride, int Tx, int Ty,
+__global__ void __launch_bounds__(kTailThreads) k_blk_tail(int64_t stride, int Tx, int Ty,
                                                            int64_t nblocks, int64_t nrows,
                                                            BlockScratch b, int64_t cap,
                                                            unsigned* status, unsigned* want) {
   pdl_begin();
   __shared__ union {
-    BlkShared<kTailThreads, kBlkMaxRuns> label;
     long long scan[1024];
     int rows[kTailRows];
   } sh;
   const int tid = threadIdx.x, warp = tid >> 5;
-  if (__syncthreads_or(tid < nblocks && b.bstat[tid].w)) {
-    const int nbx = (Tx + kBlkX - 1) / kBlkX, nby = (Ty + kBlkY - 1) / kBlkY;
-    for (int k = 0; k < nblocks; ++k) {
-      if (!b.bstat[k].w) continue;   // the same word for every thread
-      __syncthreads();
-      blk_label(sh.label, vals, stride, Tx, Ty, b, k, k / (nbx * nby), k % nbx, k / nbx % nby, status);
-      __syncthreads();
-    }
-  }
   blk_merge(stride, Tx, nblocks, b, status, warp, kTailThreads / 32);
   __syncthreads();
   blk_resolve(nblocks, b, warp, kTailThreads / 32);
@@ -1117,6 +1128,7 @@ size_t block_scratch_bytes(int groups, int Tx, int Ty, int64_t stride) {
   add(sizeof(uint32_t) * nw);                    // sbits
   add(sizeof(unsigned long long) * block_count(groups, Tx, Ty) * kBlkPairs);   // pairs
   add(sizeof(int4) * block_count(groups, Tx, Ty));   // bstat
+  add(sizeof(int) * block_count(groups, Tx, Ty));    // full
   add(sizeof(int) * 4);                          // counters
   add(sizeof(int) * nblk);                       // blkcnt
   add(sizeof(int) * (nblk + 1));                 // blkoff
@@ -1144,6 +1156,7 @@ void block_scratch_carve(void* base, int groups, int Tx, int Ty, int64_t stride,
   b->pairs = reinterpret_cast<unsigned long long*>(
       take(sizeof(unsigned long long) * block_count(groups, Tx, Ty) * kBlkPairs));
   b->bstat = reinterpret_cast<int4*>(take(sizeof(int4) * block_count(groups, Tx, Ty)));
+  b->full = reinterpret_cast<int*>(take(sizeof(int) * block_count(groups, Tx, Ty)));
   b->pcap = block_count(groups, Tx, Ty) * kBlkPairs;
   b->counters = reinterpret_cast<int*>(take(sizeof(int) * 4));
   const int64_t nrows = (int64_t)groups * Ty;
@@ -1173,19 +1186,29 @@ cudaError_t launch_block_select(const float* vals, int groups, int64_t stride, i
   int launches = 2;
   cudaError_t e = launch_pdl(k_blk_mask, dim3((unsigned)((nrows * 32 + kMaskThreads - 1) / kMaskThreads)),
                              dim3(kMaskThreads), 0, st, vals, stride, Tx, Ty, nrows, cs, tau, inv, b);
-  const dim3 grid((Tx + kBlkX - 1) / kBlkX, (Ty + kBlkY - 1) / kBlkY, groups);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_blk_cc, grid, dim3(kBlkFewThreads), 0, st, vals, stride, Tx, Ty, b, status);
+  // runs in the rows that k_blk_mask samples where a block has kDenseRuns
+  const double sampled = (double)((nrows + kMaskThreads / 32 - 1) / (kMaskThreads / 32)) / (double)nrows;
+  const unsigned dense = (unsigned)std::min(
+      4e9, (double)kDenseRuns * sampled * (double)groups * Tx * Ty / (kBlkX * kBlkY) + 1.0);
+  if (nblocks <= 152 * kBlkFullPerSm) {
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_cc_full, dim3((unsigned)nblocks), dim3(kBlkThreads), 0, st, vals, stride,
+                     Tx, Ty, (int)nblocks, (int)kFullAll, dense, b, status);
+  } else {
+    const dim3 grid((Tx + kBlkX - 1) / kBlkX, (Ty + kBlkY - 1) / kBlkY, groups);
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_cc, grid, dim3(kBlkFewThreads), 0, st, vals, stride, Tx, Ty, dense, b, status);
+    if (e == cudaSuccess)
+      e = launch_pdl(k_blk_cc_full, dim3(152 * kBlkFullPerSm), dim3(kBlkThreads), 0, st, vals, stride,
+                     Tx, Ty, (int)nblocks, (int)kFullListed, dense, b, status);
+    launches += 1;
+  }
   if (nblocks <= kTailBlocks && nrows <= kTailRows) {
     if (e == cudaSuccess)
-      e = launch_pdl(k_blk_tail, dim3(1), dim3(kTailThreads), 0, st, vals, stride, Tx, Ty, nblocks,
-                     nrows, b, cap, status, want);
+      e = launch_pdl(k_blk_tail, dim3(1), dim3(kTailThreads), 0, st, stride, Tx, Ty, nblocks, nrows,
+                     b, cap, status, want);
     launches += 1;
   } else {
-    if (e == cudaSuccess)
-      e = launch_pdl(k_blk_cc_full,
-                     dim3((unsigned)std::min<int64_t>((nblocks + kBlkThreads - 1) / kBlkThreads, 152 * 4)),
-                     dim3(kBlkThreads), 0, st, vals, stride, Tx, Ty, nblocks, b, status);
     const unsigned wgrid = (unsigned)std::min<int64_t>((nblocks + 7) / 8, 152 * 64);   // a warp per block
     if (e == cudaSuccess)
       e = launch_pdl(k_blk_merge, dim3(wgrid), dim3(256), 0, st, stride, Tx, nblocks, b, status);
@@ -1196,7 +1219,7 @@ cudaError_t launch_block_select(const float* vals, int groups, int64_t stride, i
       e = launch_pdl(k_pbits_count, dim3((unsigned)ncta), dim3(kPbThreads), 0, st, nrows, b);
     if (e == cudaSuccess)
       e = launch_pdl(k_blk_scan, dim3(2), dim3(1024), 0, st, (int)ncta, nblocks, b, cap, status, want);
-    launches += 6;
+    launches += 5;
   }
   if (e == cudaSuccess && peaks) {
     e = launch_pdl(k_pbits_write, dim3((unsigned)ncta), dim3(kPbThreads), 0, st, nrows, Tx, Ty, vals,

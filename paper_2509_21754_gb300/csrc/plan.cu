@@ -210,7 +210,8 @@ struct fitrig_plan_s {
   float* d_vp = nullptr;
   uint8_t* d_arg = nullptr;      // fused in-tile arg-max (thread-per-tile path)
   double* d_inv = nullptr;       // units + 1 reciprocal scales
-  // [0] gmax key, [1] status flags, [2] ncand, [3] wanted capacity, [4..5] d_invalid
+  // [0] gmax key, [1] status flags, [2] ncand, [3] wanted capacity, [4..5] d_invalid,
+  // [6], [7] the image and frequency branch's BlockScratch::runs
   unsigned* d_small = nullptr;
   unsigned long long* d_invalid = nullptr;   // inside d_small
   double* d_cs = nullptr;        // (units + 1) x (centre, scale)
@@ -585,11 +586,13 @@ static int allocate(fitrig_plan_t p) {
     }
     CK(dmalloc(p, &p->d_blk_f, block_scratch_bytes(1, p->Tx, p->Ty, p->vstride)));
     block_scratch_carve(p->d_blk_f, 1, p->Tx, p->Ty, p->vstride, &p->blk_f);
+    p->blk_f.runs = p->d_small + 7;
     CK(dmalloc(p, &p->d_fpeaks, sizeof(SelItem) * (size_t)std::max<int64_t>(1, p->T)));
   }
   if (p->branch & FITRIG_BRANCH_IMAGE) {
     CK(dmalloc(p, &p->d_blk, block_scratch_bytes(std::max(U, 1), p->Tx, p->Ty, p->vstride)));
     block_scratch_carve(p->d_blk, std::max(U, 1), p->Tx, p->Ty, p->vstride, &p->blk);
+    p->blk.runs = p->d_small + 6;
   }
   if (!p->side_st) {
     CK(cudaStreamCreateWithFlags(&p->side_st, cudaStreamNonBlocking));
@@ -1074,8 +1077,8 @@ static void rec(fitrig_plan_t p, int k, int end, cudaStream_t st) {
 // events (not used inside graphs).
 static cudaError_t enqueue_clear(fitrig_plan_t p, cudaStream_t st) {
   // a serving ring keeps word 0, the running maximum M over every snapshot seen
-  cudaError_t e = p->ring ? cudaMemsetAsync(p->d_small + 1, 0, 20, st)
-                          : cudaMemsetAsync(p->d_small, 0, 24, st);
+  cudaError_t e = p->ring ? cudaMemsetAsync(p->d_small + 1, 0, 28, st)
+                          : cudaMemsetAsync(p->d_small, 0, 32, st);
   if (e == cudaSuccess && p->d_smax)
     e = cudaMemsetAsync(p->d_smax, 0, sizeof(unsigned) * 2 * p->L, st);
   return e;
@@ -1293,7 +1296,7 @@ static int grow_select(fitrig_plan_t p) {
 // Post-processing again after grow_select (status words and invalid counts
 // are cleared; M and the tile statistics are kept).
 static int repost(fitrig_plan_t p, cudaStream_t st, int32_t* ncand) {
-  CK(cudaMemsetAsync(p->d_small + 1, 0, 20, st));
+  CK(cudaMemsetAsync(p->d_small + 1, 0, 28, st));
   CK(enqueue_post(p, st, true));
   CK(cudaStreamSynchronize(st));
   return finish_detect(p, ncand);
