@@ -300,7 +300,8 @@ size_t noise_scratch_bytes(int groups, int nblk);
 void noise_scratch_carve(void* base, int groups, int nblk, NoiseScratch* s);
 // Scratch of the split median/MAD form for `groups` maps of `stride` values
 // that a caller sets aside for it (0 for maps above 2 Mi values), and the same
-// for maps of any size (0 where the form does not exist): a caller that has
+// for maps of any size (0 where the form does not exist, and for the small maps
+// that are resident in one CTA's shared memory instead): a caller that has
 // that much memory idle during the estimate may lend it for larger maps.
 size_t noise_split_bytes(int groups, int64_t stride);
 size_t noise_split_need(int groups, int64_t stride);

@@ -1190,8 +1190,12 @@ static size_t split_head(int groups) {
   return ((size_t)groups * (sizeof(SplitState) + kSplitBins * sizeof(unsigned)) + 255) / 256 * 256;
 }
 
+// Maps that the resident form below takes (192 KB of keys) and that need no scratch.
+constexpr int kSmallMax = 48 * 1024;
+static_assert(kSmallMax % 4 == 0, "whole float4s");
+
 size_t noise_split_need(int groups, int64_t stride) {
-  if (stride > (int64_t)INT32_MAX - kSplitChunk || groups > 65535) return 0;
+  if (stride <= kSmallMax || stride > (int64_t)INT32_MAX - kSplitChunk || groups > 65535) return 0;
   const size_t nc = (size_t)groups * (size_t)split_chunks(stride);
   return split_head(groups) + nc * sizeof(uint4) + nc * kSplitSlot * sizeof(uint32_t) +
          (split_large(stride) ? (size_t)groups * kSplitGather * sizeof(uint32_t) : 0);
@@ -1891,8 +1895,6 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_select(const float* __r
 // their barriers and shared atomics: 1 to 64 maps of 1000 / 7000 / 16,384 /
 // 32,768 values 10 / 12 / 16 / 24 us, against 36 / 51 / 55 / 58 us for one map and
 // 60 to 94 us for 62 in the cluster form of callers without scratch.
-constexpr int kSmallMax = 48 * 1024;   // 192 KB of keys
-static_assert(kSmallMax % 4 == 0, "whole float4s");
 
 __global__ void __launch_bounds__(kSplitThreads) k_medmad_small(const float* __restrict__ vals,
                                                                 int64_t stride, int64_t n,
