@@ -175,48 +175,32 @@ __global__ void __launch_bounds__(kSlideMaxThreads) k_slide(const __grid_constan
 constexpr int kShfRows = 8;     // output rows per CTA
 constexpr int kShfWarps = 4;    // warps (column groups) per CTA
 
-// Sum and maximum over lanes l .. l + W - 1 of a warp (binary decomposition:
-// windows of 1, 2, 4, 8 lanes by doubling, then the blocks of W's bits).
+// Sum and maximum over lanes l .. l + W - 1 of a warp (windows of 2, 4 and 8
+// lanes by doubling, then W = 7 as 4 + 2 + 1 and 9 as 8 + 1).
 // Lanes whose window runs past lane 31 get values that are not used.
 template <int W>
 __device__ __forceinline__ void lane_window(float v, float q, float& s, float& m, float& sq) {
-  float s1 = v, m1 = v, q1 = q;
-  float s2 = s1 + __shfl_down_sync(0xffffffffu, s1, 1);
-  float m2 = fmaxf(m1, __shfl_down_sync(0xffffffffu, m1, 1));
-  float q2 = q1 + __shfl_down_sync(0xffffffffu, q1, 1);
-  float s4 = 0.f, m4 = 0.f, q4 = 0.f, s8 = 0.f, m8 = 0.f, q8 = 0.f;
-  if (W >= 4) {
-    s4 = s2 + __shfl_down_sync(0xffffffffu, s2, 2);
-    m4 = fmaxf(m2, __shfl_down_sync(0xffffffffu, m2, 2));
-    q4 = q2 + __shfl_down_sync(0xffffffffu, q2, 2);
-  }
-  if (W >= 8) {
-    s8 = s4 + __shfl_down_sync(0xffffffffu, s4, 4);
-    m8 = fmaxf(m4, __shfl_down_sync(0xffffffffu, m4, 4));
-    q8 = q4 + __shfl_down_sync(0xffffffffu, q4, 4);
-  }
-  // W = 3: 2 + 1; 5: 4 + 1; 7: 4 + 2 + 1; 9: 8 + 1
-  if (W == 1) {
-    s = s1; m = m1; sq = q1;
-  } else if (W == 3) {
-    s = s2 + __shfl_down_sync(0xffffffffu, s1, 2);
-    m = fmaxf(m2, __shfl_down_sync(0xffffffffu, m1, 2));
-    sq = q2 + __shfl_down_sync(0xffffffffu, q1, 2);
-  } else if (W == 5) {
-    s = s4 + __shfl_down_sync(0xffffffffu, s1, 4);
-    m = fmaxf(m4, __shfl_down_sync(0xffffffffu, m1, 4));
-    sq = q4 + __shfl_down_sync(0xffffffffu, q1, 4);
-  } else if (W == 7) {
+  static_assert(W == 7 || W == 9, "shuffle march windows");
+  const float s2 = v + __shfl_down_sync(0xffffffffu, v, 1);
+  const float m2 = fmaxf(v, __shfl_down_sync(0xffffffffu, v, 1));
+  const float q2 = q + __shfl_down_sync(0xffffffffu, q, 1);
+  const float s4 = s2 + __shfl_down_sync(0xffffffffu, s2, 2);
+  const float m4 = fmaxf(m2, __shfl_down_sync(0xffffffffu, m2, 2));
+  const float q4 = q2 + __shfl_down_sync(0xffffffffu, q2, 2);
+  if (W == 7) {
     s = s4 + __shfl_down_sync(0xffffffffu, s2, 4);
     m = fmaxf(m4, __shfl_down_sync(0xffffffffu, m2, 4));
     sq = q4 + __shfl_down_sync(0xffffffffu, q2, 4);
-    s += __shfl_down_sync(0xffffffffu, s1, 6);
-    m = fmaxf(m, __shfl_down_sync(0xffffffffu, m1, 6));
-    sq += __shfl_down_sync(0xffffffffu, q1, 6);
-  } else {   // W == 9
-    s = s8 + __shfl_down_sync(0xffffffffu, s1, 8);
-    m = fmaxf(m8, __shfl_down_sync(0xffffffffu, m1, 8));
-    sq = q8 + __shfl_down_sync(0xffffffffu, q1, 8);
+    s += __shfl_down_sync(0xffffffffu, v, 6);
+    m = fmaxf(m, __shfl_down_sync(0xffffffffu, v, 6));
+    sq += __shfl_down_sync(0xffffffffu, q, 6);
+  } else {
+    const float s8 = s4 + __shfl_down_sync(0xffffffffu, s4, 4);
+    const float m8 = fmaxf(m4, __shfl_down_sync(0xffffffffu, m4, 4));
+    const float q8 = q4 + __shfl_down_sync(0xffffffffu, q4, 4);
+    s = s8 + __shfl_down_sync(0xffffffffu, v, 8);
+    m = fmaxf(m8, __shfl_down_sync(0xffffffffu, v, 8));
+    sq = q8 + __shfl_down_sync(0xffffffffu, q, 8);
   }
 }
 
