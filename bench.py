@@ -184,7 +184,7 @@ def hbm_peak():
 
 def stack_kernel_hash():
     h = hashlib.sha256()
-    for f in ("k_stack.cu", "internal.cuh"):
+    for f in ("k_stack.cu", "march.cuh", "internal.cuh"):
         with open(os.path.join(ROOT, "paper_2509_21754_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
