@@ -543,7 +543,7 @@ class Plan:
             if stream:
                 fitrig_plan_set(self.h, OPT_STREAM, stream)
         except Exception:
-            fitrig_plan_destroy(self.h)
+            self.close()   # (not again by __del__)
             raise
         self.nsnap = nsnap
 
