@@ -234,7 +234,7 @@ struct fitrig_plan_s {
   void* d_sel = nullptr;
   SelectScratch sel{};
   fitrig_candidate* d_cand = nullptr;
-  fitrig_candidate* d_cand_tmp = nullptr;
+  fitrig_candidate* d_cand_tmp = nullptr;   // follows d_cand, in the same allocation
   int64_t cand_cap = 0;
   float* d_eta = nullptr;        // slot U of d_vp (frequency branch)
   int* d_bin = nullptr;
@@ -298,7 +298,7 @@ static void free_all(fitrig_plan_t p) {
   drop_graph(p);
   void* ptrs[] = {p->d_stack, p->d_vp,  p->d_small, p->d_cs, p->d_arg, p->d_inv,
                   p->d_noise, p->d_split, p->d_blk, p->d_noise_f, p->d_split_f,
-                  p->d_blk_f, p->d_fpeaks, p->d_sel, p->d_cand, p->d_cand_tmp,
+                  p->d_blk_f, p->d_fpeaks, p->d_sel, p->d_cand,
                   p->d_bin,   p->d_tw,  p->d_staging, p->d_push, p->d_report, p->d_accum,
                   p->d_hist,  p->d_hwts, p->d_htw,
                   p->d_smax,  p->d_mrun, p->d_wts, p->d_key, p->d_dstate};   // d_eta lives inside d_vp
@@ -446,7 +446,7 @@ static void drop_graph(fitrig_plan_t p) {
 static int alloc_select(fitrig_plan_t p) {
   ++p->sel_gen;   // the lists move: a captured detect would use the old ones
   drop_graph(p);
-  void* old[] = {p->d_sel, p->d_cand, p->d_cand_tmp};
+  void* old[] = {p->d_sel, p->d_cand};
   for (void* q : old)
     if (q) cudaFree(q);
   p->bytes -= p->sel_bytes;
@@ -491,8 +491,11 @@ static int alloc_select(fitrig_plan_t p) {
   s.bits = reinterpret_cast<uint32_t*>(b + o_bits);
   s.wbase = reinterpret_cast<int*>(b + o_wb);
   p->cand_cap = s.capacity;
-  CK(dmalloc(p, &p->d_cand, sizeof(fitrig_candidate) * cap));
-  CK(dmalloc(p, &p->d_cand_tmp, sizeof(fitrig_candidate) * cap));
+  // the two candidate buffers side by side, at 256-byte boundaries: a serving
+  // field lends both to its pushes
+  const size_t room = (cap + 7) / 8 * 8;
+  CK(dmalloc(p, &p->d_cand, sizeof(fitrig_candidate) * 2 * room));
+  p->d_cand_tmp = p->d_cand + room;
   p->sel_bytes = p->bytes - b0;
   return FITRIG_OK;
 }
@@ -1958,12 +1961,14 @@ constexpr int32_t kServeCandCap = 1 << 16;
 
 // Host rows of a field that do not fill the pitch go linearly (see Ingest) to
 // the field's two candidate buffers, which are idle from the end of one trigger
-// (the candidates are exported by then) to the next, in as many pieces as it
-// takes, and a kernel sets them at their pitch.  All of it is on the field's own
+// (the candidates are exported by then) to the next, in one piece where it fits
+// (half storage up to w = 5) or as many as it takes, and a kernel sets them at
+// their pitch.  All of it is on the field's own
 // stream: it needs no memory beside the field's reservation, and no field waits
 // for another's trigger.  Pieces below kLeastPiece (windows of 16 and more) gain
 // nothing over pitched copies.  Eight fields of 1331 to 4576 pixels a side (4 to
-// 42 MB of BF16): a round 1.35 ms, 1.65 with pitched copies.
+// 42 MB of BF16): a round 1.29 ms; 1.32 with every snapshot in two pieces, 1.65 with
+// pitched copies.
 constexpr size_t kLeastPiece = (size_t)2 << 20;
 
 bool lends_rows(fitrig_plan_t p, size_t dpitch, size_t width) {
@@ -1983,10 +1988,15 @@ bool host_memory(const void* data) {
 
 cudaError_t push_linear(fitrig_plan_t p, char* dst, size_t dpitch, const char* src, size_t width,
                         cudaStream_t st) {
-  void* const buf[2] = {p->d_cand, p->d_cand_tmp};
+  char* const buf[2] = {reinterpret_cast<char*>(p->d_cand), reinterpret_cast<char*>(p->d_cand_tmp)};
+  const size_t area = (size_t)(buf[1] - buf[0]);
   const int64_t ny = p->ny;
-  const int64_t most = (int64_t)(sizeof(fitrig_candidate) * (size_t)p->cand_cap / width);
-  const int64_t pieces = (ny + most - 1) / most, per = (ny + pieces - 1) / pieces;
+  // one copy where both buffers hold the snapshot, else as many rows as one holds
+  int64_t per = ny;
+  if ((size_t)ny * width > 2 * area) {
+    const int64_t most = (int64_t)(area / width), pieces = (ny + most - 1) / most;
+    per = (ny + pieces - 1) / pieces;
+  }
   cudaError_t e = cudaSuccess;
   for (int64_t r0 = 0; r0 < ny; r0 += 2 * per) {   // two copies, then their re-pitching
     for (int k = 0; k < 2 && e == cudaSuccess; ++k) {

@@ -16,8 +16,8 @@ if not torch.cuda.is_available():  # pragma: no cover
 from paper_2509_21754_gb300 import fitrig as F  # noqa: E402
 from paper_2509_21754_gb300 import synth  # noqa: E402
 
-# pieces of a snapshot that the lent buffer takes: two, one (pixels as tiles),
-# four, and none (pitched copies); 16-, 2- and 4-byte rows
+# pieces of a snapshot that the lent buffers take: one, one (pixels as tiles), four,
+# and none (pitched copies)
 FIELDS = [(1499, 1499, 5, F.BF16, torch.bfloat16, True),
           (1100, 1001, 1, F.F32, torch.float32, True),
           (2303, 2001, 8, F.F16, torch.float16, False),
